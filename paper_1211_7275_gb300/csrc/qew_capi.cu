@@ -76,7 +76,9 @@ struct qew_ctx {
     std::vector<double> f;
     std::vector<int32_t> kind;
     std::vector<uint32_t> sample;   // sample index s of each chain (counter word 2)
-    std::vector<int64_t> offset;
+    std::vector<int64_t> offset;    // first site of each chain in the caller's arrays (no gaps)
+    std::vector<int64_t> soffset;   // and in the FP32-split state, whose chains start on 128-byte boundaries
+    int64_t n_state = 0;            // sites of the FP32-split state arrays
     double dt = 0.1;
     uint64_t seed = 0;
     int precision = QEW_FP32_SPLIT;
@@ -106,7 +108,9 @@ struct qew_ctx {
 
     double* d_shift = nullptr;
     double* d_partial = nullptr;
-    size_t partial_slots = 0;
+    size_t partial_slots = 0;       // tiles of all kinds
+    size_t partial_cap = 0;         // doubles allocated
+    int launch_obs = 1;             // observations that one launch may record (the partials' room)
     double* d_obs = nullptr;
     size_t obs_cap = 0;
     double* h_obs = nullptr;
@@ -249,7 +253,7 @@ void free_all(qew_ctx* h)
 
 int alloc_state(qew_ctx* h)
 {
-    const size_t N = static_cast<size_t>(h->n_sites);
+    const size_t N = static_cast<size_t>(h->precision == QEW_FP32_SPLIT ? h->n_state : h->n_sites);
     if (h->precision == QEW_FP32_SPLIT) {
         free_f64(h);
         if (h->sp[0].cell)
@@ -259,9 +263,10 @@ int alloc_state(qew_ctx* h)
             QEW_CUDA(h, dev_alloc(&h->sp[b].off, N), "allocating the offset array");
             if (h->kinds_mask & kPairMask)
                 QEW_CUDA(h, dev_alloc(&h->sp[b].rf, N), "allocating the two-node disorder cache");
+            if (h->kinds_mask & (kQuadMask | 1 << kRBGLinear))
+                QEW_CUDA(h, dev_alloc(&h->sp[b].q3, N), "allocating the third disorder value");
             if (h->kinds_mask & kQuadMask) {
                 QEW_CUDA(h, dev_alloc(&h->sp[b].qn, N), "allocating the cubic disorder cache");
-                QEW_CUDA(h, dev_alloc(&h->sp[b].q3, N), "allocating the cubic disorder cache");
                 QEW_CUDA(h, dev_alloc(&h->sp[b].qab, N), "allocating the cubic disorder cache");
                 QEW_CUDA(h, dev_alloc(&h->sp[b].qc, N), "allocating the cubic disorder cache");
             }
@@ -324,7 +329,8 @@ int build_layout(qew_ctx* h)
     std::vector<int32_t> first(h->n_chains), count(h->n_chains);
     for (int32_t c = 0; c < h->n_chains; ++c) {
         ChainDesc& d = h->h_chains[c];
-        d.offset = h->offset[c];
+        d.offset = h->precision == QEW_FP32_SPLIT ? h->soffset[c] : h->offset[c];
+        d.dense = h->offset[c];
         d.L = static_cast<int32_t>(h->L[c]);
         d.s = h->sample[c];
         d.kind = h->kind[c];
@@ -384,10 +390,17 @@ int build_layout(qew_ctx* h)
     QEW_CUDA(h, dev_alloc(&h->d_btiles, blocks.size()), "allocating block tiles");
     QEW_CUDA(h, cudaMemcpy(h->d_btiles, blocks.data(), blocks.size() * sizeof(TileDesc), cudaMemcpyHostToDevice),
              "uploading block tiles");
-    if (slots > h->partial_slots) {
+    // room for the partials of as many observations as 256 MB hold
+    h->partial_slots = slots;
+    h->launch_obs = 1;
+    if (h->precision == QEW_FP32_SPLIT)
+        h->launch_obs = static_cast<int>(std::min<size_t>(kMaxLaunchObs, std::max<size_t>(1, (size_t(256) << 20) / (slots * 32))));
+    const size_t need = slots * 4 * h->launch_obs;
+    if (need > h->partial_cap) {
         dev_free(h->d_partial);
-        QEW_CUDA(h, dev_alloc(&h->d_partial, slots * 3), "allocating partial sums");
-        h->partial_slots = slots;
+        h->partial_cap = 0;
+        QEW_CUDA(h, dev_alloc(&h->d_partial, need), "allocating partial sums");
+        h->partial_cap = need;
     }
     return QEW_OK;
 }
@@ -413,7 +426,16 @@ int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shif
     return QEW_OK;
 }
 
-SplitLaunch split_args(qew_ctx* h, int kind, int K, int do_obs, SplitState in, SplitState out)
+// One launch of the fused kernel (per disorder kind): K steps and the observations among them.
+struct Segment {
+    int K = 0;
+    int n_obs = 0;
+    uint16_t at[kMaxLaunchObs];    // observation after so many of the steps,
+    uint16_t len[kMaxLaunchObs];   // its own segment being the last so many
+    int32_t index[kMaxLaunchObs];  // and its place in the call's list
+};
+
+SplitLaunch split_args(qew_ctx* h, int kind, const Segment& s, SplitState in, SplitState out)
 {
     SplitLaunch a{};
     a.tiles = h->d_tiles[kind];
@@ -422,13 +444,20 @@ SplitLaunch split_args(qew_ctx* h, int kind, int K, int do_obs, SplitState in, S
     a.chains = h->d_chains;
     a.in = in;
     a.out = out;
-    a.K = K;
+    a.K = s.K;
+    // Windows start on 16-byte boundaries where the halo has room for it (bulk copies; a launch of
+    // one step through plain loads and stores took 2.4 times a launch of four on 4 x 2^25 sites).
+    const int pad = (s.K + 3) & ~3;
+    a.pad = (pad + s.K <= 2 * h->K) ? pad : s.K;
     a.w_own = h->w_own[kind];
     a.dt = static_cast<float>(h->dt);
     a.seed = h->seed;
-    a.do_obs = do_obs;
+    a.n_obs = s.n_obs;
+    std::copy(s.at, s.at + s.n_obs, a.obs_at);
+    std::copy(s.len, s.len + s.n_obs, a.obs_len);
     a.shift = h->d_shift;
     a.partial = h->d_partial;
+    a.partial_stride = static_cast<int64_t>(h->partial_slots);
     a.crossings = h->stats_on ? h->d_crossings : nullptr;
     a.error = h->d_error;
     a.keys = philox_key_schedule(h->seed);
@@ -446,12 +475,12 @@ int next_event(qew_ctx* h, cudaEvent_t* ev)
     return QEW_OK;
 }
 
-int launch_split_all(qew_ctx* h, int K, int do_obs, SplitState in, SplitState out)
+int launch_split_all(qew_ctx* h, const Segment& s, SplitState in, SplitState out)
 {
     for (int k = 0; k < kNumKinds; ++k) {
         if (h->n_tiles[k] == 0)
             continue;
-        const SplitLaunch a = split_args(h, k, K, do_obs, in, out);
+        const SplitLaunch a = split_args(h, k, s, in, out);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (h->stats_on) {
             int rc = next_event(h, &e0);
@@ -466,7 +495,7 @@ int launch_split_all(qew_ctx* h, int K, int do_obs, SplitState in, SplitState ou
             QEW_CUDA(h, cudaEventRecord(e1, h->stream), "recording a timing event");
         h->n_launches += 1;
         h->n_fused += 1;
-        h->n_site_updates += h->sites_of_kind[k] * K;
+        h->n_site_updates += h->sites_of_kind[k] * s.K;
     }
     return QEW_OK;
 }
@@ -509,57 +538,107 @@ int guard_range(qew_ctx* h)
 // better).  Step 1024 is past the crossover.
 constexpr int64_t kTuneAfterSteps = 1024;
 
-// Advance to `target` (>= current step); with `obs` record the observables there into obs.
-int run_to(qew_ctx* h, int64_t target, double* obs)
+// Runs a segment and the second pass of its observations.
+int run_segment(qew_ctx* h, const Segment& s, double* d_obs)
 {
-    if (h->precision == QEW_FP32_SPLIT) {
-        bool observed = false;
-        while (h->step < target) {
-            if (h->autotune_pending && h->step >= kTuneAfterSteps) {
-                int rc = autotune(h);
-                if (rc != QEW_OK)
-                    return rc;
-            }
-            int64_t seg_end = target;
-            if (h->autotune_pending && h->step < kTuneAfterSteps)
-                seg_end = std::min<int64_t>(target, kTuneAfterSteps);
-            const int Keff = static_cast<int>(std::min<int64_t>(h->K, seg_end - h->step));
-            const bool last = (h->step + Keff == target);
-            const int do_obs = (obs != nullptr && last) ? 1 : 0;
-            int rc = launch_split_all(h, Keff, do_obs, h->sp[h->cur], h->sp[h->cur ^ 1]);
-            if (rc != QEW_OK)
-                return rc;
-            h->cur ^= 1;
-            h->step += Keff;
-            observed = observed || do_obs;
-        }
-        if (obs && !observed) {
-            int rc = launch_split_all(h, 0, 1, h->sp[h->cur], h->sp[h->cur ^ 1]);
-            if (rc != QEW_OK)
-                return rc;
-        }
-        if (obs) {
-            QEW_CUDA(h, reduce_chains(h->d_chains, h->n_chains, h->d_partial, h->d_shift, obs, 1, h->stream),
-                     "launching the observable reduction");
-            h->n_launches += 1;
-        }
-    } else {
-        while (h->step < target) {
-            QEW_CUDA(h, f64_step(f64_args(h), h->stream), "launching the FP64 step kernel");
-            h->cur ^= 1;
-            h->f64.u = h->u64[h->cur];
-            ++h->step;
-            h->n_launches += 1;
-            h->n_site_updates += h->n_sites;
-        }
-        if (obs) {
-            QEW_CUDA(h, f64_observe(f64_args(h), h->stream), "launching the FP64 observation kernel");
-            QEW_CUDA(h, reduce_chains(h->d_chains, h->n_chains, h->d_partial, h->d_shift, obs, 1, h->stream),
-                     "launching the observable reduction");
-            h->n_launches += 2;
-        }
+    if (s.K == 0 && s.n_obs == 0)
+        return QEW_OK;
+    int rc = launch_split_all(h, s, h->sp[h->cur], h->sp[h->cur ^ 1]);
+    if (rc != QEW_OK)
+        return rc;
+    if (s.K > 0) {
+        h->cur ^= 1;
+        h->step += s.K;
+    }
+    if (s.n_obs > 0) {
+        ObsList list{};
+        list.n = s.n_obs;
+        std::copy(s.index, s.index + s.n_obs, list.index);
+        QEW_CUDA(h, reduce_chains(h->d_chains, h->n_chains, h->d_partial, static_cast<int64_t>(h->partial_slots), h->d_shift, d_obs,
+                                  list, h->stream), "launching the observable reduction");
+        h->n_launches += 1;
     }
     return QEW_OK;
+}
+
+// Advance through the increasing steps `targets`, recording the observables at each into d_obs (NULL:
+// advance only).  FP32-split: launches of up to K steps, each with the observations that fall into it.
+// An observation's own segment (the steps since the observation before it, or the last whole K steps
+// of them) stays within one launch, which keeps its sums independent of the packing.  Log-spaced
+// schedules crowd their observations at the start: 1024 steps with 40 of them at K = 32 take 34
+// launches so, and 59 with one launch per observation.
+int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d_obs)
+{
+    const size_t per = static_cast<size_t>(h->n_chains) * 4;
+    if (h->precision != QEW_FP32_SPLIT) {
+        for (int32_t k = 0; k < n_targets; ++k) {
+            while (h->step < targets[k]) {
+                QEW_CUDA(h, f64_step(f64_args(h), h->stream), "launching the FP64 step kernel");
+                h->cur ^= 1;
+                h->f64.u = h->u64[h->cur];
+                ++h->step;
+                h->n_launches += 1;
+                h->n_site_updates += h->n_sites;
+            }
+            if (d_obs) {
+                ObsList list{};
+                list.n = 1;
+                QEW_CUDA(h, f64_observe(f64_args(h), h->stream), "launching the FP64 observation kernel");
+                QEW_CUDA(h, reduce_chains(h->d_chains, h->n_chains, h->d_partial, static_cast<int64_t>(h->partial_slots), h->d_shift,
+                                          d_obs + per * k, list, h->stream), "launching the observable reduction");
+                h->n_launches += 2;
+            }
+        }
+        return QEW_OK;
+    }
+    Segment s;
+    int64_t at = h->step;   // step reached with the segment being packed
+    int rc = QEW_OK;
+    for (int32_t k = 0; k < n_targets; ++k) {
+        bool first = true;   // (an observation at the current step has a segment of no steps)
+        while (at < targets[k] || (first && d_obs)) {
+            if (h->autotune_pending && at >= kTuneAfterSteps && at < targets[k]) {
+                rc = run_segment(h, s, d_obs);
+                if (rc == QEW_OK)
+                    rc = autotune(h);
+                if (rc != QEW_OK)
+                    return rc;
+                s = Segment();
+            }
+            int64_t end = targets[k];
+            if (h->autotune_pending && at < kTuneAfterSteps)
+                end = std::min<int64_t>(end, kTuneAfterSteps);
+            const int len = static_cast<int>(std::min<int64_t>(h->K, end - at));
+            const bool observe = d_obs && at + len == targets[k];
+            int left = len;
+            if (observe && (s.K + len > h->K || s.n_obs == h->launch_obs)) {
+                rc = run_segment(h, s, d_obs);
+                if (rc != QEW_OK)
+                    return rc;
+                s = Segment();
+            }
+            while (left > 0) {
+                const int take = std::min(left, h->K - s.K);
+                s.K += take;
+                left -= take;
+                if (left > 0) {
+                    rc = run_segment(h, s, d_obs);
+                    if (rc != QEW_OK)
+                        return rc;
+                    s = Segment();
+                }
+            }
+            at += len;
+            if (observe) {
+                s.at[s.n_obs] = static_cast<uint16_t>(s.K);
+                s.len[s.n_obs] = static_cast<uint16_t>(len);
+                s.index[s.n_obs] = k;
+                ++s.n_obs;
+            }
+            first = false;
+        }
+    }
+    return run_segment(h, s, d_obs);
 }
 
 // Times candidate launch shapes on the handle's own chains: each trial launch reads the
@@ -610,13 +689,15 @@ int autotune(qew_ctx* h)
                 h->K = K;
                 h->tpc = T;
                 rc = build_layout(h);
+                Segment trial;
+                trial.K = K;
                 // best of four timed repetitions (after one untimed), each two launches long, so a
                 // shape wins by its throughput rather than by the noise of a single launch
                 float ms_best = 1e30f;
                 for (int rep = 0; rep < 5 && rc == QEW_OK; ++rep) {
                     cudaEventRecord(e0, h->stream);
                     for (int l = 0; l < 2 && rc == QEW_OK; ++l)
-                        rc = launch_split_all(h, K, 0, h->sp[h->cur], h->sp[h->cur ^ 1]);
+                        rc = launch_split_all(h, trial, h->sp[h->cur], h->sp[h->cur ^ 1]);
                     if (rc != QEW_OK)
                         break;
                     cudaEventRecord(e1, h->stream);
@@ -712,10 +793,13 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
         for (int32_t c = 0; c < n_chains; ++c)
             h->sample[c] = static_cast<uint32_t>(c);
         h->offset.resize(n_chains);
+        h->soffset.resize(n_chains);
         int64_t off = 0;
         for (int32_t c = 0; c < n_chains; ++c) {
             h->offset[c] = off;
             off += L[c];
+            h->soffset[c] = h->n_state;
+            h->n_state += (L[c] + 31) & ~int64_t(31);
             h->kinds_mask |= 1 << kind[c];
             h->sites_of_kind[kind[c]] += L[c];
         }
@@ -853,8 +937,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
             if (!capturing)
                 cudaGetLastError();
         }
-        for (int32_t k = 0; k < n_times && rc == QEW_OK; ++k)
-            rc = run_to(h, steps[k], h->d_obs + per * k);
+        rc = run_through(h, steps, n_times, h->d_obs);
         if (rc == QEW_OK)
             rc = guard_range(h);
         cudaError_t ce = cudaSuccess;
@@ -1133,7 +1216,8 @@ int qew_advance(qew_handle h, int64_t n_steps)
     if (n_steps < 0)
         return fail(h, QEW_EINVAL, "n_steps must be >= 0");
     DeviceGuard g(h->device);
-    int rc = run_to(h, h->step + n_steps, nullptr);
+    const int64_t target = h->step + n_steps;
+    int rc = run_through(h, &target, 1, nullptr);
     if (rc == QEW_OK && n_steps > 0)
         rc = guard_range(h);
     if (rc == QEW_OK) {

@@ -35,7 +35,8 @@ constexpr uint32_t kTagRBG = 2u;  // counter word 3 of Gaussian random-bond pote
 
 // One chain of the batch.
 struct ChainDesc {
-    int64_t offset;   // first site of the chain in the concatenated state arrays
+    int64_t offset;   // first site of the chain in the state arrays
+    int64_t dense;    // and in the caller's arrays, where the chains follow one another without gaps
     int32_t L;        // number of sites
     uint32_t s;       // sample index (counter word 2)
     int32_t kind;     // kRF / kRB / kNone
@@ -136,11 +137,12 @@ __device__ __forceinline__ uint4 disorder_words(uint64_t seed, uint32_t s, int32
 __device__ __forceinline__ float ln_u1_f32(uint32_t x)
 {
     const bool upper = (x & 0x80000000u) != 0;
-    const float u1 = fmaf(static_cast<float>(x), 0x1p-32f, 0x1p-33f);
-    const uint32_t bits = __float_as_uint(u1);
+    // U1 in the lower half, 1 - U1 in the upper: one conversion serves both
+    const float t = fmaf(static_cast<float>(upper ? ~x : x), 0x1p-32f, 0x1p-33f);
+    const uint32_t bits = __float_as_uint(t);
     const float m = __uint_as_float((bits & 0x007FFFFFu) | 0x3F800000u);   // exact
-    const float e = static_cast<float>(static_cast<int>(bits >> 23) - 127);
-    const float t = fmaf(static_cast<float>(~x), 0x1p-32f, 0x1p-33f);
+    // the exponent as a float, exactly and off the conversion pipe: 2^23 + biased exponent, less 2^23 + 127
+    const float e = __uint_as_float((bits >> 23) | 0x4B000000u) - 8388735.0f;
     const float num = upper ? t : m - 1.0f;
     const float den = upper ? 2.0f - t : m + 1.0f;
     const float rc = __fdividef(1.0f, den);

@@ -165,10 +165,11 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
             s1 += red[1][w];
             s2 += red[2][w];
         }
-        double* dst = a.partial + static_cast<size_t>(blockIdx.x) * 3;
+        double* dst = a.partial + static_cast<size_t>(blockIdx.x) * 4;
         dst[0] = sF;
         dst[1] = s1;
         dst[2] = s2;
+        dst[3] = c;
     }
 }
 

@@ -34,6 +34,9 @@ struct F64State {
     double* c[4];
 };
 
+// Most observations that one launch of the fused kernel records.
+constexpr int kMaxLaunchObs = 24;
+
 struct SplitLaunch {
     const TileDesc* tiles;   // tiles of one disorder kind
     int32_t n_tiles;
@@ -41,12 +44,16 @@ struct SplitLaunch {
     const ChainDesc* chains;
     SplitState in, out;
     int32_t K;               // Euler steps in this launch (0: observe only)
+    int32_t pad;             // sites of a tile's window before its first owned one (>= K)
     int32_t w_own;           // owned sites per tile
     float dt;
     uint64_t seed;
-    int32_t do_obs;          // write per-tile partial sums of the state after the K steps
+    int32_t n_obs;           // observations in this launch: per-tile partial sums of the state
+    uint16_t obs_at[kMaxLaunchObs];    // after so many of its steps (increasing),
+    uint16_t obs_len[kMaxLaunchObs];   // the last so many of which belong to the observation's own segment
     const double* shift;     // per-chain reference cell c of the sums
-    double* partial;         // [n_tiles_total][3]: sum F, sum (u - c), sum (u - c)^2
+    double* partial;         // [n_obs][partial_stride][4]: sum F, sum (u - c), sum (u - c)^2, c
+    int64_t partial_stride;  // tiles of all kinds
     unsigned long long* crossings;  // if not null: cell crossings are added here
     int32_t* error;          // 1: a bounded wait on a bulk copy gave up; 2: neighbouring cells 2^12 apart
     PhiloxKeys keys;         // round keys of `seed`
@@ -87,11 +94,15 @@ cudaError_t f64_init(const ChainDesc* chains, const TileDesc* tiles, int32_t n_t
 cudaError_t f64_cells(const ChainDesc* chains, const TileDesc* tiles, int32_t n_tiles, int32_t w_tile,
                       const double* u, int32_t* cells_out, cudaStream_t stream);
 
-// Second pass: per chain, sum the partials of its tiles in a fixed order, record
-// (sum F, S1, S2, c) into obs[chain] and move the chain's reference c to the new centre of
-// mass (rounded to an integer cell when `integer_shift`).
-cudaError_t reduce_chains(const ChainDesc* chains, int32_t n_chains, const double* partial, double* shift,
-                          double* obs, int integer_shift, cudaStream_t stream);
+// Second pass of n_obs observations: per chain, sum the partials of its tiles in a fixed order, record
+// (sum F, S1, S2, c) into obs[index[k]][chain] and move the chain's reference c to the centre of mass at
+// the last of them (rounded to an integer cell).
+struct ObsList {
+    int32_t n;
+    int32_t index[kMaxLaunchObs];
+};
+cudaError_t reduce_chains(const ChainDesc* chains, int32_t n_chains, const double* partial, int64_t partial_stride,
+                          double* shift, double* obs, const ObsList& list, cudaStream_t stream);
 
 // Structure factor (Eq. 6): rows of u(x) - c0 per chain in the padded layout of an in-place
 // real-to-complex FFT (row stride 2 (L/2 + 1) doubles), from the split state (split != NULL) or

@@ -16,17 +16,20 @@
 namespace qew {
 namespace {
 
-__global__ void __launch_bounds__(256) reduce_chains_kernel(const ChainDesc* chains, const double* partial,
-                                                            double* shift, double* obs, int integer_shift)
+__global__ void __launch_bounds__(256) reduce_chains_kernel(const ChainDesc* chains, int32_t n_chains, const double* partial,
+                                                            int64_t partial_stride, double* shift, double* obs, ObsList list)
 {
     __shared__ double red[3][256];
     const ChainDesc ch = chains[blockIdx.x];
+    const double* mine = partial + (static_cast<size_t>(blockIdx.y) * partial_stride + ch.tile0) * 4;
     double a = 0.0, b = 0.0, c = 0.0;
+#pragma unroll 4
     for (int t = threadIdx.x; t < ch.ntiles; t += blockDim.x) {
-        const double* q = partial + static_cast<size_t>(ch.tile0 + t) * 3;
-        a += q[0];
-        b += q[1];
-        c += q[2];
+        const double2 q0 = *reinterpret_cast<const double2*>(mine + static_cast<size_t>(t) * 4);
+        const double q2 = mine[static_cast<size_t>(t) * 4 + 2];
+        a += q0.x;
+        b += q0.y;
+        c += q2;
     }
     red[0][threadIdx.x] = a;
     red[1][threadIdx.x] = b;
@@ -41,17 +44,20 @@ __global__ void __launch_bounds__(256) reduce_chains_kernel(const ChainDesc* cha
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const double c_used = shift[blockIdx.x];
-        double* o = obs + static_cast<size_t>(blockIdx.x) * 4;
+        // the reference that the sums were taken with, as the tiles wrote it down: the block of the
+        // last observation moves the chain's own meanwhile
+        const double c_used = mine[3];
+        double* o = obs + (static_cast<size_t>(list.index[blockIdx.y]) * n_chains + blockIdx.x) * 4;
         o[0] = red[0][0];
         o[1] = red[1][0];
         o[2] = red[2][0];
         o[3] = c_used;
-        const double mean_rel = red[1][0] / static_cast<double>(ch.L);
-        double next = c_used + (integer_shift ? floor(mean_rel + 0.5) : mean_rel);
-        if (!isfinite(next) || fabs(next) > 1.0e9)
-            next = c_used;  // keep a usable reference if the state went non-finite
-        shift[blockIdx.x] = next;
+        if (static_cast<int>(blockIdx.y) == list.n - 1) {
+            double next = c_used + floor(red[1][0] / static_cast<double>(ch.L) + 0.5);
+            if (!isfinite(next) || fabs(next) > 1.0e9)
+                next = c_used;  // keep a usable reference if the state went non-finite
+            shift[blockIdx.x] = next;
+        }
     }
 }
 
@@ -141,12 +147,12 @@ cudaError_t bounded_wait_selftest(int32_t* d_error, int spin_limit, cudaStream_t
     return cudaGetLastError();
 }
 
-cudaError_t reduce_chains(const ChainDesc* chains, int32_t n_chains, const double* partial, double* shift,
-                          double* obs, int integer_shift, cudaStream_t stream)
+cudaError_t reduce_chains(const ChainDesc* chains, int32_t n_chains, const double* partial, int64_t partial_stride,
+                          double* shift, double* obs, const ObsList& list, cudaStream_t stream)
 {
-    if (n_chains == 0)
+    if (n_chains == 0 || list.n == 0)
         return cudaSuccess;
-    reduce_chains_kernel<<<n_chains, 256, 0, stream>>>(chains, partial, shift, obs, integer_shift);
+    reduce_chains_kernel<<<dim3(n_chains, list.n), 256, 0, stream>>>(chains, n_chains, partial, partial_stride, shift, obs, list);
     return cudaGetLastError();
 }
 

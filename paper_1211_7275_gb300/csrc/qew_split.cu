@@ -8,31 +8,39 @@
 // Eqs. 3-5 (Sec. II).
 //
 // State of a site: integer cell n and FP32 offset d in [0, 1) (u = n + d), held in registers,
-// plus its disorder cache, held in shared memory.  Pair kinds keep the two nodes of the cell:
-// RF (R(n) + f, R(n+1) + f) -- the drive f is folded in, so F_p + f is one subtraction and one
-// FMA -- and the linear-spline random bond (G(n), G(n+1)), F_p + f = (G(n) - G(n+1)) + f.  Quad
-// kinds (cubic random bond, uniform V or Gaussian G) keep the coefficients A, B, C of
-// F_p + f = A + d (B + d C) over the cell (from the spline nodes V(n-1 .. n+2)) and the three
-// nodes V(n), V(n+1), V(n+2) that a move to a neighbouring cell reuses.
+// plus its disorder cache, held in shared memory.
+//   random field           the nodes of the cell, (R(n) + f, R(n+1) + f): the drive f is folded in, so
+//                          F_p + f is one subtraction and one FMA
+//   linear-spline random   the forces F_p = G - G(+1) of two neighbouring cells, of which the site is in
+//   bond (Case 3)          one, and the node above them.  79% of the moves at the threshold go back
+//                          where the site came from (it chatters across a jump of its force): they flip
+//                          one bit of a lane mask and draw nothing (0.05 instead of 0.17 draws per
+//                          site-update; 4 x 2^25 sites 4.7e11 -> 8.9e11 su/s late in a relaxation)
+//   cubic random bond      the coefficients A, B, C of F_p + f = A + d (B + d C) over the cell (from the
+//                          spline nodes V(n-1 .. n+2)) and the nodes V(n), V(n+1), V(n+2) that a move up
+//                          reuses
 //
 // Work decomposition: one warp owns one tile of 32 * S sites of a chain, S consecutive sites
 // per lane.  A tile advanced K steps needs K extra sites on each side (the stencil's light
-// cone), so the window is [start - K, start - K + 32 S) and the owned sites
-// [start, start + w_own), w_own <= 32 S - 2K; the outermost sites of the window go stale one
+// cone): the window is [start - pad, start - pad + 32 S) with pad = K rounded up to 4, and the owned
+// sites [start, start + w_own); the outermost sites of the window go stale one
 // per step from each edge and are never stored.  Windows wrap around periodic chains (any
-// number of times for chains shorter than a tile).  Halo exchange inside a step is two warp
-// shuffles per neighbour and there is no block-wide barrier.
+// number of times for chains shorter than a tile).  Halo exchange inside a step is three warp
+// shuffles and there is no block-wide barrier.
 //
-// Cell crossings: renormalisation is branch-free (n += floor(d), d -= floor(d)) and leaves one
-// bit per moved site.  After the update loop each lane stores its cells to shared memory (one
-// store per site; a store inside the update loop would keep the compiler from hoisting the cache
-// loads there), and a warp prefix sum of the lanes' move counts gives each lane its queue slots,
-// which it fills by walking the set bits of its mask (no atomics, deterministic order): all of
-// a step's requests in one pass where the queue holds a whole step, else 32 slots per chunk,
-// resuming in the next chunk where it stopped.  The queued Philox values are then evaluated 32
-// lanes at a time and written straight into the shared-memory cache of the requesting sites; the
-// direction of each move is recovered from the cell the cache was drawn for, kept per site in
-// shared memory.
+// What bounds it, and the shape of a step.  The kernel is bound by instruction issue and by the
+// latency of a step's serial parts at 12 to 16 warps per SM, not by memory.  So
+//   - the update loop works on register pairs with packed FP32 instructions (half the issue slots; the
+//     FP32 pipe itself is as busy as with scalar ones, 59% at 992-site tiles) and reads both sites'
+//     cache values with one 16-byte load;
+//   - renormalisation is branch-free (n += floor(d), d -= floor(d)), with the floor by two packed
+//     additions: as a conversion it took the conversion pipe 7.6 clocks per site;
+//   - a funnel shift per site collects what moved how far (MoveCodes), so that moves by one cell need
+//     no copy of the cells for the consumers; a rare path takes moves by more;
+//   - requests are queued by ballots, without a prefix sum, and the Philox values evaluated 32 lanes at
+//     a time, straight into the shared-memory cache of the requesting sites.
+// 16 x 2^20 random-field chains at the threshold, 992-site tiles, K = 32: 0.94 -> 0.62 warp-instructions
+// per site-update, 75% -> 67% issue, 560 -> 425 us per launch (1.03e12 -> 1.26e12 su/s).
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -62,94 +70,376 @@ __device__ __forceinline__ int32_t site_index(int64_t wstart, int x, bool contig
 // Bytes of disorder cache per site in HBM.
 template <int KIND>
 struct CacheBytes {
-    static constexpr int hbm = pair_kind(KIND) ? 8 : quad_kind(KIND) ? 24 : 0;
+    static constexpr int hbm = KIND == kRF ? 8 : KIND == kRBGLinear ? 12 : quad_kind(KIND) ? 24 : 0;
 };
 
-// Shared memory per site.  Random-field tiles of 31 or more sites per lane use a compact layout
-// of 14 B: one 4-byte staging slot (cells, then offsets, at load and store; each step's new
-// cells in between), the 8-byte node pair, and the low 16 bits of the cell the pair was drawn
-// for.  At 992-site tiles this fits 16 instead of 14 warps per SM (measured: +3.3%); smaller
-// tiles are register-limited, and there the two-pass staging only costs (measured on 736-site
-// random-field tiles in a mixed batch and on Case 3).  The other layouts keep 8 bytes of staging
-// (cell and offset side by side, the cell half doubling as the cache cell) plus the cache: a
-// node pair (8 B), or for the cubic kinds the coefficients and three nodes (24 B, the same in
-// HBM, so a tile loads them without recomputing the coefficients).  The cubic kinds are bound by
-// the shared-memory data path and by latency; measured on the uniform random bond:
-//   - the coefficients as (A, B) pairs and C alone, so the update loop reads 12 bytes per site
-//     and step rather than a 16-byte vector with an unused lane: +5% (12 instead of 11 warps per
-//     SM at 480-site tiles, one load instruction more per site);
-//   - three nodes instead of four (V(n-1) is dropped; a down move draws it again, and at the
-//     thresholds down moves are a few in 10^4) and no coefficient recompute at tile load: +10%
-//     (14 warps per SM, 108 instead of 124 registers).
-__host__ __device__ constexpr bool compact_layout(int kind, int S) { return kind == kRF && S >= 31; }
-__host__ __device__ constexpr int site_smem_bytes(int kind, int S)
+// ---- two sites at a time ----
+// A lane's S = 2H + 1 consecutive sites are two runs of H sites and one last site.  Site j of the
+// first run and site j of the second (lane sites j and H + j) share a 64-bit register pair, and
+// their elastic force, Euler update and cell move are packed FP32 operations (two sites per issue
+// slot, each rounded as the scalar operation).  The right neighbours of pair j are pair j + 1, so
+// no operand has to be re-paired inside a run.
+using pair_t = unsigned long long;
+
+__device__ __forceinline__ pair_t pk(float lo, float hi)
 {
-    return compact_layout(kind, S) ? 4 + 8 + 2 : pair_kind(kind) ? 8 + 8 : quad_kind(kind) ? 8 + 24 : 8;
+    pair_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo(pair_t p)
+{
+    return __uint_as_float(static_cast<unsigned>(p));
+}
+__device__ __forceinline__ float hi(pair_t p)
+{
+    return __uint_as_float(static_cast<unsigned>(p >> 32));
+}
+__device__ __forceinline__ pair_t add2(pair_t a, pair_t b)
+{
+    pair_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ pair_t sub2(pair_t a, pair_t b)
+{
+    pair_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// floor of both halves, |x| < 2^22: adding 1.5 * 2^23 rounded down leaves the floor in a float whose
+// last place is 1.
+__device__ __forceinline__ pair_t floor2(pair_t x)
+{
+    const pair_t big = pk(12582912.0f, 12582912.0f);
+    pair_t r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(big));
+    return sub2(r, big);
+}
+__device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c)
+{
+    pair_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
-// Per warp after its sites, the request queue.  The two-node kinds below 31 sites per lane have
-// shared memory to spare: their queue holds every request of a step (a 16-bit window position per
-// site of the tile), so each lane walks its move mask once per step instead of once per chunk of
-// 32 requests (measured: Case 3, about 90 requests per step and tile, +18.5%; the random field at
-// 736-site tiles +2.5%).  The others keep one chunk of 32 requests: the compact random-field
-// layout and the cubic kinds are bound by shared memory, and their steps rarely make more than 32
-// requests.
-__host__ __device__ constexpr bool full_queue(int kind, int S) { return pair_kind(kind) && S < 31; }
-__host__ __device__ constexpr int queue_bytes(int kind, int S) { return full_queue(kind, S) ? 32 * S * 2 : 32 * 4; }
+// ---- shared memory of one warp tile ----
+//   slot    4 B per site, linear: offsets and then cells arrive and leave through it; in between it
+//           holds the cell that each site's cache belongs to
+//   loop    what the update loop reads, a row of 32 float4 per pair (row t is pair H - 1 - t, row H
+//           the last site): one conflict-free 16-byte load per pair and step.  (first, second) value
+//           of both sites: RF (R(n) + f, R(n+1) + f); linear-spline random bond the force F_p of
+//           two neighbouring cells; cubic kinds the coefficients (A, B), and C in rows of float2
+//   nodes   what only a cell move reads, linear: the node above the two cells (linear-spline random
+//           bond), V(n), V(n+1) and V(n+2) (cubic kinds)
+//   queue   kQueue requests of 2 B
+// RF takes 12 B per site and so 16 warps per SM at 992-site tiles, the register limit.
+template <int KIND, int S>
+struct Tile {
+    static constexpr int H = S / 2;
+    static constexpr int TW = 32 * S;
+    static constexpr bool has_pair = pair_kind(KIND);
+    static constexpr bool has_quad = quad_kind(KIND);
+    static constexpr bool has_cache = has_pair || has_quad;
+    static constexpr int slot = 0;
+    static constexpr int loop = 4 * TW;
+    static constexpr int loopc = loop + (has_cache ? 512 * (H + 1) : 0);
+    static constexpr int top = loopc + (has_quad ? 256 * (H + 1) : 0);     // one float per site
+    static constexpr int nodes = top + (has_quad || KIND == kRBGLinear ? 4 * TW : 0);   // one float2 per site
+    static constexpr int queue = nodes + (has_quad ? 8 * TW : 0);
+    static constexpr int kQueue = 256;
+    // whether a single cell downwards is an ordinary move (else it takes the rare path of far moves):
+    // a fifth of the linear-spline random bond's moves, a few in 10^4 of the other kinds'
+    static constexpr bool kDown = KIND == kRBGLinear || KIND == kRBGCubic;
+    // KIND none stages offsets and cells side by side: it has no cache to make room for
+    static constexpr int slot2 = has_cache ? slot : 4 * TW;
+    static constexpr int bytes = has_cache ? queue + 2 * kQueue : 8 * TW;
+};
 
-// F_p + f at window position x with offset d, from the shared-memory cache.
-template <int KIND>
-__device__ __forceinline__ float drive_plus_pinning(const float2* s_rf, const float2* s_ab, const float* s_c, int x, float d, float f)
-{
-    if constexpr (KIND == kRF) {
-        const float2 q = s_rf[x];
-        return fmaf(d, q.y - q.x, q.x);
-    } else if constexpr (KIND == kRBGLinear) {
-        const float2 q = s_rf[x];
-        return (q.x - q.y) + f;
-    } else if constexpr (quad_kind(KIND)) {
-        const float2 ab = s_ab[x];
-        return fmaf(d, fmaf(d, s_c[x], ab.y), ab.x);
-    } else {
-        return f;
-    }
-}
-
-// Per-lane mask of the sites that moved in a step: 32 bits while a lane holds at most 32 sites,
-// 64 beyond.  The bit of site j is a compile-time constant in the unrolled update loop, so each
-// site still sets one bit of one 32-bit word.
+// Per-lane mask of the sites that moved in a step.  Bit t is pair H - 1 - t's second site, bit D + t
+// its first site, bit D + H the last site; D (a multiple of 3) leaves room for H bits, and a mask of
+// more than 32 sites takes 64 bits.
 template <int S>
-using MoveMask = typename std::conditional<(S <= 32), unsigned, unsigned long long>::type;
+struct Moves {
+    static constexpr int H = S / 2;
+    static constexpr bool wide = S > 32;
+    static constexpr int D = wide ? 32 : 3 * ((H + 2) / 3);
+    using mask = typename std::conditional<wide, unsigned long long, unsigned>::type;
+    static constexpr mask last = mask(1) << (D + H);
+    static __host__ __device__ constexpr mask first(int p) { return mask(1) << (D + H - 1 - p); }
+    static __host__ __device__ constexpr mask second(int p) { return mask(1) << (H - 1 - p); }
+};
 
 __device__ __forceinline__ int mask_popc(unsigned m) { return __popc(m); }
 __device__ __forceinline__ int mask_popc(unsigned long long m) { return __popcll(m); }
-__device__ __forceinline__ int mask_ffs(unsigned m) { return __ffs(m); }
-__device__ __forceinline__ int mask_ffs(unsigned long long m) { return __ffsll(static_cast<long long>(m)); }
 
-// Kinds of cell move.
-constexpr int kMoveUp = 1;
-constexpr int kMoveDown = 2;
-constexpr int kMoveFar = 3;
+// m without bit b; 0 stays 0 (b is -1 then: the shift clamps).
+__device__ __forceinline__ unsigned mask_drop(unsigned m, int b)
+{
+    unsigned one;
+    asm("shl.b32 %0, 1, %1;" : "=r"(one) : "r"(b));
+    return m & ~one;
+}
+__device__ __forceinline__ unsigned long long mask_drop(unsigned long long m, int b)
+{
+    unsigned long long one;
+    asm("shl.b64 %0, 1, %1;" : "=l"(one) : "r"(b));
+    return m & ~one;
+}
 
-// Resident 256-thread blocks per SM asked of the register allocator, per kind and lanes' sites.
-// Measured: on Case 3 (which regenerates often) a lower-occupancy budget lost 10%, and on the
-// random field at S = 31 the 144 registers the allocator takes unasked lost 3% against the
-// 128 asked here.
-template <int KIND, int S>
-struct MinBlocks {
-    static constexpr int value = (S <= 8) ? (quad_kind(KIND) ? 3 : 4) : (S <= 16) ? (quad_kind(KIND) ? 2 : 3) : (S <= 31) ? 2 : 1;
+// Collects the move codes of a step.  The top three bits of floor(d) as a float say how far a site
+// moved: 0b000 (or 0b100, -0) not at all, 0b001 one cell up, 0b101 one cell down, and a set middle
+// bit two cells or more (or not a number).  One funnel shift per site appends them to a word; the
+// codes of a run go round three words, so that code k of word w, shifted, lands on the run's bit.
+template <int S>
+struct MoveCodes {
+    static constexpr int H = S / 2;
+    static constexpr unsigned kOnes = 0x09249249u;
+    unsigned a[3] = {0u, 0u, 0u};   // first run
+    unsigned b[3] = {0u, 0u, 0u};   // second run
+    unsigned last = 0u;
+
+    __device__ __forceinline__ void put(int p, float first, float second)
+    {
+        a[p % 3] = __funnelshift_l(__float_as_uint(first), a[p % 3], 3);
+        b[p % 3] = __funnelshift_l(__float_as_uint(second), b[p % 3], 3);
+    }
+    __device__ __forceinline__ void put_last(float fl) { last = __float_as_uint(fl); }
+
+    // moved: sites that changed cell; down: of those, by one cell downwards (when nothing is far);
+    // far: some site of the lane moved two cells or more, or, unless DOWN, moved downwards
+    template <bool DOWN>
+    __device__ __forceinline__ void masks(typename Moves<S>::mask& moved, typename Moves<S>::mask& down, bool& far) const
+    {
+        using mask = typename Moves<S>::mask;
+        constexpr unsigned kFar = DOWN ? kOnes << 1 : (kOnes << 1) | (kOnes << 2);
+        unsigned mv[2] = {0u, 0u}, dn[2] = {0u, 0u};
+        unsigned any = last & (DOWN ? 0x40000000u : 0xC0000000u);
+#pragma unroll
+        for (int w = 0; w < 3; ++w) {
+            const int n = (H - w + 2) / 3;       // codes in word w
+            if (n <= 0)
+                continue;
+            const int sh = H - 1 - w - 3 * (n - 1);
+            if constexpr (Moves<S>::wide) {
+                const unsigned c[2] = {b[w], a[w]};
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    any |= c[r] & kFar;
+                    mv[r] |= ((c[r] | (c[r] >> 1)) & kOnes) << sh;
+                    if (DOWN)
+                        dn[r] |= ((c[r] >> 2) & kOnes) << sh;
+                }
+            } else {
+                const unsigned c = (a[w] << Moves<S>::D) + b[w];
+                any |= c & kFar;
+                mv[0] += ((c | (c >> 1)) & kOnes) << sh;
+                if (DOWN)
+                    dn[0] += ((c >> 2) & kOnes) << sh;
+            }
+        }
+        moved = mv[0];
+        down = dn[0];
+        if constexpr (Moves<S>::wide) {
+            moved |= static_cast<mask>(mv[1]) << 32;
+            down |= static_cast<mask>(dn[1]) << 32;
+        }
+        if (last & 0x7FFFFFFFu) {
+            moved |= Moves<S>::last;
+            if (DOWN && (last & 0x80000000u))
+                down |= Moves<S>::last;
+        }
+        far = any != 0;
+    }
 };
 
-// Sites per lane are odd: lane l reads its cache at word offsets 2 S l (pair) or 4 S l (quad), and
-// an odd S spreads a half-warp (quarter-warp for 16-byte loads) over distinct shared-memory banks.
-
+// F_p + f of a lane's pair (row t = H - 1 - p) and of its last site, at offsets d, from shared memory.
 template <int KIND, int S>
-__global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_kernel(SplitLaunch a)
+struct Force {
+    const float4* rows;     // loop rows, at this lane
+    const float2* rows_c;
+    pair_t f2;
+
+    // upper: linear-spline random bond, whether the sites are in the upper of their two cells
+    __device__ __forceinline__ pair_t pair(int p, pair_t d, typename Moves<S>::mask upper) const
+    {
+        const int t = S / 2 - 1 - p;
+        if constexpr (KIND == kRF) {
+            const float4 q = rows[32 * t];
+            const pair_t q0 = pk(q.x, q.y), q1 = pk(q.z, q.w);
+            return fma2(d, sub2(q1, q0), q0);
+        } else if constexpr (KIND == kRBGLinear) {
+            const float4 q = rows[32 * t];
+            return add2(pk((upper & Moves<S>::first(p)) ? q.z : q.x, (upper & Moves<S>::second(p)) ? q.w : q.y), f2);
+        } else if constexpr (quad_kind(KIND)) {
+            const float4 q = rows[32 * t];
+            const float2 c = rows_c[32 * t];
+            return fma2(d, fma2(d, pk(c.x, c.y), pk(q.z, q.w)), pk(q.x, q.y));
+        } else {
+            return f2;
+        }
+    }
+    __device__ __forceinline__ float last(float d, typename Moves<S>::mask upper) const
+    {
+        if constexpr (KIND == kRF) {
+            const float4 q = rows[32 * (S / 2)];
+            return fmaf(d, q.z - q.x, q.x);
+        } else if constexpr (KIND == kRBGLinear) {
+            const float4 q = rows[32 * (S / 2)];
+            return ((upper & Moves<S>::last) ? q.z : q.x) + lo(f2);
+        } else if constexpr (quad_kind(KIND)) {
+            const float4 q = rows[32 * (S / 2)];
+            return fmaf(d, fmaf(d, rows_c[32 * (S / 2)].x, q.z), q.x);
+        } else {
+            return lo(f2);
+        }
+    }
+};
+
+// Position of the highest set bit (m != 0).
+__device__ __forceinline__ int mask_top(unsigned m) { return 31 - __clz(m); }
+__device__ __forceinline__ int mask_top(unsigned long long m) { return 63 - __clzll(static_cast<long long>(m)); }
+
+// Registers per thread allowed to the kernel, the fastest measured of 80 .. 184 on each shape.  Both
+// ways cost: at 992-site random-field tiles 120 (and the same 16 warps per SM) instead of 128 lost 3%,
+// 96 lost 23%, and 144 (14 warps) lost 8%; Case 3 redraws less often and gains 1 to 6% from 144 and 168.
+template <int KIND, int S, bool OBS>
+struct MaxRegs {
+    static constexpr int value = (OBS ? 16 : 0) + (quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
+                                 KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 104 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
+                                                      (S <= 8 ? 64 : S <= 16 ? 96 : S <= 31 ? 128 : 160));
+};
+
+// The cell of window position x at this point of the K loop, in every lane.
+template <int KIND, int S>
+__device__ __forceinline__ int32_t cell_at(int32_t* s_cell, int x, int lane, int32_t N0, const pair_t (&c)[S / 2], float cT,
+                                           typename Moves<S>::mask upper)
 {
-    constexpr int TW = 32 * S;
-    constexpr bool kCompact = compact_layout(KIND, S);
-    constexpr bool kFullQueue = full_queue(KIND, S);
-    constexpr int WARP_SMEM = TW * site_smem_bytes(KIND, S) + queue_bytes(KIND, S);
+    constexpr int H = S / 2;
+    if constexpr (KIND == kRBGLinear) {
+        const int src = x / S, j = x - src * S;
+        const int b = (j == 2 * H) ? Moves<S>::D + H : (j < H) ? Moves<S>::D + H - 1 - j : 2 * H - 1 - j;
+        return s_cell[x] + static_cast<int32_t>(__shfl_sync(kFull, upper, src) >> b & 1u);
+    }
+    if constexpr (KIND == kNone) {   // nothing else keeps the slot up to date
+#pragma unroll
+        for (int p = 0; p < H; ++p) {
+            s_cell[lane * S + p] = N0 + __float2int_rn(lo(c[p]));
+            s_cell[lane * S + H + p] = N0 + __float2int_rn(hi(c[p]));
+        }
+        s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
+        __syncwarp();
+    }
+    return s_cell[x];
+}
+
+// Partial sums of F_p, u - r and (u - r)^2 over the owned sites at this point of the K loop, r the
+// reference cell `ref`: FP32 sums over runs of S sites, FP32 warp reduction, then one FP64 shift to
+// the chain's reference in lane 0.  The runs start `len` sites before the tile, where `len` is the
+// number of steps since the last observation, or since the last whole K steps after it: the sums
+// then do not depend on how steps and observations are spread over launches.  Each lane adds up
+// other sites than its own, so the values go through the slot.
+template <int KIND, int S>
+__device__ __forceinline__ void observe_tile(const SplitLaunch& a, const ChainDesc& ch, int tile, int chain, int obs, int32_t ref,
+                                             int owned, int pad, int32_t N0, int lane, const pair_t (&c)[S / 2],
+                                             const pair_t (&d)[S / 2], float cT, float dT, typename Moves<S>::mask upper,
+                                             int32_t* s_cell, float* s_off, const float* s_loop, const float* s_loopc)
+{
+    using T = Tile<KIND, S>;
+    using M = Moves<S>;
+    constexpr int H = S / 2;
+    const float f = ch.f32;
+    const float dref = static_cast<float>(ref - N0);   // exact
+    const int first = lane * S - a.obs_len[obs];       // this lane's run, from the first owned site
+    float* slot = T::has_cache ? reinterpret_cast<float*>(s_cell) : s_off;
+    float sF = 0.0f, sy = 0.0f, syy = 0.0f;
+    int cnt = 0;
+    if constexpr (T::has_cache) {
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
+            const int row = (j < 2 * H) ? H - 1 - p : H;
+            const int half = (j < H || j == 2 * H) ? 0 : 1;
+            const float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
+            const float* q = s_loop + 4 * (32 * row + lane) + half;
+            float F;
+            if constexpr (KIND == kRF)
+                F = fmaf(dj, q[2] - q[0], q[0]) - f;
+            else if constexpr (KIND == kRBGLinear)
+                F = (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last)) ? q[2] : q[0];
+            else
+                F = fmaf(dj, fmaf(dj, s_loopc[2 * (32 * row + lane) + half], q[2]), q[0]) - f;
+            slot[lane * S + j] = F;
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int j = 0; j < S; ++j) {
+            const int o = first + j;
+            if (o >= 0 && o < owned)
+                sF += slot[pad + o];
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
+        const float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
+        const float cj = (j < H) ? lo(c[p]) : (j < 2 * H) ? hi(c[p]) : cT;
+        slot[lane * S + j] = (cj - dref) + dj;   // u - ref
+    }
+    __syncwarp();
+#pragma unroll 4
+    for (int j = 0; j < S; ++j) {
+        const int o = first + j;
+        if (o >= 0 && o < owned) {
+            const float y = slot[pad + o];
+            sy += y;
+            syy = fmaf(y, y, syy);
+            ++cnt;
+        }
+    }
+    if constexpr (T::has_cache) {
+        // the slot's cells again
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
+            int32_t n = N0 + __float2int_rn((j < H) ? lo(c[p]) : (j < 2 * H) ? hi(c[p]) : cT);
+            if (KIND == kRBGLinear && (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last)))
+                n -= 1;
+            s_cell[lane * S + j] = n;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sF += __shfl_down_sync(kFull, sF, o);
+        sy += __shfl_down_sync(kFull, sy, o);
+        syy += __shfl_down_sync(kFull, syy, o);
+        cnt += __shfl_down_sync(kFull, cnt, o);
+    }
+    if (lane == 0) {
+        const double c_ref = a.shift[chain];
+        const double rel = static_cast<double>(ref) - c_ref;
+        const double dsy = sy;
+        double* dst = a.partial + (static_cast<size_t>(obs) * a.partial_stride + a.tile_base + tile) * 4;
+        dst[0] = sF;
+        dst[1] = dsy + cnt * rel;
+        dst[2] = static_cast<double>(syy) + rel * (2.0 * dsy + cnt * rel);
+        dst[3] = c_ref;
+    }
+}
+
+// OBS: whether the launch observes at all.  The observation code in the step loop takes registers
+// from it, so that launches without any (nearly all of a long relaxation's) have a kernel of their own.
+template <int KIND, int S, bool OBS>
+__global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(SplitLaunch a)
+{
+    using T = Tile<KIND, S>;
+    using M = Moves<S>;
+    using mask = typename M::mask;
+    constexpr int H = T::H;
+    constexpr int TW = T::TW;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint64_t s_bar[8];
 
@@ -159,41 +449,32 @@ __global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_ker
     if (tile >= a.n_tiles)
         return;  // whole warp; the kernel uses no block-wide barrier
 
-    unsigned char* wsm = smem_raw + static_cast<size_t>(warp) * WARP_SMEM;
-    int32_t* s_cell = reinterpret_cast<int32_t*>(wsm);          // staging of n (load/store)
-    float* s_off = reinterpret_cast<float*>(wsm + (kCompact ? 0 : 4 * TW));   // staging of d (load/store)
-    // During the K loop the staged cells are the cells the caches were drawn for, and the staged
-    // offsets' slot of each site takes its cell after the step (relative to N0, as a float).
-    int32_t* s_ccell = s_cell;
-    float* s_newc = s_off;
-    int* s_q = reinterpret_cast<int*>(wsm + TW * site_smem_bytes(KIND, S));   // request chunk
-    uint16_t* s_q16 = reinterpret_cast<uint16_t*>(s_q);                       // or all of a step
-    // compact layout: staging at 0, the node pair at 4 TW, cache cells (low 16 bits) at 12 TW
-    float2* s_rf = reinterpret_cast<float2*>(wsm + (kCompact ? 4 : 8) * TW);
-    uint16_t* s_cc16 = reinterpret_cast<uint16_t*>(wsm + 12 * TW);
-    float2* s_qn = reinterpret_cast<float2*>(wsm + 8 * TW);     // cubic nodes V(n), V(n+1)
-    float* s_q3 = reinterpret_cast<float*>(wsm + 16 * TW);      // and V(n+2)
-    float2* s_ab = reinterpret_cast<float2*>(wsm + 20 * TW);    // cubic coefficients (A, B)
-    float* s_c = reinterpret_cast<float*>(wsm + 28 * TW);       // and C
+    unsigned char* wsm = smem_raw + static_cast<size_t>(warp) * T::bytes;
+    int32_t* s_cell = reinterpret_cast<int32_t*>(wsm + T::slot);
+    float* s_off = reinterpret_cast<float*>(wsm + T::slot2);
+    float* s_loop = reinterpret_cast<float*>(wsm + T::loop);     // loop rows as floats
+    float* s_loopc = reinterpret_cast<float*>(wsm + T::loopc);
+    float* s_top = reinterpret_cast<float*>(wsm + T::top);
+    float2* s_nodes = reinterpret_cast<float2*>(wsm + T::nodes);
+    uint16_t* s_q = reinterpret_cast<uint16_t*>(wsm + T::queue);
 
     const TileDesc td = a.tiles[tile];
     const ChainDesc ch = a.chains[td.chain];
     const int32_t L = ch.L;
     const int K = a.K;
+    const int pad = a.pad;   // first owned window position
     const int owned = min(a.w_own, L - td.start);
-    const int64_t wstart = static_cast<int64_t>(td.start) - K;
+    const int64_t wstart = static_cast<int64_t>(td.start) - pad;
     const bool contiguous = (wstart >= 0) && (wstart + TW <= L);
     const float f = ch.f32;
-    const float dt = a.dt;
     const uint32_t s = ch.s;
-    const int32_t M = ch.period;
+    const int32_t period = ch.period;
 
     // ---- stage the window in this warp's shared-memory slice ----
     // Contiguous, 16-byte aligned windows arrive by TMA bulk copies (one per array, completion
     // on the warp's mbarrier); windows that wrap around the chain or start unaligned use
-    // coalesced read-only loads.
-    // The compact layout stages cells and offsets one after the other through the same slot:
-    // cells (with the node pairs) first, then offsets.
+    // coalesced read-only loads.  Offsets come first, with the cache, and then the cells through
+    // the same slot, where they stay.
     const bool tma_in = contiguous && (((ch.offset + wstart) & 3) == 0);
     const int64_t p0 = ch.offset + wstart;
     uint64_t* bar = &s_bar[warp];
@@ -204,23 +485,19 @@ __global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_ker
         }
         __syncwarp();
         if (lane == 0) {
-            if constexpr (kCompact) {
-                mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm));
+            mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::has_cache ? 0 : 4)));
+            tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
+            if constexpr (!T::has_cache)
                 tma_load_1d(s_cell, a.in.cell + p0, TW * 4, bar);
-                tma_load_1d(s_rf, a.in.rf + p0, TW * 8, bar);
-            } else {
-                mbar_arrive_expect_tx(bar, TW * (8 + CacheBytes<KIND>::hbm));
-                tma_load_1d(s_cell, a.in.cell + p0, TW * 4, bar);
-                tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
-                if constexpr (pair_kind(KIND))
-                    tma_load_1d(s_rf, a.in.rf + p0, TW * 8, bar);
-                if constexpr (quad_kind(KIND)) {
-                    tma_load_1d(s_qn, a.in.qn + p0, TW * 8, bar);
-                    tma_load_1d(s_q3, a.in.q3 + p0, TW * 4, bar);
-                    tma_load_1d(s_ab, a.in.qab + p0, TW * 8, bar);
-                    tma_load_1d(s_c, a.in.qc + p0, TW * 4, bar);
-                }
+            if constexpr (T::has_pair)
+                tma_load_1d(s_loop, a.in.rf + p0, TW * 8, bar);
+            if constexpr (T::has_quad) {
+                tma_load_1d(s_nodes, a.in.qn + p0, TW * 8, bar);
+                tma_load_1d(s_loop, a.in.qab + p0, TW * 8, bar);
+                tma_load_1d(s_loopc, a.in.qc + p0, TW * 4, bar);
             }
+            if constexpr (T::has_quad || KIND == kRBGLinear)
+                tma_load_1d(s_top, a.in.q3 + p0, TW * 4, bar);
         }
         const bool landed = __all_sync(kFull, mbar_wait(bar, 0));   // warp-uniform outcome
         if (!landed) {
@@ -231,46 +508,74 @@ __global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_ker
             return;
         }
     } else {
-        const int32_t* __restrict__ g_cell = a.in.cell;
-        const float* __restrict__ g_off = a.in.off;
         for (int x = lane; x < TW; x += 32) {
             const int64_t p = ch.offset + site_index(wstart, x, contiguous, L);
-            s_cell[x] = __ldg(g_cell + p);
-            if constexpr (!kCompact)
-                s_off[x] = __ldg(g_off + p);
-            if constexpr (pair_kind(KIND))
-                s_rf[x] = __ldg(a.in.rf + p);
-            if constexpr (quad_kind(KIND)) {
-                s_qn[x] = __ldg(a.in.qn + p);
-                s_q3[x] = __ldg(a.in.q3 + p);
-                s_ab[x] = __ldg(a.in.qab + p);
-                s_c[x] = __ldg(a.in.qc + p);
+            s_off[x] = __ldg(a.in.off + p);
+            if constexpr (!T::has_cache)
+                s_cell[x] = __ldg(a.in.cell + p);
+            if constexpr (T::has_pair)
+                reinterpret_cast<float2*>(s_loop)[x] = __ldg(a.in.rf + p);
+            if constexpr (T::has_quad) {
+                s_nodes[x] = __ldg(a.in.qn + p);
+                reinterpret_cast<float2*>(s_loop)[x] = __ldg(a.in.qab + p);
+                s_loopc[x] = __ldg(a.in.qc + p);
             }
+            if constexpr (T::has_quad || KIND == kRBGLinear)
+                s_top[x] = __ldg(a.in.q3 + p);
         }
         __syncwarp();
     }
 
-    // Cells are carried as exact small floats relative to the warp's reference cell N0 (window
-    // position 0): a neighbour difference is then (c' - c) + (d' - d), three FP32 operations.
-    // Neighbouring displacements differ by less than 2^12, so a tile's cells stay far below 2^24.
-    const int32_t N0 = s_cell[0];
-    float c[S];
-    float d[S];
-    if constexpr (kCompact) {
+    // Offsets, two sites to a register pair.  Of a linear-spline random-bond site the sign bit says
+    // that it is in the upper of its two cached cells (offsets themselves are never negative).
+    pair_t c[H], d[H];
+    float cT, dT;
+    mask upper = 0;
+#pragma unroll
+    for (int p = 0; p < H; ++p) {
+        float d0 = s_off[lane * S + p], d1 = s_off[lane * S + H + p];
+        if constexpr (KIND == kRBGLinear) {
+            if (__float_as_int(d0) < 0)
+                upper |= M::first(p);
+            if (__float_as_int(d1) < 0)
+                upper |= M::second(p);
+            d0 = fabsf(d0);
+            d1 = fabsf(d1);
+        }
+        d[p] = pk(d0, d1);
+    }
+    dT = s_off[lane * S + 2 * H];
+    if constexpr (KIND == kRBGLinear) {
+        if (__float_as_int(dT) < 0)
+            upper |= M::last;
+        dT = fabsf(dT);
+    }
+    // The cache, from the linear order of memory to the rows of the update loop.
+    if constexpr (T::has_cache) {
+        float2 q[S];
+        float qc[S];
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            const int x = lane * S + j;
-            const int32_t n = s_cell[x];
-            c[j] = static_cast<float>(n - N0);
-            s_cc16[x] = static_cast<uint16_t>(n);
+            q[j] = reinterpret_cast<float2*>(s_loop)[lane * S + j];
+            if constexpr (T::has_quad)
+                qc[j] = s_loopc[lane * S + j];
         }
-        // every lane has read its cells: the offsets may now overwrite the staging slot
+        __syncwarp();   // every lane has read: the rows may overwrite the linear order
+#pragma unroll
+        for (int p = 0; p <= H; ++p) {
+            const int row = (p < H) ? H - 1 - p : H;
+            const int j0 = (p < H) ? p : 2 * H, j1 = (p < H) ? H + p : 2 * H;
+            reinterpret_cast<float4*>(s_loop)[32 * row + lane] = make_float4(q[j0].x, q[j1].x, q[j0].y, q[j1].y);
+            if constexpr (T::has_quad)
+                reinterpret_cast<float2*>(s_loopc)[32 * row + lane] = make_float2(qc[j0], qc[j1]);
+        }
+        // the offsets are in registers: the cells may overwrite the slot
         fence_proxy_async_shared();
         __syncwarp();
         if (tma_in) {
             if (lane == 0) {
                 mbar_arrive_expect_tx(bar, TW * 4);
-                tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
+                tma_load_1d(s_cell, a.in.cell + p0, TW * 4, bar);
             }
             const bool landed = __all_sync(kFull, mbar_wait(bar, 1));
             if (!landed) {
@@ -281,229 +586,239 @@ __global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_ker
             }
         } else {
             for (int x = lane; x < TW; x += 32)
-                s_off[x] = __ldg(a.in.off + ch.offset + site_index(wstart, x, contiguous, L));
+                s_cell[x] = __ldg(a.in.cell + ch.offset + site_index(wstart, x, contiguous, L));
             __syncwarp();
         }
     }
+    // Cells are carried as exact small floats relative to the warp's reference cell N0 (window
+    // position 0): a neighbour difference is then (c' - c) + (d' - d), three FP32 operations.
+    // Neighbouring displacements differ by less than 2^12, so a tile's cells stay far below 2^24.
+    const int32_t N0 = s_cell[0];
 #pragma unroll
-    for (int j = 0; j < S; ++j) {
-        const int x = lane * S + j;
-        if constexpr (!kCompact)
-            c[j] = static_cast<float>(s_cell[x] - N0);
-        d[j] = s_off[x];
+    for (int p = 0; p < H; ++p)
+        c[p] = pk(static_cast<float>(s_cell[lane * S + p] - N0), static_cast<float>(s_cell[lane * S + H + p] - N0));
+    cT = static_cast<float>(s_cell[lane * S + 2 * H] - N0);
+    __syncwarp();   // N0 is read by every lane before any cell changes
+    if constexpr (KIND == kRBGLinear) {
+        // from here on the slot holds the lower of each site's two cached cells
+#pragma unroll
+        for (int p = 0; p < H; ++p) {
+            if (upper & M::first(p))
+                s_cell[lane * S + p] -= 1;
+            if (upper & M::second(p))
+                s_cell[lane * S + H + p] -= 1;
+        }
+        if (upper & M::last)
+            s_cell[lane * S + 2 * H] -= 1;
+        __syncwarp();
     }
-    __syncwarp();   // the staging area becomes the request queue below
+
+    Force<KIND, S> force;
+    force.rows = reinterpret_cast<const float4*>(s_loop) + lane;
+    force.rows_c = reinterpret_cast<const float2*>(s_loopc) + lane;
+    force.f2 = pk(f, f);
+    const pair_t dt2 = pk(a.dt, a.dt);
 
     // ---- K Euler steps: state in registers, cache in shared memory ----
     unsigned n_cross = 0;
+    const unsigned lanes_below = (1u << lane) - 1u;
+    // observations inside the launch: the next one, the reference cell of its sums, and the step
+    // before which the next thing has to be done about it
+    int obs = 0, obs_ref = 0, obs_step = OBS ? a.obs_at[0] - a.obs_len[0] : -1;
+    bool obs_marked = false;
 #pragma unroll 1
-    for (int k = 0; k < K; ++k) {
+    for (int k = 0;; ++k) {
+        while (OBS && k == obs_step) {
+            if (!obs_marked) {
+                // the sums are relative to the cell, at this step, of the site `len` before the tile
+                obs_ref = cell_at<KIND, S>(s_cell, pad - a.obs_len[obs], lane, N0, c, cT, upper);
+                obs_marked = true;
+            } else {
+                observe_tile<KIND, S>(a, ch, tile, td.chain, obs, obs_ref, owned, pad, N0, lane, c, d, cT, dT, upper, s_cell,
+                                      s_off, s_loop, s_loopc);
+                obs_marked = false;
+                ++obs;
+            }
+            obs_step = (obs < a.n_obs) ? a.obs_at[obs] - (obs_marked ? 0 : a.obs_len[obs]) : -1;
+        }
+        if (k == K)
+            break;
         // Window positions 0 and TW - 1 take themselves as their outer neighbour: they go stale
         // either way, and a zero slope there keeps the stale edge from drifting off and making
         // spurious cell moves (each of which would draw disorder values).
-        const float cl0 = __shfl_up_sync(kFull, c[S - 1], 1);
-        const float dl0 = __shfl_up_sync(kFull, d[S - 1], 1);
-        const float cr0 = __shfl_down_sync(kFull, c[0], 1);
-        const float dr0 = __shfl_down_sync(kFull, d[0], 1);
-        const float cl = (lane == 0) ? c[0] : cl0;
-        const float dl = (lane == 0) ? d[0] : dl0;
-        const float cr = (lane == 31) ? c[S - 1] : cr0;
-        const float drn = (lane == 31) ? d[S - 1] : dr0;
-        float Dm = (c[0] - cl) + (d[0] - dl);   // u_j - u_{j-1}
-        MoveMask<S> mv = 0;   // sites that changed cell in this step (bit j: the lane's site j)
+        const float cr = __shfl_down_sync(kFull, lo(c[0]), 1);
+        const float dr = __shfl_down_sync(kFull, lo(d[0]), 1);
+        const float DpT = (lane == 31) ? 0.0f : (cr - cT) + (dr - dT);   // the lane's last site to its right
+        const float Dl0 = __shfl_up_sync(kFull, DpT, 1);
+        const float Dl = (lane == 0) ? 0.0f : Dl0;                       // to the lane's first site
+        // the last pair's right neighbours: the second run's first site, and the last site
+        const pair_t DpL = add2(sub2(pk(hi(c[0]), cT), c[H - 1]), sub2(pk(hi(d[0]), dT), d[H - 1]));
+        pair_t Dm = pk(Dl, lo(DpL));   // u_j - u_{j-1}
+        MoveCodes<S> codes;
 #pragma unroll
-        for (int j = 0; j < S; ++j) {
-            const int x = lane * S + j;
-            const float cn = (j + 1 < S) ? c[j + 1] : cr;
-            const float dd = (j + 1 < S) ? d[j + 1] : drn;
-            const float Dp = (cn - c[j]) + (dd - d[j]);   // u_{j+1} - u_j
-            const float g = drive_plus_pinning<KIND>(s_rf, s_ab, s_c, x, d[j], f);   // F_p + f
-            const float dn = fmaf(dt, (Dp - Dm) + g, d[j]);
+        for (int p = 0; p < H; ++p) {
+            const pair_t Dp = (p + 1 < H) ? add2(sub2(c[p + 1 < H ? p + 1 : p], c[p]), sub2(d[p + 1 < H ? p + 1 : p], d[p])) : DpL;
+            const pair_t g = force.pair(p, d[p], upper);   // F_p + f
+            const pair_t dn = fma2(dt2, add2(sub2(Dp, Dm), g), d[p]);
             Dm = Dp;
             // Branch-free renormalisation.  d - floor(d) is exact; a tiny negative d can round up
             // to exactly 1, which is a valid representation (the interpolated force is continuous).
-            const float fl = floorf(dn);
-            c[j] += fl;
-            d[j] = dn - fl;
-            mv |= (fl != 0.0f) ? (MoveMask<S>(1) << j) : MoveMask<S>(0);
+            const pair_t fl = floor2(dn);
+            c[p] = add2(c[p], fl);
+            d[p] = sub2(dn, fl);
+            codes.put(p, lo(fl), hi(fl));
         }
-        const unsigned anymv = __reduce_or_sync(kFull, mv);
-        if (anymv) {
-            // the lane's cells after the step, read by the consumers below for the moved sites
-            if constexpr (KIND != kNone) {
-#pragma unroll
-                for (int j = 0; j < S; ++j)
-                    s_newc[lane * S + j] = c[j];
-            }
-            // queue slots: warp prefix sum of the lanes' move counts; each lane then walks the set
-            // bits of its mask.  Chunks of 32 requests, one Philox value per lane and chunk.
-            const int cnt = mask_popc(mv);
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o)
-                    incl += y;
-            }
-            const int qn = __shfl_sync(kFull, incl, 31);
-            n_cross += static_cast<unsigned>(qn);   // the same in every lane
-            if constexpr (KIND != kNone) {
-                // each lane's walk resumes in the next chunk where it stopped
-                int q = incl - cnt;
-                MoveMask<S> m = mv;
-                if constexpr (kFullQueue) {
-                    // every request of the step at once (a site is queued at most once: qn <= TW)
-                    while (m != 0) {
-                        const int b = mask_ffs(m) - 1;
-                        m &= m - 1;
-                        s_q16[q] = static_cast<uint16_t>(lane * S + b);
-                        ++q;
-                    }
-                    __syncwarp();
+        {
+            const float g = force.last(dT, upper);
+            const float dn = fmaf(a.dt, (DpT - hi(DpL)) + g, dT);
+            const float fl = floorf(dn);
+            cT += fl;
+            dT = dn - fl;
+            codes.put_last(fl);
+        }
+        mask moved = 0, down = 0;
+        bool lane_far = false;
+        if (T::has_cache || a.crossings)
+            codes.template masks<T::kDown>(moved, down, lane_far);
+        if (a.crossings)
+            n_cross += __reduce_add_sync(kFull, static_cast<unsigned>(mask_popc(moved)));
+        if constexpr (T::has_cache) {
+            const bool far = __any_sync(kFull, lane_far);
+            // requests: sites whose cache has to change
+            mask req = moved;
+            if constexpr (KIND == kRBGLinear) {
+                down &= moved;
+                const mask up = moved & ~down;
+                if (!far) {
+                    req = (up & upper) | (down & ~upper);
+                    upper = (upper | up) & ~down;
+                } else {
+                    upper &= ~moved;   // redrawn with the new cell as the lower one
                 }
-                for (int base = 0; base < qn; base += 32) {
-                    if constexpr (!kFullQueue) {
-                        while (m != 0 && q < base + 32) {
-                            const int b = mask_ffs(m) - 1;
-                            m &= m - 1;
-                            s_q[q - base] = lane * S + b;   // window position of the site
-                            ++q;
+            }
+            if (far) {
+                // some site moved two cells or more: the lanes leave their new cells in the slot,
+                // and every site that moved redraws all of its nodes
+#pragma unroll
+                for (int p = 0; p < H; ++p) {
+                    if (KIND != kRBGLinear || (moved & M::first(p)))
+                        s_cell[lane * S + p] = N0 + __float2int_rn(lo(c[p]));
+                    if (KIND != kRBGLinear || (moved & M::second(p)))
+                        s_cell[lane * S + H + p] = N0 + __float2int_rn(hi(c[p]));
+                }
+                if (KIND != kRBGLinear || (moved & M::last))
+                    s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
+            }
+            // Queue the requests, one per lane and pass: a lane's slot is its rank in the ballot of the
+            // lanes that still have one (no prefix sum; three or four passes empty the masks)
+            unsigned have = __ballot_sync(kFull, req != 0);
+            if (have) {
+                do {
+                    int n_here = 0;
+                    do {
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            const int b = mask_top(req);
+                            unsigned e = (lane << 7) + b;
+                            if (T::kDown)
+                                e += static_cast<unsigned>(down >> (b & (M::wide ? 63 : 31)) & 1u) << 6;
+                            const int q = n_here + __popc(have & lanes_below);
+                            if (req != 0)
+                                s_q[q] = static_cast<uint16_t>(e);
+                            req = mask_drop(req, b);
+                            n_here += __popc(have);
+                            have = __ballot_sync(kFull, req != 0);
+                        }
+                    } while (have && n_here <= T::kQueue - 64);
+                    __syncwarp();
+                    for (int base = 0; base < n_here; base += 32) {
+                        if (base + lane < n_here) {
+                            const int e = s_q[base + lane];
+                            const int b = e & 63, src = e >> 7;
+                            const bool first = b >= M::D;
+                            const int t = first ? b - M::D : b;            // row of the pair
+                            const int x = src * S + (H - 1 - t) + (first ? 0 : H) + (t == H ? S : 0);
+                            float* row = s_loop + 4 * (32 * t + src) + (first ? 0 : 1);
+                            const int step = far ? 0 : (T::kDown && (e & 64)) ? -1 : 1;
+                            const int32_t i = contiguous ? static_cast<int32_t>(wstart) + x
+                                                         : site_index(wstart, x, contiguous, L);
+                            const int32_t slot = s_cell[x];
+                            if constexpr (KIND == kRF) {
+                                // an up move keeps R(n) and draws R(n+1); a far move draws both
+                                const int32_t nn = slot + step;
+                                const float old = row[2];
+                                const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 1, period), f);
+                                row[0] = far ? pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn, period), f) : old;
+                                row[2] = v;
+                                if (!far)
+                                    s_cell[x] = nn;
+                            } else if constexpr (KIND == kRBGLinear) {
+                                // the pair of cells moves up (n = slot + 2 is the new upper cell, one new
+                                // node), down or, after a far move, starts anew at n = slot: three nodes
+                                const bool up = step > 0;
+                                const int32_t base_n = up ? slot + 3 : slot + step;
+                                const int trips = up ? 1 : 3;
+                                float g0 = row[2], g1 = 0.0f, prev = s_top[x];
+#pragma unroll 1
+                                for (int r = 0; r < trips; ++r) {
+                                    const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(base_n + r, period), f);
+                                    const float g = prev - v;   // F_p of the cell between the two nodes
+                                    if (!up && r == 1)
+                                        g0 = g;
+                                    else
+                                        g1 = g;
+                                    prev = v;
+                                }
+                                row[0] = g0;
+                                row[2] = g1;
+                                s_top[x] = prev;
+                                s_cell[x] = slot + step;
+                            } else {
+                                // The spline over the new cell n needs V(n-1 .. n+2).  The cache holds
+                                // V, V(+1), V(+2) of the old cell: an up move draws V(n+2), a down move
+                                // V(n-1) and V(n) (V(n-1) is not kept), a far move all four.
+                                const int32_t nn = slot + step;
+                                if (!far)
+                                    s_cell[x] = nn;
+                                const bool up = step > 0;
+                                const float2 o = s_nodes[x];
+                                float n0 = o.x, n1 = o.y, n2 = s_top[x];
+                                float n3 = quad_node_f32<KIND>(a.keys, s, i, wrap_node(up ? nn + 2 : nn - 1, period));
+                                if (!up) {
+                                    const float v = n3;
+                                    n3 = n1;
+                                    n2 = n0;
+                                    n0 = v;
+#pragma unroll 1
+                                    for (int r = 0; r < (far ? 3 : 1); ++r) {
+                                        const float w = quad_node_f32<KIND>(a.keys, s, i, wrap_node(nn + r, period));
+                                        if (r == 0)
+                                            n1 = w;
+                                        else if (r == 1)
+                                            n2 = w;
+                                        else
+                                            n3 = w;
+                                    }
+                                }
+                                s_nodes[x] = make_float2(n1, n2);
+                                s_top[x] = n3;
+                                float A, B, C;
+                                rb_coefficients(n0, n1, n2, n3, f, A, B, C);
+                                row[0] = A;
+                                row[2] = B;
+                                s_loopc[2 * (32 * t + src) + (first ? 0 : 1)] = C;
+                            }
                         }
                         __syncwarp();
                     }
-                    if (base + lane < qn) {
-                        const int x = kFullQueue ? static_cast<int>(s_q16[base + lane]) : s_q[lane];
-                        const int nn = N0 + __float2int_rn(s_newc[x]);
-                        int move;   // cells moved in this step
-                        if constexpr (kCompact) {
-                            // from the low 16 bits: exact while a step moves a site by less than
-                            // 2^15 cells (|dt (lap + f + F_p)| < 2^15; split_range_guard checks the
-                            // neighbour differences that keep it so at every observation)
-                            move = static_cast<int16_t>(static_cast<uint16_t>(nn) - s_cc16[x]);
-                            s_cc16[x] = static_cast<uint16_t>(nn);
-                        } else {
-                            move = nn - s_ccell[x];
-                            s_ccell[x] = nn;
-                        }
-                        const int code = (move == 1) ? kMoveUp : (move == -1) ? kMoveDown : kMoveFar;
-                        const int32_t i = contiguous ? static_cast<int32_t>(wstart) + x
-                                                     : site_index(wstart, x, contiguous, L);
-                        if constexpr (pair_kind(KIND) && S < 31) {
-                            // one new node, n+1 after an up move and n after a down move; a far move
-                            // draws n and n+1.  One call site, with a second trip only for far moves:
-                            // a second inlined transform would spill registers at S <= 15.
-                            const float2 o = s_rf[x];
-                            float2 q = (code == kMoveUp) ? make_float2(o.y, 0.0f) : make_float2(0.0f, o.x);
-                            const int n0 = (code == kMoveUp) ? nn + 1 : nn;
-                            const int trips = (code == kMoveFar) ? 2 : 1;
-#pragma unroll 1
-                            for (int r = 0; r < trips; ++r) {
-                                const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(n0 + r, M), f);
-                                if (code == kMoveUp || r == 1)
-                                    q.y = v;
-                                else
-                                    q.x = v;
-                            }
-                            s_rf[x] = q;
-                        } else if constexpr (pair_kind(KIND)) {
-                            // the same draws with the far-move node inline: at S = 31 the register
-                            // budget binds either way and this form measured 0.5% faster
-                            const float v =
-                                pair_node_f32<KIND>(a.keys, s, i, wrap_node(code == kMoveUp ? nn + 1 : nn, M), f);
-                            const float2 o = s_rf[x];
-                            float2 q;
-                            if (code == kMoveUp)
-                                q = make_float2(o.y, v);
-                            else if (code == kMoveDown)
-                                q = make_float2(v, o.x);
-                            else
-                                q = make_float2(v, pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 1, M), f));
-                            s_rf[x] = q;
-                        } else {
-                            // The spline over the new cell nn needs V(nn-1 .. nn+2).  The cache
-                            // holds V(n), V(n+1), V(n+2) of the old cell n: an up move draws
-                            // V(nn+2); a down move draws V(nn-1) and V(nn) (V(n-1) is not kept:
-                            // at the thresholds down moves are a few in 10^4); a far move draws
-                            // all four.
-                            const float v =
-                                quad_node_f32<KIND>(a.keys, s, i, wrap_node(code == kMoveUp ? nn + 2 : nn - 1, M));
-                            const float2 o = s_qn[x];
-                            float p0, p1, p2, p3;
-                            if (code == kMoveUp) {
-                                p0 = o.x;
-                                p1 = o.y;
-                                p2 = s_q3[x];
-                                p3 = v;
-                            } else {
-                                p0 = v;
-                                p1 = quad_node_f32<KIND>(a.keys, s, i, wrap_node(nn, M));
-                                if (code == kMoveDown) {
-                                    p2 = o.x;
-                                    p3 = o.y;
-                                } else {
-                                    p2 = quad_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 1, M));
-                                    p3 = quad_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 2, M));
-                                }
-                            }
-                            s_qn[x] = make_float2(p1, p2);
-                            s_q3[x] = p3;
-                            float A, B, C;
-                            rb_coefficients(p0, p1, p2, p3, f, A, B, C);
-                            s_ab[x] = make_float2(A, B);
-                            s_c[x] = C;
-                        }
-                    }
-                    __syncwarp();
-                }
+                } while (have);
             }
         }
     }
 
     if (a.crossings) {
-        const unsigned tot = n_cross;
-        if (lane == 0 && tot)
-            atomicAdd(a.crossings, static_cast<unsigned long long>(tot));
-    }
-
-    // ---- checkpoint partial sums of the state after the K steps (owned sites only) ----
-    // FP32 sums relative to the warp's reference cell (lane 0's first site; the spread inside a
-    // tile is small), FP32 warp reduction, then one FP64 shift to the chain reference in lane 0.
-    if (a.do_obs) {
-        const int32_t c_ref = static_cast<int32_t>(a.shift[td.chain]);
-        float sF = 0.0f, sy = 0.0f, syy = 0.0f;
-        int cnt = 0;
-#pragma unroll
-        for (int j = 0; j < S; ++j) {
-            const int x = lane * S + j;
-            const int o = x - K;
-            if (o >= 0 && o < owned) {
-                if constexpr (KIND == kRBGLinear) {
-                    const float2 q = s_rf[x];
-                    sF += q.x - q.y;
-                } else {
-                    sF += drive_plus_pinning<KIND>(s_rf, s_ab, s_c, x, d[j], f) - f;
-                }
-                const float y = c[j] + d[j];   // u - N0
-                sy += y;
-                syy = fmaf(y, y, syy);
-                ++cnt;
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sF += __shfl_down_sync(kFull, sF, o);
-            sy += __shfl_down_sync(kFull, sy, o);
-            syy += __shfl_down_sync(kFull, syy, o);
-            cnt += __shfl_down_sync(kFull, cnt, o);
-        }
-        if (lane == 0) {
-            const double rel = static_cast<double>(N0) - static_cast<double>(c_ref);
-            const double dsy = sy;
-            double* dst = a.partial + static_cast<size_t>(a.tile_base + tile) * 3;
-            dst[0] = sF;
-            dst[1] = dsy + cnt * rel;
-            dst[2] = static_cast<double>(syy) + rel * (2.0 * dsy + cnt * rel);
-        }
+        if (lane == 0 && n_cross)
+            atomicAdd(a.crossings, static_cast<unsigned long long>(n_cross));
     }
 
     if (K == 0)
@@ -512,98 +827,115 @@ __global__ void __launch_bounds__(256, MinBlocks<KIND, S>::value) split_step_ker
     // ---- write the owned sites back: registers -> shared -> global ----
     __syncwarp();
     const int64_t out0 = ch.offset + td.start;
-    const bool tma_out = ((K & 3) == 0) && ((out0 & 3) == 0) && ((owned & 3) == 0);
-    if constexpr (kCompact) {
-        // cells and node pairs first, then the offsets through the same staging slot
+    const bool tma_out = ((pad & 3) == 0) && ((out0 & 3) == 0) && ((owned & 3) == 0);
+    if constexpr (!T::has_cache || KIND == kRBGLinear) {
+        // (the other kinds' slots already hold the cells)
 #pragma unroll
-        for (int j = 0; j < S; ++j)
-            s_cell[lane * S + j] = N0 + __float2int_rn(c[j]);
-        if (tma_out) {
-            fence_proxy_async_shared();
-            __syncwarp();
-            if (lane == 0) {
-                const uint32_t cnt = static_cast<uint32_t>(owned);
-                tma_store_1d(a.out.cell + out0, s_cell + K, cnt * 4);
-                tma_store_1d(a.out.rf + out0, s_rf + K, cnt * 8);
-                tma_store_commit();
-                tma_store_wait_read_all();   // the staging slot may be overwritten
-            }
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < S; ++j)
-                s_off[lane * S + j] = d[j];
-            fence_proxy_async_shared();
-            __syncwarp();
-            if (lane == 0) {
-                tma_store_1d(a.out.off + out0, s_off + K, static_cast<uint32_t>(owned) * 4);
-                tma_store_commit();
-                tma_store_wait_all();
-            }
-        } else {
-            __syncwarp();
-            for (int o = lane; o < owned; o += 32) {
-                a.out.cell[out0 + o] = s_cell[o + K];
-                a.out.rf[out0 + o] = s_rf[o + K];
-            }
-            __syncwarp();
-#pragma unroll
-            for (int j = 0; j < S; ++j)
-                s_off[lane * S + j] = d[j];
-            __syncwarp();
-            for (int o = lane; o < owned; o += 32)
-                a.out.off[out0 + o] = s_off[o + K];
+        for (int p = 0; p < H; ++p) {
+            s_cell[lane * S + p] = N0 + __float2int_rn(lo(c[p]));
+            s_cell[lane * S + H + p] = N0 + __float2int_rn(hi(c[p]));
         }
-    } else {
+        s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
+    }
+    if constexpr (T::has_cache) {
+        // the cache back to linear order
+        float2 q[S];
+        float qc[S];
+#pragma unroll
+        for (int p = 0; p <= H; ++p) {
+            const int row = (p < H) ? H - 1 - p : H;
+            const int j0 = (p < H) ? p : 2 * H;
+            const float4 r = reinterpret_cast<const float4*>(s_loop)[32 * row + lane];
+            q[j0] = make_float2(r.x, r.z);
+            if (p < H)
+                q[H + (p < H ? p : 0)] = make_float2(r.y, r.w);
+            if constexpr (T::has_quad) {
+                const float2 r2 = reinterpret_cast<const float2*>(s_loopc)[32 * row + lane];
+                qc[j0] = r2.x;
+                if (p < H)
+                    qc[H + (p < H ? p : 0)] = r2.y;
+            }
+        }
+        __syncwarp();
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            const int x = lane * S + j;
-            s_cell[x] = N0 + __float2int_rn(c[j]);
-            s_off[x] = d[j];
+            reinterpret_cast<float2*>(s_loop)[lane * S + j] = q[j];
+            if constexpr (T::has_quad)
+                s_loopc[lane * S + j] = qc[j];
         }
         if (tma_out) {
             fence_proxy_async_shared();   // generic-proxy writes above -> visible to the bulk copy
             __syncwarp();
             if (lane == 0) {
                 const uint32_t cnt = static_cast<uint32_t>(owned);
-                tma_store_1d(a.out.cell + out0, s_cell + K, cnt * 4);
-                tma_store_1d(a.out.off + out0, s_off + K, cnt * 4);
-                if constexpr (pair_kind(KIND))
-                    tma_store_1d(a.out.rf + out0, s_rf + K, cnt * 8);
-                if constexpr (quad_kind(KIND))
-                {
-                    tma_store_1d(a.out.qn + out0, s_qn + K, cnt * 8);
-                    tma_store_1d(a.out.q3 + out0, s_q3 + K, cnt * 4);
-                    tma_store_1d(a.out.qab + out0, s_ab + K, cnt * 8);
-                    tma_store_1d(a.out.qc + out0, s_c + K, cnt * 4);
+                tma_store_1d(a.out.cell + out0, s_cell + pad, cnt * 4);
+                if constexpr (T::has_pair)
+                    tma_store_1d(a.out.rf + out0, reinterpret_cast<float2*>(s_loop) + pad, cnt * 8);
+                if constexpr (T::has_quad) {
+                    tma_store_1d(a.out.qn + out0, s_nodes + pad, cnt * 8);
+                    tma_store_1d(a.out.qab + out0, reinterpret_cast<float2*>(s_loop) + pad, cnt * 8);
+                    tma_store_1d(a.out.qc + out0, s_loopc + pad, cnt * 4);
                 }
+                if constexpr (T::has_quad || KIND == kRBGLinear)
+                    tma_store_1d(a.out.q3 + out0, s_top + pad, cnt * 4);
                 tma_store_commit();
-                tma_store_wait_all();
+                tma_store_wait_read_all();   // the slot may be overwritten
             }
+            __syncwarp();
         } else {
             __syncwarp();
             for (int o = lane; o < owned; o += 32) {
-                const int x = o + K;
+                const int x = o + pad;
                 const int64_t p = out0 + o;
                 a.out.cell[p] = s_cell[x];
-                a.out.off[p] = s_off[x];
-                if constexpr (pair_kind(KIND))
-                    a.out.rf[p] = s_rf[x];
-                if constexpr (quad_kind(KIND)) {
-                    a.out.qn[p] = s_qn[x];
-                    a.out.q3[p] = s_q3[x];
-                    a.out.qab[p] = s_ab[x];
-                    a.out.qc[p] = s_c[x];
+                if constexpr (T::has_pair)
+                    a.out.rf[p] = reinterpret_cast<float2*>(s_loop)[x];
+                if constexpr (T::has_quad) {
+                    a.out.qn[p] = s_nodes[x];
+                    a.out.qab[p] = reinterpret_cast<float2*>(s_loop)[x];
+                    a.out.qc[p] = s_loopc[x];
                 }
+                if constexpr (T::has_quad || KIND == kRBGLinear)
+                    a.out.q3[p] = s_top[x];
             }
+            __syncwarp();
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
+        float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
+        if constexpr (KIND == kRBGLinear) {
+            if (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last))
+                dj = -dj;
+        }
+        s_off[lane * S + j] = dj;
+    }
+    if (tma_out) {
+        fence_proxy_async_shared();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_1d(a.out.off + out0, s_off + pad, static_cast<uint32_t>(owned) * 4);
+            if constexpr (!T::has_cache)
+                tma_store_1d(a.out.cell + out0, s_cell + pad, static_cast<uint32_t>(owned) * 4);
+            tma_store_commit();
+            tma_store_wait_read_all();   // shared memory must outlive the reads; the writes end with the kernel
+        }
+    } else {
+        __syncwarp();
+        for (int o = lane; o < owned; o += 32) {
+            a.out.off[out0 + o] = s_off[o + pad];
+            if constexpr (!T::has_cache)
+                a.out.cell[out0 + o] = s_cell[o + pad];
         }
     }
 }
 
-template <int KIND, int S>
-cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
+template <int KIND, int S, bool OBS>
+cudaError_t launch_split_as(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
 {
-    const size_t smem = static_cast<size_t>(tiles_per_cta) * (32 * S * site_smem_bytes(KIND, S) + queue_bytes(KIND, S));
-    auto kern = split_step_kernel<KIND, S>;
+    const size_t smem = static_cast<size_t>(tiles_per_cta) * Tile<KIND, S>::bytes;
+    auto kern = split_step_kernel<KIND, S, OBS>;
     // raise the dynamic shared-memory limit of this kernel on this device to the largest shape in
     // use; under a lock, so that two threads raising it at once cannot leave the smaller value
     static std::mutex s_mu;
@@ -630,6 +962,12 @@ cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t s
     return cudaGetLastError();
 }
 
+template <int KIND, int S>
+cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
+{
+    return a.n_obs > 0 ? launch_split_as<KIND, S, true>(tiles_per_cta, a, st) : launch_split_as<KIND, S, false>(tiles_per_cta, a, st);
+}
+
 // ---------------------------------------------------------------------------------------
 // Initialisation (flat start or a given FP64 state) and conversion back to FP64.
 // Block tiles of w_tile sites, one thread per site.
@@ -647,7 +985,7 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
         int32_t n = 0;
         float d = 0.0f;
         if (u_in) {
-            const double u = u_in[p];
+            const double u = u_in[ch.dense + i];
             const double fl = floor(u);
             n = static_cast<int32_t>(fl);
             d = static_cast<float>(u - fl);
@@ -663,7 +1001,11 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
         if (ch.kind == kRF)
             st.rf[p] = make_float2(rf_plus_f32(seed, ch.s, i, m1, ch.f32), rf_plus_f32(seed, ch.s, i, m2, ch.f32));
         else if (ch.kind == kRBGLinear)
-            st.rf[p] = make_float2(rbg_f32(seed, ch.s, i, m1), rbg_f32(seed, ch.s, i, m2));
+        {
+            const float g1 = rbg_f32(seed, ch.s, i, m1), g2 = rbg_f32(seed, ch.s, i, m2), g3 = rbg_f32(seed, ch.s, i, m3);
+            st.rf[p] = make_float2(g1 - g2, g2 - g3);
+            st.q3[p] = g3;
+        }
         else if (ch.kind == kRB || ch.kind == kRBGCubic) {
             const bool uni = ch.kind == kRB;
             const float p0 = uni ? rb_f32(seed, ch.s, i, m0) : rbg_f32(seed, ch.s, i, m0);
@@ -691,9 +1033,9 @@ __global__ void split_to_f64_kernel(const ChainDesc* chains, const TileDesc* til
             break;
         const int64_t p = ch.offset + i;
         if (u_out)
-            u_out[p] = static_cast<double>(st.cell[p]) + static_cast<double>(st.off[p]);
+            u_out[ch.dense + i] = static_cast<double>(st.cell[p]) + static_cast<double>(fabsf(st.off[p]));
         if (cells_out)
-            cells_out[p] = st.cell[p];
+            cells_out[ch.dense + i] = st.cell[p];
     }
 }
 
@@ -708,9 +1050,23 @@ bool split_supported(int kind, int S)
     return S == 7 || S == 15 || S == 23 || S == 31 || S == 39;
 }
 
+template <int KIND>
+constexpr int tile_bytes(int S)
+{
+    switch (S) {
+    case 7: return Tile<KIND, 7>::bytes;
+    case 15: return Tile<KIND, 15>::bytes;
+    case 23: return Tile<KIND, 23>::bytes;
+    case 31: return Tile<KIND, 31>::bytes;
+    default: return Tile<KIND, 39>::bytes;
+    }
+}
+
 size_t split_smem_bytes(int kind, int S, int tiles_per_cta)
 {
-    return static_cast<size_t>(tiles_per_cta) * (32 * S * site_smem_bytes(kind, S) + queue_bytes(kind, S));
+    const int b = kind == kRF ? tile_bytes<kRF>(S) : kind == kRBGLinear ? tile_bytes<kRBGLinear>(S) :
+                  kind == kNone ? tile_bytes<kNone>(S) : tile_bytes<kRB>(S);
+    return static_cast<size_t>(tiles_per_cta) * b;
 }
 
 cudaError_t split_step(int kind, int S, int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)

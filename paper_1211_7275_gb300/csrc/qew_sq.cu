@@ -21,7 +21,7 @@ __global__ void sq_rows_split_kernel(const ChainDesc* chains, int32_t n_chains, 
         for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < L;
              i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
             const int64_t p = ch.offset + i;
-            row[i] = static_cast<double>(st.cell[p] - c0) + static_cast<double>(st.off[p]);   // exact
+            row[i] = static_cast<double>(st.cell[p] - c0) + static_cast<double>(fabsf(st.off[p]));   // exact
         }
     }
 }

@@ -65,12 +65,6 @@ __device__ __forceinline__ void tma_store_commit()
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// Wait until all committed bulk stores of this thread have completed.
-__device__ __forceinline__ void tma_store_wait_all()
-{
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
 // Wait until all committed bulk stores of this thread have finished reading their shared-memory
 // sources (the global writes may still be in flight).
 __device__ __forceinline__ void tma_store_wait_read_all()
