@@ -103,7 +103,10 @@ struct qew_ctx {
 
     SplitState sp[2] = {};
     int cur = 0;
-    F64State f64 = {};
+    F64State f64[2] = {};            // disorder caches: two copies when a launch takes several steps
+    F64Shape f64s = {256, 4, 1, false};
+    TileDesc* d_ftiles = nullptr;    // tiles of the FP64 step kernel
+    int32_t n_ftiles = 0;
     double* u64[2] = {nullptr, nullptr};
 
     double* d_shift = nullptr;
@@ -202,10 +205,12 @@ void free_f64(qew_ctx* h)
 {
     dev_free(h->u64[0]);
     dev_free(h->u64[1]);
-    dev_free(h->f64.ncache);
-    for (int c = 0; c < 4; ++c)
-        dev_free(h->f64.c[c]);
-    h->f64.u = nullptr;
+    for (int b = 0; b < 2; ++b) {
+        dev_free(h->f64[b].ncache);
+        for (double*& c : h->f64[b].c)
+            dev_free(c);
+        h->f64[b].u = nullptr;
+    }
 }
 
 void free_events(qew_ctx* h)
@@ -240,6 +245,7 @@ void free_all(qew_ctx* h)
     for (int k = 0; k < kNumKinds; ++k)
         dev_free(h->d_tiles[k]);
     dev_free(h->d_btiles);
+    dev_free(h->d_ftiles);
     dev_free(h->d_shift);
     dev_free(h->d_partial);
     dev_free(h->d_obs);
@@ -277,9 +283,11 @@ int alloc_state(qew_ctx* h)
             return QEW_OK;
         QEW_CUDA(h, dev_alloc(&h->u64[0], N), "allocating the FP64 state");
         QEW_CUDA(h, dev_alloc(&h->u64[1], N), "allocating the FP64 state");
-        QEW_CUDA(h, dev_alloc(&h->f64.ncache, N), "allocating the FP64 cache cells");
-        for (int c = 0; c < h->n_cache; ++c)
-            QEW_CUDA(h, dev_alloc(&h->f64.c[c], N), "allocating the FP64 disorder cache");
+        for (int b = 0; b < (h->f64s.K > 1 ? 2 : 1); ++b) {
+            QEW_CUDA(h, dev_alloc(&h->f64[b].ncache, N), "allocating the FP64 cache cells");
+            for (int c = 0; c < h->n_cache; ++c)
+                QEW_CUDA(h, dev_alloc(&h->f64[b].c[c], N), "allocating the FP64 disorder cache");
+        }
     }
     return QEW_OK;
 }
@@ -324,7 +332,10 @@ int build_layout(qew_ctx* h)
     for (int k = 0; k < kNumKinds; ++k)
         h->w_own[k] = 32 * kind_S(k, h->S) - 2 * h->K;
     std::vector<TileDesc> lists[kNumKinds];
-    std::vector<TileDesc> blocks;
+    std::vector<TileDesc> blocks, ftiles;
+    h->f64s = f64_shape(h->n_sites);
+    h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
+                 h->f64s.look ? ((h->kinds_mask >> kRBGLinear & 1) ? 4 : 3) : 2;
     h->h_chains.assign(h->n_chains, ChainDesc{});
     std::vector<int32_t> first(h->n_chains), count(h->n_chains);
     for (int32_t c = 0; c < h->n_chains; ++c) {
@@ -345,6 +356,9 @@ int build_layout(qew_ctx* h)
             for (int64_t st = 0; st < d.L; st += h->w_own[d.kind])
                 lst.push_back(TileDesc{c, static_cast<int32_t>(st)});
             count[c] = static_cast<int32_t>(lst.size()) - first[c];
+        } else {
+            for (int64_t st = 0; st < d.L; st += h->f64s.w_own())
+                ftiles.push_back(TileDesc{c, static_cast<int32_t>(st)});
         }
     }
     size_t slots = 0;
@@ -390,6 +404,13 @@ int build_layout(qew_ctx* h)
     QEW_CUDA(h, dev_alloc(&h->d_btiles, blocks.size()), "allocating block tiles");
     QEW_CUDA(h, cudaMemcpy(h->d_btiles, blocks.data(), blocks.size() * sizeof(TileDesc), cudaMemcpyHostToDevice),
              "uploading block tiles");
+    dev_free(h->d_ftiles);
+    h->n_ftiles = static_cast<int32_t>(ftiles.size());
+    if (!ftiles.empty()) {
+        QEW_CUDA(h, dev_alloc(&h->d_ftiles, ftiles.size()), "allocating FP64 tiles");
+        QEW_CUDA(h, cudaMemcpy(h->d_ftiles, ftiles.data(), ftiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice),
+                 "uploading FP64 tiles");
+    }
     // room for the partials of as many observations as 256 MB hold
     h->partial_slots = slots;
     h->launch_obs = 1;
@@ -415,8 +436,8 @@ int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shif
         QEW_CUDA(h, split_init(h->d_chains, h->n_chains, h->d_btiles, h->n_btiles, kBlockTile, h->sp[0], h->seed,
                                h->kinds_mask & kQuadMask, d_u_in, h->stream), "launching the state initialisation");
     } else {
-        h->f64.u = h->u64[0];
-        QEW_CUDA(h, f64_init(h->d_chains, h->d_btiles, h->n_btiles, kBlockTile, h->f64, h->seed, h->kinds_mask & kQuadMask,
+        h->f64[0].u = h->u64[0];
+        QEW_CUDA(h, f64_init(h->d_chains, h->d_btiles, h->n_btiles, kBlockTile, h->f64[0], h->seed, h->f64s.look,
                              d_u_in, h->stream), "launching the FP64 state initialisation");
     }
     h->n_launches += 1;
@@ -500,6 +521,12 @@ int launch_split_all(qew_ctx* h, const Segment& s, SplitState in, SplitState out
     return QEW_OK;
 }
 
+// The disorder caches that belong to displacement buffer `b`.
+F64State& f64_cache(qew_ctx* h, int b)
+{
+    return h->f64[h->f64s.K > 1 ? b : 0];
+}
+
 F64Launch f64_args(qew_ctx* h)
 {
     F64Launch a{};
@@ -507,13 +534,29 @@ F64Launch f64_args(qew_ctx* h)
     a.n_tiles = h->n_btiles;
     a.w_tile = kBlockTile;
     a.chains = h->d_chains;
-    a.st = h->f64;
+    a.st = f64_cache(h, h->cur);
+    a.look = h->f64s.look;
     a.u_in = h->u64[h->cur];
-    a.u_out = h->u64[h->cur ^ 1];
-    a.dt = h->dt;
-    a.seed = h->seed;
     a.shift = h->d_shift;
     a.partial = h->d_partial;
+    return a;
+}
+
+F64Step f64_step_args(qew_ctx* h, int K)
+{
+    F64Step a{};
+    a.tiles = h->d_ftiles;
+    a.n_tiles = h->n_ftiles;
+    a.w_own = h->f64s.w_own();
+    a.K = K;
+    a.n_nodes = h->n_cache;
+    a.chains = h->d_chains;
+    a.u_in = h->u64[h->cur];
+    a.u_out = h->u64[h->cur ^ 1];
+    a.in = f64_cache(h, h->cur);
+    a.out = f64_cache(h, h->cur ^ 1);
+    a.dt = h->dt;
+    a.seed = h->seed;
     return a;
 }
 
@@ -573,12 +616,12 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
     if (h->precision != QEW_FP32_SPLIT) {
         for (int32_t k = 0; k < n_targets; ++k) {
             while (h->step < targets[k]) {
-                QEW_CUDA(h, f64_step(f64_args(h), h->stream), "launching the FP64 step kernel");
+                const int K = static_cast<int>(std::min<int64_t>(h->f64s.K, targets[k] - h->step));
+                QEW_CUDA(h, f64_step(f64_step_args(h, K), h->f64s, h->stream), "launching the FP64 step kernel");
                 h->cur ^= 1;
-                h->f64.u = h->u64[h->cur];
-                ++h->step;
+                h->step += K;
                 h->n_launches += 1;
-                h->n_site_updates += h->n_sites;
+                h->n_site_updates += h->n_sites * K;
             }
             if (d_obs) {
                 ObsList list{};
@@ -804,7 +847,6 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
             h->sites_of_kind[kind[c]] += L[c];
         }
         h->n_sites = off;
-        h->n_cache = (h->kinds_mask & kQuadMask) ? 4 : 2;
         h->dt = dt;
         h->seed = seed;
         h->precision = precision;
@@ -908,7 +950,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
     int64_t n_launch = 0, at = h->step;
     for (int32_t k = 0; k < n_times; ++k) {
         const int64_t seg = steps[k] - at;
-        n_launch += (h->precision == QEW_FP32_SPLIT) ? (seg + h->K - 1) / h->K + 2 : seg + 2;
+        n_launch += (h->precision == QEW_FP32_SPLIT) ? (seg + h->K - 1) / h->K + 2 : (seg + h->f64s.K - 1) / h->f64s.K + 2;
         at = steps[k];
     }
     const int shape[4] = {h->S, h->K, h->tpc, h->precision};
@@ -922,7 +964,6 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
         QEW_CUDA(h, cudaGraphLaunch(h->gexec, h->stream), "replaying the observation graph");
         h->step = h->g_step1;
         h->cur = h->g_cur1;
-        h->f64.u = h->u64[h->cur];
         h->n_launches += h->g_launches;
         h->n_fused += h->g_fused;
         h->n_site_updates += h->g_su;
@@ -951,8 +992,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
                     cudaGraphDestroy(graph);
                 h->step = step0;   // nothing ran: undo the host-side bookkeeping
                 h->cur = cur0;
-                h->f64.u = h->u64[h->cur];
-                if (rc != QEW_OK)
+                        if (rc != QEW_OK)
                     return rc;
                 return cuda_fail(h, ce != cudaSuccess ? ce : ee, "capturing the observation graph");
             }
@@ -962,8 +1002,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
                 h->gexec = nullptr;
                 h->step = step0;
                 h->cur = cur0;
-                h->f64.u = h->u64[h->cur];
-                return cuda_fail(h, ce, "instantiating the observation graph");
+                        return cuda_fail(h, ce, "instantiating the observation graph");
             }
             h->g_steps.assign(steps, steps + n_times);
             h->g_step0 = step0;

@@ -1,6 +1,6 @@
-// qew_fp64.cu -- the plain FP64 path of the qEW relaxation: one Euler step per launch, one
-// thread per site, FP64 state in HBM (ping-pong), and each site's disorder values cached in
-// HBM for the cell they were drawn for (regenerated when the site changes cell).
+// qew_fp64.cu -- the plain FP64 path of the qEW relaxation: FP64 state in HBM (ping-pong), one thread
+// per site and Euler step, and each site's disorder values cached for the cell they were drawn for
+// (regenerated when the site changes cell).
 //
 // Method: Eq. 1 of arXiv:1211.7275 with eta = c = 1, periodic in x, explicit Euler with all
 // forces from the old state (Sec. III.B); pinning force by linear interpolation of R (RF), as
@@ -29,107 +29,235 @@ __device__ __forceinline__ double node_f64(uint64_t seed, uint32_t s, int32_t i,
         return rbg_f64(seed, s, i, n);
 }
 
+// ---- the step kernel ----
+// A block advances a tile of w_own sites by K steps on the window of w_own + 2 (K - 1) sites whose
+// values the last owned one depends on (plus one neighbour on each side): one site per thread and
+// round, displacements in shared memory (double-buffered), what the update reads in registers.
+//
+// What bounds it: the FP64 unit takes one warp instruction in 16 clocks per SM, and the next
+// instruction of the same warp waits 65.  A step itself is 11 FP64 operations (RF); a disorder value
+// (log, sqrt, cospi) is some 80.  So
+//   - a cell is left when u - floor is outside [0, 1), an integer test of its high word: no floor and
+//     no conversion for the sites that stay;
+//   - the sites of the block that did change cell are queued and their values drawn by as few warps as
+//     hold them.  Drawn where they occur, a warp with one crossing among its 32 sites spent the time
+//     of 32 (16 x 2^20 RF sites over the first 64 steps: 2.03 ms per step then, 0.65 now);
+//   - a small batch is spread over many SMs in small tiles and advanced K steps per launch.
+// Loop values of a site: RF R(n), R(n+1); linear spline F; cubic ca, 2 b, 3 c of the force.
+// Cached nodes of a site in cell n: V(n + lo) .. V(n + lo + n_nodes - 1), the force's.  With look-ahead
+// there are n_look of them, from V(n + lo_look): the one a move up will need, and for the linear spline,
+// whose sites move up and down across a node, also the one a move down will; the force's start at
+// `used`.
 template <int KIND>
-__device__ __forceinline__ double pinning_f64(double u, int64_t p, int32_t i, uint32_t s, uint64_t seed,
-                                              const F64State& st, int32_t period)
+struct F64Site {
+    static constexpr int n_nodes = pair_kind(KIND) ? 2 : quad_kind(KIND) ? 4 : 0;
+    static constexpr int lo = quad_kind(KIND) ? -1 : 0;
+    static constexpr int n_look = KIND == kRBGLinear ? 4 : n_nodes > 0 ? n_nodes + 1 : 0;
+    static constexpr int lo_look = KIND == kRBGLinear ? -1 : lo;
+    static constexpr int used = lo - lo_look;
+    static constexpr int n_loop = KIND == kRF ? 2 : KIND == kRBGLinear ? 1 : quad_kind(KIND) ? 3 : 0;
+};
+// A node that has not been drawn.
+constexpr int kNoNode = 0x7FF80000;   // high word (a quiet NaN)
+__device__ __forceinline__ bool no_node(double v) { return __double2hiint(v) == kNoNode; }
+
+// The loop values of a cell from its nodes, in the rounding sequence of the force's definition.
+template <int KIND>
+__device__ __forceinline__ void loop_values(const double* p, double* v)
 {
-    if constexpr (KIND == kNone) {
+    if constexpr (KIND == kRF) {
+        v[0] = p[0];
+        v[1] = p[1];
+    } else if constexpr (KIND == kRBGLinear) {
+        v[0] = __dsub_rn(p[0], p[1]);   // minus the slope of the linear spline through G
+    } else if constexpr (quad_kind(KIND)) {
+        // -1/2 [(p2 - p0) + 2 b d + 3 c d^2], b = 2p0 - 5p1 + 4p2 - p3, c = -p0 + 3p1 - 3p2 + p3
+        v[0] = __dsub_rn(p[2], p[0]);
+        v[1] = __dmul_rn(2.0, __dsub_rn(__dadd_rn(__dsub_rn(__dmul_rn(2.0, p[0]), __dmul_rn(5.0, p[1])), __dmul_rn(4.0, p[2])), p[3]));
+        v[2] = __dmul_rn(3.0, __dadd_rn(__dsub_rn(__dsub_rn(__dmul_rn(3.0, p[1]), p[0]), __dmul_rn(3.0, p[2])), p[3]));
+    }
+}
+
+template <int KIND>
+__device__ __forceinline__ double force_f64(double d, const double* v)
+{
+    if constexpr (KIND == kRF)
+        return __dadd_rn(__dmul_rn(__dsub_rn(1.0, d), v[0]), __dmul_rn(d, v[1]));
+    else if constexpr (KIND == kRBGLinear)
+        return v[0];
+    else if constexpr (quad_kind(KIND))
+        return __dmul_rn(-0.5, __dadd_rn(__dadd_rn(v[0], __dmul_rn(v[1], d)), __dmul_rn(__dmul_rn(v[2], d), d)));
+    else
         return 0.0;
-    } else {
-        const double fl = floor(u);
-        const int32_t n = static_cast<int32_t>(fl);
-        const double d = __dsub_rn(u, fl);
-        const int32_t nc = st.ncache[p];
-        if constexpr (pair_kind(KIND)) {
-            double r0, r1;
-            if (n == nc) {
-                r0 = st.c[0][p];
-                r1 = st.c[1][p];
-            } else {
-                if (n == nc + 1) {
-                    r0 = st.c[1][p];
-                    r1 = node_f64<KIND>(seed, s, i, n + 1, period);
-                } else if (n == nc - 1) {
-                    r1 = st.c[0][p];
-                    r0 = node_f64<KIND>(seed, s, i, n, period);
-                } else {
-                    r0 = node_f64<KIND>(seed, s, i, n, period);
-                    r1 = node_f64<KIND>(seed, s, i, n + 1, period);
+}
+
+template <int KIND, int SPT>
+__device__ __forceinline__ void f64_step_body(const F64Step& a, const TileDesc td, const ChainDesc& ch, double* smem)
+{
+    using V = F64Site<KIND>;
+    constexpr int NN = V::n_nodes, NL = V::n_loop;
+    const int NT = blockDim.x;
+    const int tid = threadIdx.x;
+    const int W = NT * SPT;          // room for active sites
+    const int32_t L = ch.L;
+    const int K = a.K;
+    const int owned = min(a.w_own, L - td.start);
+    const int active = owned + 2 * (K - 1);
+    const int64_t first = static_cast<int64_t>(td.start) - (K - 1);   // site of window position 0
+
+    double* s_u = smem;                                     // [2][W + 2]: positions -1 .. W
+    double* s_p = s_u + 2 * (W + 2);                        // nodes [NN][W]
+    int32_t* s_cell = reinterpret_cast<int32_t*>(s_p + static_cast<size_t>(a.n_nodes) * W);   // cell of the nodes
+    uint16_t* s_q = reinterpret_cast<uint16_t*>(s_cell + W);
+    __shared__ int s_count[3];
+    if (tid < 3)
+        s_count[tid] = 0;
+
+    auto site_of = [&](int x) -> int32_t {
+        const int64_t g = first + x;
+        return (g >= 0 && g < L) ? static_cast<int32_t>(g) : wrap_site(g, L);
+    };
+
+    double u[SPT], cell[SPT], v[SPT][NL > 0 ? NL : 1];
+    int32_t n0[SPT];
+#pragma unroll
+    for (int r = 0; r < SPT; ++r) {
+        const int x = tid + r * NT;
+        if (x < active) {
+            const int64_t p = ch.offset + site_of(x);
+            u[r] = a.u_in[p];
+            if constexpr (NN > 0) {
+                n0[r] = a.in.ncache[p];
+                cell[r] = static_cast<double>(n0[r]);
+                s_cell[x] = n0[r];
+                double nodes[NN];
+#pragma unroll
+                for (int c = 0; c < NN; ++c) {
+                    nodes[c] = a.in.c[c][p];
+                    s_p[c * W + x] = nodes[c];
                 }
-                st.ncache[p] = n;
-                st.c[0][p] = r0;
-                st.c[1][p] = r1;
+                loop_values<KIND>(nodes, v[r]);
             }
-            if constexpr (KIND == kRF)
-                return __dadd_rn(__dmul_rn(__dsub_rn(1.0, d), r0), __dmul_rn(d, r1));
-            else
-                return __dsub_rn(r0, r1);   // minus the slope of the linear spline through G
-        } else {
-            double p0, p1, p2, p3;
-            if (n == nc) {
-                p0 = st.c[0][p];
-                p1 = st.c[1][p];
-                p2 = st.c[2][p];
-                p3 = st.c[3][p];
-            } else {
-                if (n == nc + 1) {
-                    p0 = st.c[1][p];
-                    p1 = st.c[2][p];
-                    p2 = st.c[3][p];
-                    p3 = node_f64<KIND>(seed, s, i, n + 2, period);
-                } else if (n == nc - 1) {
-                    p1 = st.c[0][p];
-                    p2 = st.c[1][p];
-                    p3 = st.c[2][p];
-                    p0 = node_f64<KIND>(seed, s, i, n - 1, period);
-                } else {
-                    p0 = node_f64<KIND>(seed, s, i, n - 1, period);
-                    p1 = node_f64<KIND>(seed, s, i, n, period);
-                    p2 = node_f64<KIND>(seed, s, i, n + 1, period);
-                    p3 = node_f64<KIND>(seed, s, i, n + 2, period);
+        }
+    }
+    if (tid < 2) {   // the window's outer neighbours, as they are at the start
+        const int x = tid == 0 ? -1 : active;
+        const double un = a.u_in[ch.offset + site_of(x)];
+        s_u[x + 1] = un;
+        s_u[(W + 2) + x + 1] = un;
+    }
+    __syncthreads();   // (the request counters)
+
+    for (int k = 0;; ++k) {
+        double* now = s_u + (k & 1) * (W + 2) + 1;
+        double d[SPT];
+        bool moved[SPT];
+#pragma unroll
+        for (int r = 0; r < SPT; ++r) {
+            const int x = tid + r * NT;
+            moved[r] = false;
+            if (x < active) {
+                now[x] = u[r];
+                if constexpr (NN > 0) {
+                    d[r] = __dsub_rn(u[r], cell[r]);
+                    moved[r] = static_cast<unsigned>(__double2hiint(d[r])) >= 0x3FF00000u;   // not in [0, 1)
+                    if (moved[r])
+                        s_q[atomicAdd(&s_count[k % 3], 1)] = static_cast<uint16_t>(x);
                 }
-                st.ncache[p] = n;
-                st.c[0][p] = p0;
-                st.c[1][p] = p1;
-                st.c[2][p] = p2;
-                st.c[3][p] = p3;
             }
-            // -1/2 [(p2 - p0) + 2 b d + 3 c d^2], b = 2p0 - 5p1 + 4p2 - p3, c = -p0 + 3p1 - 3p2 + p3
-            const double ca = __dsub_rn(p2, p0);
-            const double cb = __dsub_rn(__dadd_rn(__dsub_rn(__dmul_rn(2.0, p0), __dmul_rn(5.0, p1)), __dmul_rn(4.0, p2)), p3);
-            const double cc = __dadd_rn(__dsub_rn(__dsub_rn(__dmul_rn(3.0, p1), p0), __dmul_rn(3.0, p2)), p3);
-            const double t1 = __dmul_rn(__dmul_rn(2.0, cb), d);
-            const double t2 = __dmul_rn(__dmul_rn(__dmul_rn(3.0, cc), d), d);
-            return __dmul_rn(-0.5, __dadd_rn(__dadd_rn(ca, t1), t2));
+        }
+        __syncthreads();
+        if constexpr (NN > 0) {
+            const int nq = s_count[k % 3];
+            if (tid == 0)
+                s_count[(k + 2) % 3] = 0;   // last read in step k - 1, next used in step k + 2
+            if (nq > 0) {
+                for (int q = tid; q < nq; q += NT) {
+                    const int x = s_q[q];
+                    const int32_t n = __double2int_rd(now[x]);
+                    const int32_t move = n - s_cell[x];
+                    if (move != 0) {   // 0: u - floor rounded up to 1
+                        double p[NN];
+                        const int shift = (move == 1 || move == -1) ? move : NN;
+                        if (shift == 1) {
+#pragma unroll
+                            for (int c = 0; c + 1 < NN; ++c)
+                                p[c] = s_p[(c + 1) * W + x];
+                        } else if (shift == -1) {
+#pragma unroll
+                            for (int c = 1; c < NN; ++c)
+                                p[c] = s_p[(c - 1) * W + x];
+                        }
+                        const int32_t i = site_of(x);
+                        const int trips = (shift == NN) ? NN : 1;
+#pragma unroll 1
+                        for (int j = 0; j < trips; ++j) {
+                            const int c = (shift == 1) ? NN - 1 : j;
+                            const double w = node_f64<KIND>(a.seed, ch.s, i, n + V::lo + c, ch.period);
+#pragma unroll
+                            for (int cc = 0; cc < NN; ++cc)
+                                if (cc == c)
+                                    p[cc] = w;
+                        }
+#pragma unroll
+                        for (int c = 0; c < NN; ++c)
+                            s_p[c * W + x] = p[c];
+                        s_cell[x] = n;
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < SPT; ++r) {
+                    if (moved[r]) {
+                        const int x = tid + r * NT;
+                        double p[NN];
+#pragma unroll
+                        for (int c = 0; c < NN; ++c)
+                            p[c] = s_p[c * W + x];
+                        loop_values<KIND>(p, v[r]);
+                        cell[r] = static_cast<double>(s_cell[x]);
+                        d[r] = __dsub_rn(u[r], cell[r]);
+                    }
+                }
+            }
+        }
+        if (k == K)
+            break;
+#pragma unroll
+        for (int r = 0; r < SPT; ++r) {
+            const int x = tid + r * NT;
+            if (x < active) {
+                const double lap = __fma_rn(-2.0, u[r], __dadd_rn(now[x + 1], now[x - 1]));   // 2 u is exact
+                u[r] = __dadd_rn(u[r], __dmul_rn(a.dt, __dadd_rn(__dadd_rn(lap, ch.f64), force_f64<KIND>(d[r], v[r]))));
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < SPT; ++r) {
+        const int x = tid + r * NT;
+        const int o = x - (K - 1);
+        if (x < active && o >= 0 && o < owned) {
+            const int64_t p = ch.offset + td.start + o;
+            a.u_out[p] = u[r];
+            if constexpr (NN > 0) {
+                const int32_t n = s_cell[x];
+                if (a.out.ncache != a.in.ncache || n != n0[r]) {
+                    a.out.ncache[p] = n;
+#pragma unroll
+                    for (int c = 0; c < NN; ++c)
+                        a.out.c[c][p] = s_p[c * W + x];
+                }
+            }
         }
     }
 }
 
-template <int KIND>
-__device__ __forceinline__ void f64_step_body(const F64Launch& a)
-{
-    const TileDesc td = a.tiles[blockIdx.x];
-    const ChainDesc ch = a.chains[td.chain];
-    const int32_t L = ch.L;
-    for (int x = threadIdx.x; x < a.w_tile; x += blockDim.x) {
-        const int32_t i = td.start + x;
-        if (i >= L)
-            break;
-        const int64_t p = ch.offset + i;
-        const double u = a.u_in[p];
-        const double ul = a.u_in[ch.offset + (i == 0 ? L - 1 : i - 1)];
-        const double ur = a.u_in[ch.offset + (i + 1 == L ? 0 : i + 1)];
-        const double F = pinning_f64<KIND>(u, p, i, ch.s, a.seed, a.st, ch.period);
-        const double lap = __dsub_rn(__dadd_rn(ur, ul), __dmul_rn(2.0, u));
-        a.u_out[p] = __dadd_rn(u, __dmul_rn(a.dt, __dadd_rn(__dadd_rn(lap, ch.f64), F)));
-    }
-}
-
 // Per block tile: sum F, sum (u - c), sum (u - c)^2 of the current state u_in, c the chain's
-// reference shift.
+// reference shift.  (The cached cell is floor(u) between launches.)
 template <int KIND>
 __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*red)[256 / 32])
 {
+    using V = F64Site<KIND>;
     const TileDesc td = a.tiles[blockIdx.x];
     const ChainDesc ch = a.chains[td.chain];
     const double c = a.shift[td.chain];
@@ -140,7 +268,14 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
             break;
         const int64_t p = ch.offset + i;
         const double u = a.u_in[p];
-        tF = __dadd_rn(tF, pinning_f64<KIND>(u, p, i, ch.s, a.seed, a.st, ch.period));
+        if constexpr (V::n_nodes > 0) {
+            double nodes[V::n_nodes], v[V::n_loop];
+#pragma unroll
+            for (int k = 0; k < V::n_nodes; ++k)
+                nodes[k] = a.st.c[a.look ? V::used + k : k][p];
+            loop_values<KIND>(nodes, v);
+            tF = __dadd_rn(tF, force_f64<KIND>(__dsub_rn(u, static_cast<double>(a.st.ncache[p])), v));
+        }
         const double y = __dsub_rn(u, c);
         t1 = __dadd_rn(t1, y);
         t2 = __dadd_rn(t2, __dmul_rn(y, y));
@@ -173,8 +308,20 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
     }
 }
 
+template <int KIND>
+__device__ __forceinline__ void init_nodes(const F64State& st, int64_t p, uint64_t seed, uint32_t s, int32_t i, int32_t n,
+                                           int32_t period, int look)
+{
+    using V = F64Site<KIND>;
+    const int count = look ? V::n_look : V::n_nodes;
+    const int lo = look ? V::lo_look : V::lo;
+#pragma unroll 1
+    for (int c = 0; c < count; ++c)
+        st.c[c][p] = node_f64<KIND>(seed, s, i, n + lo + c, period);
+}
+
 __global__ void f64_init_kernel(const ChainDesc* chains, const TileDesc* tiles, int32_t w_tile, F64State st,
-                                uint64_t seed, const double* u_in)
+                                uint64_t seed, const double* u_in, int look)
 {
     const TileDesc td = tiles[blockIdx.x];
     const ChainDesc ch = chains[td.chain];
@@ -188,19 +335,14 @@ __global__ void f64_init_kernel(const ChainDesc* chains, const TileDesc* tiles, 
         const int32_t n = static_cast<int32_t>(floor(u));
         st.ncache[p] = n;
         const int32_t M = ch.period;
-        if (ch.kind == kRF) {
-            st.c[0][p] = rf_f64(seed, ch.s, i, wrap_node(n, M));
-            st.c[1][p] = rf_f64(seed, ch.s, i, wrap_node(n + 1, M));
-        } else if (ch.kind == kRBGLinear) {
-            st.c[0][p] = rbg_f64(seed, ch.s, i, wrap_node(n, M));
-            st.c[1][p] = rbg_f64(seed, ch.s, i, wrap_node(n + 1, M));
-        } else if (ch.kind == kRB) {
-            for (int c = 0; c < 4; ++c)
-                st.c[c][p] = rb_f64(seed, ch.s, i, wrap_node(n - 1 + c, M));
-        } else if (ch.kind == kRBGCubic) {
-            for (int c = 0; c < 4; ++c)
-                st.c[c][p] = rbg_f64(seed, ch.s, i, wrap_node(n - 1 + c, M));
-        }
+        if (ch.kind == kRF)
+            init_nodes<kRF>(st, p, seed, ch.s, i, n, M, look);
+        else if (ch.kind == kRBGLinear)
+            init_nodes<kRBGLinear>(st, p, seed, ch.s, i, n, M, look);
+        else if (ch.kind == kRB)
+            init_nodes<kRB>(st, p, seed, ch.s, i, n, M, look);
+        else if (ch.kind == kRBGCubic)
+            init_nodes<kRBGCubic>(st, p, seed, ch.s, i, n, M, look);
     }
 }
 
@@ -218,20 +360,200 @@ __global__ void f64_cells_kernel(const ChainDesc* chains, const TileDesc* tiles,
     }
 }
 
-// Block tiles of mixed kinds share one launch: the kind is uniform per block (one chain).
-__global__ void __launch_bounds__(256) f64_step_any(F64Launch a)
+// The same for few sites (one per thread), where a draw is 5500 clocks of waiting and a step 900: each
+// site holds the next node it will need, so a move up only shifts its nodes and lists the site; the
+// listed sites' missing nodes are drawn together once a warp of them has gathered, or at once when a
+// force needs one.  One 1024-site RF chain at f = 1, us per step: 22.7 with one launch per step on one
+// SM, 3.3 in small tiles with every draw in its own step, 1.47 so.
+template <int KIND>
+__device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc td, const ChainDesc& ch, double* smem)
 {
-    const int kind = a.chains[a.tiles[blockIdx.x].chain].kind;
-    if (kind == kRF)
-        f64_step_body<kRF>(a);
-    else if (kind == kRB)
-        f64_step_body<kRB>(a);
-    else if (kind == kRBGLinear)
-        f64_step_body<kRBGLinear>(a);
-    else if (kind == kRBGCubic)
-        f64_step_body<kRBGCubic>(a);
+    using V = F64Site<KIND>;
+    constexpr int NN = V::n_nodes, NX = V::n_look, NL = V::n_loop;
+    const int NT = blockDim.x;
+    const int gather = max(32, NT / 4);
+    const int x = threadIdx.x;
+    const int32_t L = ch.L;
+    const int K = a.K;
+    const int owned = min(a.w_own, L - td.start);
+    const int active = owned + 2 * (K - 1);
+    const int64_t first = static_cast<int64_t>(td.start) - (K - 1);   // site of window position 0
+
+    double* s_u = smem;                                     // [2][NT + 2]: positions -1 .. NT
+    double* s_p = s_u + 2 * (NT + 2);                       // nodes [NX][NT]
+    int32_t* s_cell = reinterpret_cast<int32_t*>(s_p + static_cast<size_t>(a.n_nodes) * NT);
+    uint16_t* s_q = reinterpret_cast<uint16_t*>(s_cell + NT);
+    __shared__ int s_count[2];   // listed sites; the two take turns
+    if (x < 2)
+        s_count[x] = 0;
+
+    auto site_of = [&](int at) -> int32_t {
+        const int64_t g = first + at;
+        return (g >= 0 && g < L) ? static_cast<int32_t>(g) : wrap_site(g, L);
+    };
+    const bool mine = x < active;
+    double u = 0.0, cell = 0.0, d = 0.0, v[NL > 0 ? NL : 1];
+    int32_t n = 0;
+    bool missing = false;
+    if (mine) {
+        const int64_t p = ch.offset + site_of(x);
+        u = a.u_in[p];
+        if constexpr (NX > 0) {
+            n = a.in.ncache[p];
+            cell = static_cast<double>(n);
+            s_cell[x] = n;
+            double nodes[NX];
+#pragma unroll
+            for (int c = 0; c < NX; ++c) {
+                nodes[c] = a.in.c[c][p];
+                s_p[c * NT + x] = nodes[c];
+                missing = missing || no_node(nodes[c]);
+            }
+            loop_values<KIND>(nodes + V::used, v);
+        }
+    }
+    if (x < 2) {   // the window's outer neighbours, as they are at the start
+        const int at = x == 0 ? -1 : active;
+        const double un = a.u_in[ch.offset + site_of(at)];
+        s_u[at + 1] = un;
+        s_u[(NT + 2) + at + 1] = un;
+    }
+    __syncthreads();
+    int turn = 0, slot = -1;
+    if (missing) {
+        slot = atomicAdd(&s_count[0], 1);
+        s_q[slot] = static_cast<uint16_t>(x);
+    }
+
+    for (int k = 0;; ++k) {
+        double* now = s_u + (k & 1) * (NT + 2) + 1;
+        if constexpr (NX > 0) {
+            bool urgent = false;
+            if (mine) {
+                now[x] = u;
+                d = __dsub_rn(u, cell);
+                const unsigned h = static_cast<unsigned>(__double2hiint(d));
+                if (h >= 0x3FF00000u) {   // not in [0, 1)
+                    // (1, 2) is one cell up and (-1, 0) one down, exactly; else the floor decides (u - floor
+                    // may have rounded up to 1)
+                    int32_t move;
+                    if (h < 0x40000000u && !(h == 0x3FF00000u && __double2loint(d) == 0))
+                        move = 1;
+                    else if (h >= 0x80000000u && h < 0xBFF00000u)
+                        move = -1;
+                    else
+                        move = __double2int_rd(u) - n;
+                    if (move != 0) {
+                        n += move;
+                        cell = static_cast<double>(n);
+                        d = __dsub_rn(u, cell);
+                        const double none = __hiloint2double(kNoNode, 0);
+                        double nodes[NX];
+#pragma unroll
+                        for (int c = 0; c < NX; ++c) {
+                            nodes[c] = none;
+                            if (move == 1 && c + 1 < NX)
+                                nodes[c] = s_p[(c + 1) * NT + x];
+                            if (move == -1 && c > 0)
+                                nodes[c] = s_p[(c - 1) * NT + x];
+                        }
+#pragma unroll
+                        for (int c = 0; c < NX; ++c) {
+                            s_p[c * NT + x] = nodes[c];
+                            if (c >= V::used && c < V::used + NN)
+                                urgent = urgent || no_node(nodes[c]);
+                        }
+                        s_cell[x] = n;
+                        loop_values<KIND>(nodes + V::used, v);
+                        if (slot < 0) {
+                            slot = atomicAdd(&s_count[turn], 1);
+                            s_q[slot] = static_cast<uint16_t>(x);
+                        }
+                    }
+                }
+            }
+            if (__syncthreads_or(urgent || slot >= gather - 1)) {
+                const int listed = s_count[turn];
+                for (int q = x; q < listed; q += NT) {
+                    const int at = s_q[q];
+                    const int32_t i = site_of(at), base = s_cell[at] + V::lo_look;
+#pragma unroll 1
+                    for (int c = 0; c < NX; ++c)
+                        if (no_node(s_p[c * NT + at]))
+                            s_p[c * NT + at] = node_f64<KIND>(a.seed, ch.s, i, base + c, ch.period);
+                }
+                turn ^= 1;
+                slot = -1;
+                if (x == 0)
+                    s_count[turn] = 0;   // last read a gathering ago
+                __syncthreads();
+                if (urgent) {
+                    double nodes[NN];
+#pragma unroll
+                    for (int c = 0; c < NN; ++c)
+                        nodes[c] = s_p[(V::used + c) * NT + x];
+                    loop_values<KIND>(nodes, v);
+                }
+            }
+        } else {
+            if (mine)
+                now[x] = u;
+            __syncthreads();
+        }
+        if (k == K)
+            break;
+        if (mine) {
+            const double lap = __fma_rn(-2.0, u, __dadd_rn(now[x + 1], now[x - 1]));   // 2 u is exact
+            u = __dadd_rn(u, __dmul_rn(a.dt, __dadd_rn(__dadd_rn(lap, ch.f64), force_f64<KIND>(d, v))));
+        }
+    }
+    const int o = x - (K - 1);
+    if (mine && o >= 0 && o < owned) {
+        const int64_t p = ch.offset + td.start + o;
+        a.u_out[p] = u;
+        if constexpr (NX > 0) {
+            a.out.ncache[p] = n;
+#pragma unroll
+            for (int c = 0; c < NX; ++c)
+                a.out.c[c][p] = s_p[c * NT + x];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256, 1) f64_look_any(F64Step a)
+{
+    extern __shared__ double smem_f64[];
+    const TileDesc td = a.tiles[blockIdx.x];
+    const ChainDesc ch = a.chains[td.chain];
+    if (ch.kind == kRF)
+        f64_look_body<kRF>(a, td, ch, smem_f64);
+    else if (ch.kind == kRB)
+        f64_look_body<kRB>(a, td, ch, smem_f64);
+    else if (ch.kind == kRBGLinear)
+        f64_look_body<kRBGLinear>(a, td, ch, smem_f64);
+    else if (ch.kind == kRBGCubic)
+        f64_look_body<kRBGCubic>(a, td, ch, smem_f64);
     else
-        f64_step_body<kNone>(a);
+        f64_look_body<kNone>(a, td, ch, smem_f64);
+}
+
+// Tiles of mixed kinds share one launch: the kind is uniform per block (one chain).
+template <int SPT>
+__global__ void __launch_bounds__(256, 1) f64_step_any(F64Step a)
+{
+    extern __shared__ double smem_f64[];
+    const TileDesc td = a.tiles[blockIdx.x];
+    const ChainDesc ch = a.chains[td.chain];
+    if (ch.kind == kRF)
+        f64_step_body<kRF, SPT>(a, td, ch, smem_f64);
+    else if (ch.kind == kRB)
+        f64_step_body<kRB, SPT>(a, td, ch, smem_f64);
+    else if (ch.kind == kRBGLinear)
+        f64_step_body<kRBGLinear, SPT>(a, td, ch, smem_f64);
+    else if (ch.kind == kRBGCubic)
+        f64_step_body<kRBGCubic, SPT>(a, td, ch, smem_f64);
+    else
+        f64_step_body<kNone, SPT>(a, td, ch, smem_f64);
 }
 
 __global__ void __launch_bounds__(256) f64_observe_any(F64Launch a)
@@ -252,11 +574,54 @@ __global__ void __launch_bounds__(256) f64_observe_any(F64Launch a)
 
 }  // namespace
 
-cudaError_t f64_step(const F64Launch& a, cudaStream_t st)
+size_t f64_step_smem(const F64Shape& s, int n_nodes)
+{
+    const size_t W = static_cast<size_t>(s.threads) * s.sites_per_thread;
+    return 8 * (2 * (W + 2) + n_nodes * W) + 4 * W + 2 * W;
+}
+
+// Shape by the number of sites, each line where the next shape measured faster (RF, us per step):
+//   1024 sites    128 threads x 32 steps with look-ahead 1.47, x 16 steps 1.60, without look-ahead 4.9
+//   2^16 sites    256 x 16 with look-ahead 3.0, 128 x 16 3.6, 128 x 32 5.3, without 5.1
+//   2^19 sites    256 x 16 with look-ahead 21.0, without 25.7
+//   2^24 sites    128 threads of 4 sites x 8 steps without look-ahead 651 (Case 3 on half of them 367, against
+//                 550 with look-ahead, whose outer nodes its moves up and down keep discarding), 4 steps 669
+// Few sites are latency: 65 clocks per FP64 operation whatever a block does, so small tiles on as many
+// SMs as there are.  Then it is FP64 throughput, where a wide halo is work done twice.  Beyond 2^26
+// sites one step per launch updates the cached disorder in place, which takes no second copy of it.
+F64Shape f64_shape(int64_t n_sites)
+{
+    if (n_sites <= (int64_t(1) << 13))
+        return F64Shape{128, 1, 32, true};
+    if (n_sites <= (int64_t(1) << 15))
+        return F64Shape{128, 1, 16, true};
+    if (n_sites <= (int64_t(1) << 20))
+        return F64Shape{256, 1, 16, true};
+    if (n_sites <= (int64_t(1) << 26))
+        return F64Shape{128, 4, 8, false};
+    return F64Shape{256, 4, 1, false};
+}
+
+template <int SPT>
+static cudaError_t f64_step_as(const F64Step& a, const F64Shape& s, cudaStream_t st)
+{
+    const size_t smem = f64_step_smem(s, a.n_nodes);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(f64_step_any<SPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+        if (e != cudaSuccess)
+            return e;
+    }
+    f64_step_any<SPT><<<a.n_tiles, s.threads, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t f64_step(const F64Step& a, const F64Shape& s, cudaStream_t st)
 {
     if (a.n_tiles == 0)
         return cudaSuccess;
-    f64_step_any<<<a.n_tiles, 256, 0, st>>>(a);
+    if (!s.look)
+        return f64_step_as<4>(a, s, st);
+    f64_look_any<<<a.n_tiles, s.threads, f64_step_smem(s, a.n_nodes), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -269,11 +634,11 @@ cudaError_t f64_observe(const F64Launch& a, cudaStream_t st)
 }
 
 cudaError_t f64_init(const ChainDesc* chains, const TileDesc* tiles, int32_t n_tiles, int32_t w_tile, F64State st,
-                     uint64_t seed, int, const double* u_in, cudaStream_t stream)
+                     uint64_t seed, int look, const double* u_in, cudaStream_t stream)
 {
     if (n_tiles == 0)
         return cudaSuccess;
-    f64_init_kernel<<<n_tiles, 256, 0, stream>>>(chains, tiles, w_tile, st, seed, u_in);
+    f64_init_kernel<<<n_tiles, 256, 0, stream>>>(chains, tiles, w_tile, st, seed, u_in, look);
     return cudaGetLastError();
 }
 

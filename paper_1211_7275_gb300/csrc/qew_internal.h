@@ -27,11 +27,12 @@ struct SplitState {
 };
 
 // FP64 state: displacement u, and the disorder cache of the cell `ncache` it was drawn for:
-// RF R(n), R(n+1) in c[0], c[1]; RB V(n-1..n+2) in c[0..3].
+// RF R(n), R(n+1) in c[0], c[1]; RB V(n-1..n+2) in c[0..3]; with look-ahead (few sites) one node more,
+// and for the linear-spline random bond one less as well, not drawn yet where it is a NaN.  Between launches ncache is floor(u).
 struct F64State {
     double* u;
     int32_t* ncache;
-    double* c[4];
+    double* c[5];
 };
 
 // Most observations that one launch of the fused kernel records.
@@ -73,24 +74,46 @@ cudaError_t split_to_f64(const ChainDesc* chains, const TileDesc* tiles, int32_t
 cudaError_t split_range_guard(const ChainDesc* chains, int32_t n_chains, int64_t max_L, const int32_t* cell,
                               int32_t* error, cudaStream_t stream);
 
-struct F64Launch {
+struct F64Launch {           // an observation
     const TileDesc* tiles;   // block tiles of w_tile sites
     int32_t n_tiles;
     int32_t w_tile;
     const ChainDesc* chains;
-    F64State st;             // cache is updated in place
+    F64State st;
+    int32_t look;            // the caches hold look-ahead nodes
     const double* u_in;
-    double* u_out;
-    double dt;
-    uint64_t seed;
     const double* shift;
     double* partial;
 };
 
-cudaError_t f64_step(const F64Launch& a, cudaStream_t st);
+// Launch shape of the FP64 step kernel: a block of `threads` threads with `sites_per_thread` sites each
+// advances up to K steps.
+struct F64Shape {
+    int threads, sites_per_thread, K;
+    bool look;   // sites hold the nodes their next move will need (one site per thread)
+    int w_own() const { return threads * sites_per_thread - 2 * (K - 1); }
+};
+
+struct F64Step {
+    const TileDesc* tiles;   // tiles of w_own sites
+    int32_t n_tiles;
+    int32_t w_own;
+    int32_t K;               // steps in this launch, up to the shape's
+    int32_t n_nodes;         // nodes per site of the batch's largest cache (room in shared memory)
+    const ChainDesc* chains;
+    const double* u_in;
+    double* u_out;
+    F64State in, out;        // disorder caches (the same arrays for in place: K = 1 only)
+    double dt;
+    uint64_t seed;
+};
+
+F64Shape f64_shape(int64_t n_sites);
+size_t f64_step_smem(const F64Shape& s, int n_nodes);
+cudaError_t f64_step(const F64Step& a, const F64Shape& s, cudaStream_t st);
 cudaError_t f64_observe(const F64Launch& a, cudaStream_t st);
 cudaError_t f64_init(const ChainDesc* chains, const TileDesc* tiles, int32_t n_tiles, int32_t w_tile,
-                     F64State st, uint64_t seed, int any_rb, const double* u_in, cudaStream_t stream);
+                     F64State st, uint64_t seed, int look, const double* u_in, cudaStream_t stream);
 cudaError_t f64_cells(const ChainDesc* chains, const TileDesc* tiles, int32_t n_tiles, int32_t w_tile,
                       const double* u, int32_t* cells_out, cudaStream_t stream);
 
