@@ -135,6 +135,8 @@ int qew_set_samples(qew_handle h, const uint32_t* s);
  * own chains, without changing their state, as soon as they are at least 1024 Euler steps past
  * the flat start (the best shape changes while the rate of cell crossings decays after the flat
  * start); until then the default shape is used.
+ * A handle whose shape was neither set nor autotuned runs the launches between its observations in a
+ * shape chosen by its number of sites.
  * Results never depend on the shape beyond FP32 rounding order, which is identical: each
  * site's arithmetic is the same for every shape.
  */

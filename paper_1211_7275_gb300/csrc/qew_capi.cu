@@ -88,9 +88,13 @@ struct qew_ctx {
     int n_cache = 2;
     int32_t period = 0;   // disorder period M in u (0: aperiodic)
 
-    // launch shape of the fused kernel (defaults: the best measured shapes on a GB300)
+    // launch shape of the fused kernel: sites per lane, steps per launch, warp tiles per block
     int S = 23, K = 16, tpc = 2;
     bool autotune_pending = false;
+    // Shape of the launches without observations; the same unless the handle has its default shape
+    // (step_shape).  The sums of an observation follow the tiles of the shape above.
+    int step_S = 23, step_K = 16, step_tpc = 2;
+    bool shape_given = false;
 
     std::vector<ChainDesc> h_chains;
     ChainDesc* d_chains = nullptr;
@@ -98,6 +102,9 @@ struct qew_ctx {
     int32_t n_tiles[kNumKinds] = {};
     int32_t tile_base[kNumKinds] = {};
     int32_t w_own[kNumKinds] = {};   // sites a warp tile owns, per disorder kind
+    TileDesc* d_step_tiles[kNumKinds] = {};   // the same of the step shape, where it is another one
+    int32_t n_step_tiles[kNumKinds] = {};
+    int32_t step_w_own[kNumKinds] = {};
     TileDesc* d_btiles = nullptr;
     int32_t n_btiles = 0;
 
@@ -242,8 +249,10 @@ void free_all(qew_ctx* h)
     free_split(h);
     free_f64(h);
     dev_free(h->d_chains);
-    for (int k = 0; k < kNumKinds; ++k)
+    for (int k = 0; k < kNumKinds; ++k) {
         dev_free(h->d_tiles[k]);
+        dev_free(h->d_step_tiles[k]);
+    }
     dev_free(h->d_btiles);
     dev_free(h->d_ftiles);
     dev_free(h->d_shift);
@@ -324,14 +333,48 @@ size_t max_kind_smem(const qew_ctx* h, int S, int tiles_per_cta)
     return m;
 }
 
+// Step shape of a handle in its default shape, by the number of sites.  Few sites are latency: a
+// launch costs some 9 us beside its steps, so deep launches, and a step of a warp of 7 sites per lane
+// takes half the time of one of 23.  More sites fill the SMs better with wider tiles (less halo, fuller
+// Philox rounds).  us per step, default shape | best, 4 chains of the random field, Case 3, uniform and
+// Gaussian cubic random bond:
+//   2^16 sites   1.84 | .82 (224 x 48), 2.10 | .97, 1.13 | .73, 1.36 | 1.04
+//   2^18         1.96 | .99 (480 x 48), 2.19 | 1.17, 1.32 | .91, 1.62 | 1.39
+//   2^20         1.89 | 1.38 (992 x 48) and 1.42 (736 x 48), 2.26 | 1.75 (736 x 48), 2.54 | 1.75 (480 x 48), 3.61 | 2.73
+//   2^22         4.84 | 3.73 (992 x 48), 6.21 | 5.15 (736 x 48), 8.21 | 5.23 (480 x 48), 11.5 | 7.7 (480 x 32)
+void step_shape(qew_ctx* h)
+{
+    h->step_S = h->S;
+    h->step_K = h->K;
+    h->step_tpc = h->tpc;
+    if (h->shape_given)
+        return;
+    h->step_K = 48;
+    h->step_tpc = 1;
+    if (h->n_sites < (int64_t(3) << 16)) {
+        h->step_S = 7;
+    } else if (h->n_sites < (int64_t(3) << 18)) {
+        h->step_S = 15;
+    } else if (h->kinds_mask >> kRBGLinear & 1) {
+        h->step_S = 23;
+        h->step_tpc = 2;
+    } else {
+        h->step_S = h->n_sites < (int64_t(3) << 19) ? 23 : 31;
+    }
+}
+
 // Tile lists for the current precision and launch shape; uploads chain descriptors and sizes
 // the partial-sum buffer.
 int build_layout(qew_ctx* h)
 {
     drop_graph(h);   // captured launches point at the descriptors rebuilt here
-    for (int k = 0; k < kNumKinds; ++k)
+    step_shape(h);
+    const bool own_step = h->precision == QEW_FP32_SPLIT && !h->shape_given;
+    for (int k = 0; k < kNumKinds; ++k) {
         h->w_own[k] = 32 * kind_S(k, h->S) - 2 * h->K;
-    std::vector<TileDesc> lists[kNumKinds];
+        h->step_w_own[k] = 32 * kind_S(k, h->step_S) - 2 * h->step_K;
+    }
+    std::vector<TileDesc> lists[kNumKinds], step_lists[kNumKinds];
     std::vector<TileDesc> blocks, ftiles;
     h->f64s = f64_shape(h->n_sites);
     h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
@@ -356,6 +399,9 @@ int build_layout(qew_ctx* h)
             for (int64_t st = 0; st < d.L; st += h->w_own[d.kind])
                 lst.push_back(TileDesc{c, static_cast<int32_t>(st)});
             count[c] = static_cast<int32_t>(lst.size()) - first[c];
+            if (own_step)
+                for (int64_t st = 0; st < d.L; st += h->step_w_own[d.kind])
+                    step_lists[d.kind].push_back(TileDesc{c, static_cast<int32_t>(st)});
         } else {
             for (int64_t st = 0; st < d.L; st += h->f64s.w_own())
                 ftiles.push_back(TileDesc{c, static_cast<int32_t>(st)});
@@ -387,8 +433,10 @@ int build_layout(qew_ctx* h)
             h->n_tiles[k] = 0;
     }
     dev_free(h->d_chains);
-    for (int k = 0; k < kNumKinds; ++k)
+    for (int k = 0; k < kNumKinds; ++k) {
         dev_free(h->d_tiles[k]);
+        dev_free(h->d_step_tiles[k]);
+    }
     dev_free(h->d_btiles);
     QEW_CUDA(h, dev_alloc(&h->d_chains, h->h_chains.size()), "allocating chain descriptors");
     QEW_CUDA(h, cudaMemcpy(h->d_chains, h->h_chains.data(), h->h_chains.size() * sizeof(ChainDesc),
@@ -398,6 +446,14 @@ int build_layout(qew_ctx* h)
             continue;
         QEW_CUDA(h, dev_alloc(&h->d_tiles[k], lists[k].size()), "allocating tile lists");
         QEW_CUDA(h, cudaMemcpy(h->d_tiles[k], lists[k].data(), lists[k].size() * sizeof(TileDesc),
+                               cudaMemcpyHostToDevice), "uploading tile lists");
+    }
+    for (int k = 0; k < kNumKinds; ++k) {
+        h->n_step_tiles[k] = static_cast<int32_t>(step_lists[k].size());
+        if (step_lists[k].empty())
+            continue;
+        QEW_CUDA(h, dev_alloc(&h->d_step_tiles[k], step_lists[k].size()), "allocating tile lists");
+        QEW_CUDA(h, cudaMemcpy(h->d_step_tiles[k], step_lists[k].data(), step_lists[k].size() * sizeof(TileDesc),
                                cudaMemcpyHostToDevice), "uploading tile lists");
     }
     h->n_btiles = static_cast<int32_t>(blocks.size());
@@ -450,6 +506,7 @@ int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shif
 // One launch of the fused kernel (per disorder kind): K steps and the observations among them.
 struct Segment {
     int K = 0;
+    bool step_only = false;        // in the step shape (no observations)
     int n_obs = 0;
     uint16_t at[kMaxLaunchObs];    // observation after so many of the steps,
     uint16_t len[kMaxLaunchObs];   // its own segment being the last so many
@@ -459,8 +516,9 @@ struct Segment {
 SplitLaunch split_args(qew_ctx* h, int kind, const Segment& s, SplitState in, SplitState out)
 {
     SplitLaunch a{};
-    a.tiles = h->d_tiles[kind];
-    a.n_tiles = h->n_tiles[kind];
+    const bool other = s.step_only && !h->shape_given;
+    a.tiles = other ? h->d_step_tiles[kind] : h->d_tiles[kind];
+    a.n_tiles = other ? h->n_step_tiles[kind] : h->n_tiles[kind];
     a.tile_base = h->tile_base[kind];
     a.chains = h->d_chains;
     a.in = in;
@@ -469,8 +527,8 @@ SplitLaunch split_args(qew_ctx* h, int kind, const Segment& s, SplitState in, Sp
     // Windows start on 16-byte boundaries where the halo has room for it (bulk copies; a launch of
     // one step through plain loads and stores took 2.4 times a launch of four on 4 x 2^25 sites).
     const int pad = (s.K + 3) & ~3;
-    a.pad = (pad + s.K <= 2 * h->K) ? pad : s.K;
-    a.w_own = h->w_own[kind];
+    a.pad = (pad + s.K <= 2 * (other ? h->step_K : h->K)) ? pad : s.K;
+    a.w_own = other ? h->step_w_own[kind] : h->w_own[kind];
     a.dt = static_cast<float>(h->dt);
     a.seed = h->seed;
     a.n_obs = s.n_obs;
@@ -511,7 +569,8 @@ int launch_split_all(qew_ctx* h, const Segment& s, SplitState in, SplitState out
                 return rc;
             QEW_CUDA(h, cudaEventRecord(e0, h->stream), "recording a timing event");
         }
-        QEW_CUDA(h, split_step(k, kind_S(k, h->S), h->tpc, a, h->stream), "launching the fused step kernel");
+        QEW_CUDA(h, split_step(k, kind_S(k, s.step_only ? h->step_S : h->S), s.step_only ? h->step_tpc : h->tpc, a, h->stream),
+                 "launching the fused step kernel");
         if (h->stats_on)
             QEW_CUDA(h, cudaEventRecord(e1, h->stream), "recording a timing event");
         h->n_launches += 1;
@@ -637,6 +696,20 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
     Segment s;
     int64_t at = h->step;   // step reached with the segment being packed
     int rc = QEW_OK;
+    // steps without observations, in launches of the step shape as even as they come
+    auto run_steps = [&](int64_t n) -> int {
+        while (n > 0) {
+            const int64_t launches = (n + h->step_K - 1) / h->step_K;
+            Segment b;
+            b.step_only = true;
+            b.K = static_cast<int>(std::min<int64_t>({n, h->step_K, ((n + launches - 1) / launches + 3) & ~int64_t(3)}));
+            const int e = run_segment(h, b, nullptr);
+            if (e != QEW_OK)
+                return e;
+            n -= b.K;
+        }
+        return QEW_OK;
+    };
     for (int32_t k = 0; k < n_targets; ++k) {
         bool first = true;   // (an observation at the current step has a segment of no steps)
         while (at < targets[k] || (first && d_obs)) {
@@ -651,6 +724,22 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
             int64_t end = targets[k];
             if (h->autotune_pending && at < kTuneAfterSteps)
                 end = std::min<int64_t>(end, kTuneAfterSteps);
+            // Where launches without observations have their own shape, all steps but the segment of an
+            // observation at `end` take it (the segment is what is left over whole K steps).
+            if (!h->shape_given && at < end) {
+                const bool observed = d_obs && end == targets[k];
+                const int64_t bulk = observed ? (end - at - 1) / h->K * h->K : end - at;
+                if (bulk > 0) {
+                    rc = run_segment(h, s, d_obs);
+                    if (rc == QEW_OK)
+                        rc = run_steps(bulk);
+                    if (rc != QEW_OK)
+                        return rc;
+                    s = Segment();
+                    at += bulk;
+                    continue;
+                }
+            }
             const int len = static_cast<int>(std::min<int64_t>(h->K, end - at));
             const bool observe = d_obs && at + len == targets[k];
             int left = len;
@@ -696,9 +785,11 @@ int autotune(qew_ctx* h)
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
             std::tie(h->S, h->K, h->tpc) = it->second;
+            h->shape_given = true;
             return build_layout(h);
         }
     }
+    h->shape_given = true;
     const int S_all[] = {7, 15, 23, 31, 39};
     const int K_all[] = {4, 8, 16, 32};
     const int T_all[] = {1, 2, 4};
@@ -1226,6 +1317,7 @@ int qew_set_tuning(qew_handle h, int32_t tile_w, int32_t K, int32_t tiles_per_ct
     h->S = S;
     h->K = K;
     h->tpc = tiles_per_cta;
+    h->shape_given = true;
     h->autotune_pending = false;
     return build_layout(h);
 }
