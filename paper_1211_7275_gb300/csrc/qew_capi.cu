@@ -98,11 +98,11 @@ struct qew_ctx {
 
     std::vector<ChainDesc> h_chains;
     ChainDesc* d_chains = nullptr;
-    TileDesc* d_tiles[kNumKinds] = {};
+    WarpTile* d_tiles[kNumKinds] = {};
     int32_t n_tiles[kNumKinds] = {};
     int32_t tile_base[kNumKinds] = {};
     int32_t w_own[kNumKinds] = {};   // sites a warp tile owns, per disorder kind
-    TileDesc* d_step_tiles[kNumKinds] = {};   // the same of the step shape, where it is another one
+    WarpTile* d_step_tiles[kNumKinds] = {};   // the same of the step shape, where it is another one
     int32_t n_step_tiles[kNumKinds] = {};
     int32_t step_w_own[kNumKinds] = {};
     TileDesc* d_btiles = nullptr;
@@ -374,13 +374,14 @@ int build_layout(qew_ctx* h)
         h->w_own[k] = 32 * kind_S(k, h->S) - 2 * h->K;
         h->step_w_own[k] = 32 * kind_S(k, h->step_S) - 2 * h->step_K;
     }
-    std::vector<TileDesc> lists[kNumKinds], step_lists[kNumKinds];
+    // first tile of each chain in its kind's list, and the lists' lengths, in both shapes
+    std::vector<int32_t> first(h->n_chains), step_first(h->n_chains);
+    int64_t n_list[kNumKinds] = {}, n_step_list[kNumKinds] = {};
     std::vector<TileDesc> blocks, ftiles;
     h->f64s = f64_shape(h->n_sites);
     h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
                  h->f64s.look ? ((h->kinds_mask >> kRBGLinear & 1) ? 4 : 3) : 2;
     h->h_chains.assign(h->n_chains, ChainDesc{});
-    std::vector<int32_t> first(h->n_chains), count(h->n_chains);
     for (int32_t c = 0; c < h->n_chains; ++c) {
         ChainDesc& d = h->h_chains[c];
         d.offset = h->precision == QEW_FP32_SPLIT ? h->soffset[c] : h->offset[c];
@@ -394,14 +395,13 @@ int build_layout(qew_ctx* h)
         for (int64_t st = 0; st < d.L; st += kBlockTile)   // 64-bit: L may reach 2^31 - 1
             blocks.push_back(TileDesc{c, static_cast<int32_t>(st)});
         if (h->precision == QEW_FP32_SPLIT) {
-            auto& lst = lists[d.kind];
-            first[c] = static_cast<int32_t>(lst.size());
-            for (int64_t st = 0; st < d.L; st += h->w_own[d.kind])
-                lst.push_back(TileDesc{c, static_cast<int32_t>(st)});
-            count[c] = static_cast<int32_t>(lst.size()) - first[c];
-            if (own_step)
-                for (int64_t st = 0; st < d.L; st += h->step_w_own[d.kind])
-                    step_lists[d.kind].push_back(TileDesc{c, static_cast<int32_t>(st)});
+            first[c] = static_cast<int32_t>(n_list[d.kind]);
+            d.ntiles = static_cast<int32_t>((int64_t(d.L) + h->w_own[d.kind] - 1) / h->w_own[d.kind]);
+            n_list[d.kind] += d.ntiles;
+            if (own_step) {
+                step_first[c] = static_cast<int32_t>(n_step_list[d.kind]);
+                n_step_list[d.kind] += (int64_t(d.L) + h->step_w_own[d.kind] - 1) / h->step_w_own[d.kind];
+            }
         } else {
             for (int64_t st = 0; st < d.L; st += h->f64s.w_own())
                 ftiles.push_back(TileDesc{c, static_cast<int32_t>(st)});
@@ -412,12 +412,11 @@ int build_layout(qew_ctx* h)
         int32_t base = 0;
         for (int k = 0; k < kNumKinds; ++k) {
             h->tile_base[k] = base;
-            h->n_tiles[k] = static_cast<int32_t>(lists[k].size());
+            h->n_tiles[k] = static_cast<int32_t>(n_list[k]);
             base += h->n_tiles[k];
         }
         for (int32_t c = 0; c < h->n_chains; ++c) {
             h->h_chains[c].tile0 = h->tile_base[h->kind[c]] + first[c];
-            h->h_chains[c].ntiles = count[c];
         }
         slots = static_cast<size_t>(base);
     } else {
@@ -439,32 +438,42 @@ int build_layout(qew_ctx* h)
     }
     dev_free(h->d_btiles);
     QEW_CUDA(h, dev_alloc(&h->d_chains, h->h_chains.size()), "allocating chain descriptors");
-    QEW_CUDA(h, cudaMemcpy(h->d_chains, h->h_chains.data(), h->h_chains.size() * sizeof(ChainDesc),
-                           cudaMemcpyHostToDevice), "uploading chain descriptors");
-    for (int k = 0; k < kNumKinds; ++k) {
-        if (lists[k].empty())
-            continue;
-        QEW_CUDA(h, dev_alloc(&h->d_tiles[k], lists[k].size()), "allocating tile lists");
-        QEW_CUDA(h, cudaMemcpy(h->d_tiles[k], lists[k].data(), lists[k].size() * sizeof(TileDesc),
-                               cudaMemcpyHostToDevice), "uploading tile lists");
-    }
-    for (int k = 0; k < kNumKinds; ++k) {
-        h->n_step_tiles[k] = static_cast<int32_t>(step_lists[k].size());
-        if (step_lists[k].empty())
-            continue;
-        QEW_CUDA(h, dev_alloc(&h->d_step_tiles[k], step_lists[k].size()), "allocating tile lists");
-        QEW_CUDA(h, cudaMemcpy(h->d_step_tiles[k], step_lists[k].data(), step_lists[k].size() * sizeof(TileDesc),
-                               cudaMemcpyHostToDevice), "uploading tile lists");
+    QEW_CUDA(h, cudaMemcpyAsync(h->d_chains, h->h_chains.data(), h->h_chains.size() * sizeof(ChainDesc),
+                                cudaMemcpyHostToDevice, h->stream), "uploading chain descriptors");
+    // the warp tiles are written on the device, from the chains and these
+    int32_t* d_first = nullptr;
+    if (h->precision == QEW_FP32_SPLIT) {
+        QEW_CUDA(h, dev_alloc(&d_first, 2 * static_cast<size_t>(h->n_chains)), "allocating tile lists");
+        std::vector<int32_t> both(first);
+        both.insert(both.end(), step_first.begin(), step_first.end());
+        cudaError_t e = cudaMemcpyAsync(d_first, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
+        for (int k = 0; k < kNumKinds; ++k) {
+            h->n_step_tiles[k] = static_cast<int32_t>(n_step_list[k]);
+            if (e == cudaSuccess && n_list[k] > 0)
+                e = dev_alloc(&h->d_tiles[k], n_list[k]);
+            if (e == cudaSuccess && n_list[k] > 0)
+                e = split_tiles(h->d_chains, h->n_chains, k, h->w_own[k], d_first, h->d_tiles[k], h->stream);
+            if (e == cudaSuccess && n_step_list[k] > 0)
+                e = dev_alloc(&h->d_step_tiles[k], n_step_list[k]);
+            if (e == cudaSuccess && n_step_list[k] > 0)
+                e = split_tiles(h->d_chains, h->n_chains, k, h->step_w_own[k], d_first + h->n_chains, h->d_step_tiles[k], h->stream);
+        }
+        if (e == cudaSuccess)
+            e = cudaStreamSynchronize(h->stream);
+        dev_free(d_first);
+        QEW_CUDA(h, e, "writing tile lists");
     }
     h->n_btiles = static_cast<int32_t>(blocks.size());
     QEW_CUDA(h, dev_alloc(&h->d_btiles, blocks.size()), "allocating block tiles");
-    QEW_CUDA(h, cudaMemcpy(h->d_btiles, blocks.data(), blocks.size() * sizeof(TileDesc), cudaMemcpyHostToDevice),
+    QEW_CUDA(h, cudaMemcpyAsync(h->d_btiles, blocks.data(), blocks.size() * sizeof(TileDesc), cudaMemcpyHostToDevice,
+                                h->stream),
              "uploading block tiles");
     dev_free(h->d_ftiles);
     h->n_ftiles = static_cast<int32_t>(ftiles.size());
     if (!ftiles.empty()) {
         QEW_CUDA(h, dev_alloc(&h->d_ftiles, ftiles.size()), "allocating FP64 tiles");
-        QEW_CUDA(h, cudaMemcpy(h->d_ftiles, ftiles.data(), ftiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice),
+        QEW_CUDA(h, cudaMemcpyAsync(h->d_ftiles, ftiles.data(), ftiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice,
+                                    h->stream),
                  "uploading FP64 tiles");
     }
     // room for the partials of as many observations as 256 MB hold
@@ -520,7 +529,6 @@ SplitLaunch split_args(qew_ctx* h, int kind, const Segment& s, SplitState in, Sp
     a.tiles = other ? h->d_step_tiles[kind] : h->d_tiles[kind];
     a.n_tiles = other ? h->n_step_tiles[kind] : h->n_tiles[kind];
     a.tile_base = h->tile_base[kind];
-    a.chains = h->d_chains;
     a.in = in;
     a.out = out;
     a.K = s.K;

@@ -57,11 +57,23 @@ __host__ __device__ __forceinline__ int32_t wrap_node(int32_t n, int32_t period)
     return r < 0 ? r + period : r;
 }
 
-// One warp tile of the fused kernel (or one block tile of the FP64 kernels): chain and first
-// owned site.
+// One block tile of the FP64, initialisation and conversion kernels: chain and first owned site.
 struct TileDesc {
     int32_t chain;
     int32_t start;
+};
+
+// One warp tile of the fused kernel: its first owned site (in the state arrays and in its chain) and
+// what the kernel needs of the chain, so that a tile starts with one load and not with two that wait
+// for one another.
+struct alignas(32) WarpTile {
+    int64_t p;        // state index of the first owned site
+    int32_t start;    // its index in the chain
+    int32_t L;
+    int32_t chain;
+    uint32_t s;
+    float f;
+    int32_t period;
 };
 
 // ---------------------------------------------------------------------------------------

@@ -306,8 +306,8 @@ __device__ __forceinline__ int mask_top(unsigned long long m) { return 63 - __cl
 template <int KIND, int S, bool OBS>
 struct MaxRegs {
     static constexpr int value = (OBS ? 16 : 0) + (quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
-                                 KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 104 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
-                                                      (S <= 8 ? 64 : S <= 16 ? 96 : S <= 31 ? 128 : 160));
+                                 KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 112 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
+                                                      (S <= 8 ? 64 : S <= 16 ? 112 : S <= 31 ? 128 : 160));
 };
 
 // The cell of window position x at this point of the K loop, in every lane.
@@ -340,7 +340,7 @@ __device__ __forceinline__ int32_t cell_at(int32_t* s_cell, int x, int lane, int
 // then do not depend on how steps and observations are spread over launches.  Each lane adds up
 // other sites than its own, so the values go through the slot.
 template <int KIND, int S>
-__device__ __forceinline__ void observe_tile(const SplitLaunch& a, const ChainDesc& ch, int tile, int chain, int obs, int32_t ref,
+__device__ __forceinline__ void observe_tile(const SplitLaunch& a, float f, int tile, int chain, int obs, int32_t ref,
                                              int owned, int pad, int32_t N0, int lane, const pair_t (&c)[S / 2],
                                              const pair_t (&d)[S / 2], float cT, float dT, typename Moves<S>::mask upper,
                                              int32_t* s_cell, float* s_off, const float* s_loop, const float* s_loopc)
@@ -348,7 +348,6 @@ __device__ __forceinline__ void observe_tile(const SplitLaunch& a, const ChainDe
     using T = Tile<KIND, S>;
     using M = Moves<S>;
     constexpr int H = S / 2;
-    const float f = ch.f32;
     const float dref = static_cast<float>(ref - N0);   // exact
     const int first = lane * S - a.obs_len[obs];       // this lane's run, from the first owned site
     float* slot = T::has_cache ? reinterpret_cast<float*>(s_cell) : s_off;
@@ -430,6 +429,15 @@ __device__ __forceinline__ void observe_tile(const SplitLaunch& a, const ChainDe
     }
 }
 
+// A value that is the same in every lane, in a uniform register: the warp reduction returns it there,
+// and what is computed from it (addresses, the disorder's counter words, branches) follows.  Per-lane
+// registers are what the kernel is short of; the warp index alone gained 0.5% (random field) to 4%
+// (uniform random bond).
+__device__ __forceinline__ unsigned uniform(unsigned v)
+{
+    return __reduce_max_sync(kFull, v);
+}
+
 // OBS: whether the launch observes at all.  The observation code in the step loop takes registers
 // from it, so that launches without any (nearly all of a long relaxation's) have a kernel of their own.
 template <int KIND, int S, bool OBS>
@@ -444,7 +452,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
     __shared__ uint64_t s_bar[8];
 
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = static_cast<int>(uniform(threadIdx.x >> 5));
     const int tile = blockIdx.x * (blockDim.x >> 5) + warp;
     if (tile >= a.n_tiles)
         return;  // whole warp; the kernel uses no block-wide barrier
@@ -458,33 +466,31 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
     float2* s_nodes = reinterpret_cast<float2*>(wsm + T::nodes);
     uint16_t* s_q = reinterpret_cast<uint16_t*>(wsm + T::queue);
 
-    const TileDesc td = a.tiles[tile];
-    const ChainDesc ch = a.chains[td.chain];
-    const int32_t L = ch.L;
     const int K = a.K;
     const int pad = a.pad;   // first owned window position
-    const int owned = min(a.w_own, L - td.start);
-    const int64_t wstart = static_cast<int64_t>(td.start) - pad;
+    const WarpTile wt = a.tiles[tile];
+    const int32_t L = static_cast<int32_t>(uniform(wt.L));
+    const int32_t start = static_cast<int32_t>(uniform(wt.start));
+    const int owned = min(a.w_own, L - start);
+    const int64_t wstart = static_cast<int64_t>(start) - pad;
     const bool contiguous = (wstart >= 0) && (wstart + TW <= L);
-    const float f = ch.f32;
-    const uint32_t s = ch.s;
-    const int32_t period = ch.period;
+    const float f = __uint_as_float(uniform(__float_as_uint(wt.f)));
+    const uint32_t s = uniform(wt.s);
+    const int32_t period = static_cast<int32_t>(uniform(wt.period));
+    const int64_t chain0 = wt.p - wt.start;   // state index of the chain's first site
 
     // ---- stage the window in this warp's shared-memory slice ----
     // Contiguous, 16-byte aligned windows arrive by TMA bulk copies (one per array, completion
     // on the warp's mbarrier); windows that wrap around the chain or start unaligned use
     // coalesced read-only loads.  Offsets come first, with the cache, and then the cells through
     // the same slot, where they stay.
-    const bool tma_in = contiguous && (((ch.offset + wstart) & 3) == 0);
-    const int64_t p0 = ch.offset + wstart;
+    const int64_t p0 = wt.p - pad;
+    const bool tma_in = contiguous && (p0 & 3) == 0;
     uint64_t* bar = &s_bar[warp];
     if (tma_in) {
         if (lane == 0) {
             mbar_init(bar, 1);
             fence_mbar_init();
-        }
-        __syncwarp();
-        if (lane == 0) {
             mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::has_cache ? 0 : 4)));
             tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
             if constexpr (!T::has_cache)
@@ -509,7 +515,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
         }
     } else {
         for (int x = lane; x < TW; x += 32) {
-            const int64_t p = ch.offset + site_index(wstart, x, contiguous, L);
+            const int64_t p = chain0 + site_index(wstart, x, contiguous, L);
             s_off[x] = __ldg(a.in.off + p);
             if constexpr (!T::has_cache)
                 s_cell[x] = __ldg(a.in.cell + p);
@@ -586,14 +592,14 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
             }
         } else {
             for (int x = lane; x < TW; x += 32)
-                s_cell[x] = __ldg(a.in.cell + ch.offset + site_index(wstart, x, contiguous, L));
+                s_cell[x] = __ldg(a.in.cell + chain0 + site_index(wstart, x, contiguous, L));
             __syncwarp();
         }
     }
     // Cells are carried as exact small floats relative to the warp's reference cell N0 (window
     // position 0): a neighbour difference is then (c' - c) + (d' - d), three FP32 operations.
     // Neighbouring displacements differ by less than 2^12, so a tile's cells stay far below 2^24.
-    const int32_t N0 = s_cell[0];
+    const int32_t N0 = static_cast<int32_t>(uniform(s_cell[0]));
 #pragma unroll
     for (int p = 0; p < H; ++p)
         c[p] = pk(static_cast<float>(s_cell[lane * S + p] - N0), static_cast<float>(s_cell[lane * S + H + p] - N0));
@@ -634,7 +640,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
                 obs_ref = cell_at<KIND, S>(s_cell, pad - a.obs_len[obs], lane, N0, c, cT, upper);
                 obs_marked = true;
             } else {
-                observe_tile<KIND, S>(a, ch, tile, td.chain, obs, obs_ref, owned, pad, N0, lane, c, d, cT, dT, upper, s_cell,
+                observe_tile<KIND, S>(a, f, tile, wt.chain, obs, obs_ref, owned, pad, N0, lane, c, d, cT, dT, upper, s_cell,
                                       s_off, s_loop, s_loopc);
                 obs_marked = false;
                 ++obs;
@@ -820,13 +826,13 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
         if (lane == 0 && n_cross)
             atomicAdd(a.crossings, static_cast<unsigned long long>(n_cross));
     }
-
     if (K == 0)
         return;
 
+
     // ---- write the owned sites back: registers -> shared -> global ----
     __syncwarp();
-    const int64_t out0 = ch.offset + td.start;
+    const int64_t out0 = wt.p;
     const bool tma_out = ((pad & 3) == 0) && ((out0 & 3) == 0) && ((owned & 3) == 0);
     if constexpr (!T::has_cache || KIND == kRBGLinear) {
         // (the other kinds' slots already hold the cells)
@@ -919,7 +925,8 @@ __global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(Sp
             if constexpr (!T::has_cache)
                 tma_store_1d(a.out.cell + out0, s_cell + pad, static_cast<uint32_t>(owned) * 4);
             tma_store_commit();
-            tma_store_wait_read_all();   // shared memory must outlive the reads; the writes end with the kernel
+            // shared memory must outlive the reads (the writes end with the kernel)
+            tma_store_wait_read_all();
         }
     } else {
         __syncwarp();
@@ -966,6 +973,19 @@ template <int KIND, int S>
 cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
 {
     return a.n_obs > 0 ? launch_split_as<KIND, S, true>(tiles_per_cta, a, st) : launch_split_as<KIND, S, false>(tiles_per_cta, a, st);
+}
+
+__global__ void split_tiles_kernel(const ChainDesc* chains, int kind, int32_t w_own, const int32_t* first, WarpTile* tiles)
+{
+    const int32_t c = blockIdx.x;
+    const ChainDesc ch = chains[c];
+    if (ch.kind != kind)
+        return;
+    WarpTile* mine = tiles + first[c];
+    for (int64_t k = threadIdx.x; k * w_own < ch.L; k += blockDim.x) {
+        const int32_t start = static_cast<int32_t>(k * w_own);
+        mine[k] = WarpTile{ch.offset + start, start, ch.L, c, ch.s, ch.f32, ch.period};
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1106,6 +1126,13 @@ cudaError_t split_step(int kind, int S, int tiles_per_cta, const SplitLaunch& a,
         }
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int kind, int32_t w_own, const int32_t* first,
+                        WarpTile* tiles, cudaStream_t stream)
+{
+    split_tiles_kernel<<<n_chains, 256, 0, stream>>>(chains, kind, w_own, first, tiles);
+    return cudaGetLastError();
 }
 
 cudaError_t split_init(const ChainDesc* chains, int32_t, const TileDesc* tiles, int32_t n_tiles, int32_t w_tile,
