@@ -220,11 +220,20 @@ __device__ __forceinline__ float gauss_value_f32(uint4 w)
     return gauss_value_plus_f32(w, 0.0f);
 }
 
-__device__ __forceinline__ double gauss_value_f64(uint4 w)
+// The two factors of the FP64 value, and the value: their product.
+__device__ __forceinline__ double gauss_radius_f64(uint4 w)
 {
     const double u1 = (static_cast<double>(w.x) + 0.5) * 0x1p-32;
+    return sqrt(-2.0 * log(u1));
+}
+__device__ __forceinline__ double gauss_angle_f64(uint4 w)
+{
     const double u2 = (static_cast<double>(w.y) + 0.5) * 0x1p-32;
-    return sqrt(-2.0 * log(u1)) * cospi(2.0 * u2);
+    return cospi(2.0 * u2);
+}
+__device__ __forceinline__ double gauss_value_f64(uint4 w)
+{
+    return __dmul_rn(gauss_radius_f64(w), gauss_angle_f64(w));
 }
 
 // V = (x0 + 1/2) 2^-31 - 1, uniform on (-1, 1).
