@@ -303,11 +303,11 @@ __device__ __forceinline__ int mask_top(unsigned long long m) { return 63 - __cl
 // Registers per thread allowed to the kernel, the fastest measured of 80 .. 184 on each shape.  Both
 // ways cost: at 992-site random-field tiles 120 (and the same 16 warps per SM) instead of 128 lost 3%,
 // 96 lost 23%, and 144 (14 warps) lost 8%; Case 3 redraws less often and gains 1 to 6% from 144 and 168.
-template <int KIND, int S, bool OBS>
+template <int KIND, int S>
 struct MaxRegs {
-    static constexpr int value = (OBS ? 16 : 0) + (quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
+    static constexpr int value = quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
                                  KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 112 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
-                                                      (S <= 8 ? 64 : S <= 16 ? 112 : S <= 31 ? 128 : 160));
+                                                      (S <= 8 ? 64 : S <= 16 ? 112 : S <= 31 ? 128 : 160);
 };
 
 // The cell of window position x at this point of the K loop, in every lane.
@@ -353,25 +353,35 @@ __device__ __forceinline__ void observe_tile(const SplitLaunch& a, float f, int 
     float* slot = T::has_cache ? reinterpret_cast<float*>(s_cell) : s_off;
     float sF = 0.0f, sy = 0.0f, syy = 0.0f;
     int cnt = 0;
+    // The run's loads have to be ahead of its serial sums.  4 x 2^25 random-field sites, 36 observations
+    // over 1024 steps: 16.2 ms with four ahead and two 4-byte loads per cached value, 9.1 so.
+    constexpr int kRun = KIND == kRF ? S : 8;
     if constexpr (T::has_cache) {
 #pragma unroll
-        for (int j = 0; j < S; ++j) {
-            const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
-            const int row = (j < 2 * H) ? H - 1 - p : H;
-            const int half = (j < H || j == 2 * H) ? 0 : 1;
-            const float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
-            const float* q = s_loop + 4 * (32 * row + lane) + half;
-            float F;
-            if constexpr (KIND == kRF)
-                F = fmaf(dj, q[2] - q[0], q[0]) - f;
-            else if constexpr (KIND == kRBGLinear)
-                F = (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last)) ? q[2] : q[0];
-            else
-                F = fmaf(dj, fmaf(dj, s_loopc[2 * (32 * row + lane) + half], q[2]), q[0]) - f;
-            slot[lane * S + j] = F;
+        for (int p = 0; p <= H; ++p) {
+            // both sites of a pair from one row (the last site's row has one)
+            const int row = (p < H) ? H - 1 - p : H;
+            const int j0 = (p < H) ? p : 2 * H;
+            const float4 q = reinterpret_cast<const float4*>(s_loop)[32 * row + lane];
+            const float d0 = (p < H) ? lo(d[p < H ? p : 0]) : dT, d1 = hi(d[p < H ? p : 0]);
+            float F0, F1;
+            if constexpr (KIND == kRF) {
+                F0 = fmaf(d0, q.z - q.x, q.x) - f;
+                F1 = fmaf(d1, q.w - q.y, q.y) - f;
+            } else if constexpr (KIND == kRBGLinear) {
+                F0 = (upper & ((p < H) ? M::first(p) : M::last)) ? q.z : q.x;
+                F1 = (upper & M::second(p < H ? p : 0)) ? q.w : q.y;
+            } else {
+                const float2 C = reinterpret_cast<const float2*>(s_loopc)[32 * row + lane];
+                F0 = fmaf(d0, fmaf(d0, C.x, q.z), q.x) - f;
+                F1 = fmaf(d1, fmaf(d1, C.y, q.w), q.y) - f;
+            }
+            slot[lane * S + j0] = F0;
+            if (p < H)
+                slot[lane * S + H + p] = F1;
         }
         __syncwarp();
-#pragma unroll 4
+#pragma unroll kRun
         for (int j = 0; j < S; ++j) {
             const int o = first + j;
             if (o >= 0 && o < owned)
@@ -387,7 +397,7 @@ __device__ __forceinline__ void observe_tile(const SplitLaunch& a, float f, int 
         slot[lane * S + j] = (cj - dref) + dj;   // u - ref
     }
     __syncwarp();
-#pragma unroll 4
+#pragma unroll kRun
     for (int j = 0; j < S; ++j) {
         const int o = first + j;
         if (o >= 0 && o < owned) {
@@ -441,7 +451,7 @@ __device__ __forceinline__ unsigned uniform(unsigned v)
 // OBS: whether the launch observes at all.  The observation code in the step loop takes registers
 // from it, so that launches without any (nearly all of a long relaxation's) have a kernel of their own.
 template <int KIND, int S, bool OBS>
-__global__ void __maxnreg__((MaxRegs<KIND, S, OBS>::value)) split_step_kernel(SplitLaunch a)
+__global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLaunch a)
 {
     using T = Tile<KIND, S>;
     using M = Moves<S>;
