@@ -334,14 +334,15 @@ size_t max_kind_smem(const qew_ctx* h, int S, int tiles_per_cta)
 }
 
 // Step shape of a handle in its default shape, by the number of sites.  Few sites are latency: a
-// launch costs some 9 us beside its steps, so deep launches, and a step of a warp of 7 sites per lane
-// takes half the time of one of 23.  More sites fill the SMs better with wider tiles (less halo, fuller
-// Philox rounds).  us per step, default shape | best, 4 chains of the random field, Case 3, uniform and
-// Gaussian cubic random bond:
-//   2^16 sites   1.84 | .82 (224 x 48), 2.10 | .97, 1.13 | .73, 1.36 | 1.04
-//   2^18         1.96 | .99 (480 x 48), 2.19 | 1.17, 1.32 | .91, 1.62 | 1.39
-//   2^20         1.89 | 1.38 (992 x 48) and 1.42 (736 x 48), 2.26 | 1.75 (736 x 48), 2.54 | 1.75 (480 x 48), 3.61 | 2.73
-//   2^22         4.84 | 3.73 (992 x 48), 6.21 | 5.15 (736 x 48), 8.21 | 5.23 (480 x 48), 11.5 | 7.7 (480 x 32)
+// launch costs some 7 us beside its steps, so deep launches, and a step of a warp of 7 or 15 sites per
+// lane takes half the time of one of 23.  More sites fill the SMs better with wider tiles (less halo,
+// fuller Philox rounds).  us per step in the default shape and the two best (tile x K), 4 chains:
+//   sites  random field              Case 3                    uniform cubic             Gaussian cubic
+//   2^13   1.57 .70 224x48 .74 480x96   1.85 .87 480x96 .91 224x48   1.04 .65 both               1.32 .93 224x48 1.07 480x96
+//   2^17   1.65 .72 480x96 .78 224x48   1.90 .88 480x96 .95 480x64   1.06 .67 480x96 .74 224x48   1.43 1.09 224x48 1.12 480x96
+//   2^19   1.96 .97 736x96 1.02 480x96  2.16 1.21 480x96 1.25 480x64  1.52 .95 480x96 1.01 480x48  2.09 1.56 480x96 1.58 480x64
+//   2^20   1.91 1.21 992x64 1.28 736x64 2.23 1.63 736x64 1.67 992x64  2.39 1.63 480x64 1.67 480x48 3.42 2.62 480x32 2.63 480x48
+//   2^22   4.63 3.32 992x64 3.40 992x48 6.10 4.95 736x48 5.07 736x64  7.65 5.05 480x48 5.24 480x64 11.0 7.43 480x32 7.66 480x48
 void step_shape(qew_ctx* h)
 {
     h->step_S = h->S;
@@ -349,17 +350,25 @@ void step_shape(qew_ctx* h)
     h->step_tpc = h->tpc;
     if (h->shape_given)
         return;
-    h->step_K = 48;
-    h->step_tpc = 1;
-    if (h->n_sites < (int64_t(3) << 16)) {
+    const int64_t n = h->n_sites;
+    const bool case1 = h->kinds_mask >> kRBGCubic & 1, case3 = h->kinds_mask >> kRBGLinear & 1;
+    h->step_tpc = n < (int64_t(1) << 18) ? 1 : 2;
+    if (n < (int64_t(3) << 15) || (case1 && n < (int64_t(3) << 16))) {
         h->step_S = 7;
-    } else if (h->n_sites < (int64_t(3) << 18)) {
+        h->step_K = 48;
+    } else if (n < (int64_t(3) << 17) || (case3 && n < (int64_t(3) << 18))) {
         h->step_S = 15;
-    } else if (h->kinds_mask >> kRBGLinear & 1) {
+        h->step_K = 96;
+    } else if (n < (int64_t(3) << 18)) {
         h->step_S = 23;
-        h->step_tpc = 2;
+        h->step_K = 96;
     } else {
-        h->step_S = h->n_sites < (int64_t(3) << 19) ? 23 : 31;
+        h->step_S = case3 ? 23 : 31;
+        h->step_K = n < (int64_t(3) << 19) || !(case3 || (h->kinds_mask & kQuadMask)) ? 64 : 48;
+        if (case1)
+            h->step_K = 32;
+        if (h->kinds_mask & kQuadMask)
+            h->step_tpc = 1;
     }
 }
 

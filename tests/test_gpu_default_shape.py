@@ -35,7 +35,7 @@ def both(qew, L, f, kind, given):
 
 
 @pytest.mark.parametrize("kind", [RF, RB, NONE, RBG_LINEAR, RBG_CUBIC])
-@pytest.mark.parametrize("L", [[1, 129, 777, 5000], [(3 << 16) - 1], [(3 << 16)], [(3 << 18) - 1, 1], [(3 << 19) + 5]])
+@pytest.mark.parametrize("L", [[1, 129, 777, 5000], [3 << 15], [(3 << 16) - 1], [(3 << 16)], [3 << 17], [(3 << 18) - 1, 1], [(3 << 19) + 5]])
 def test_default_shape_equals_the_same_shape_given(qew, kind, L):
     given = (224, 16, 2) if kind in (RB, RBG_CUBIC) else (736, 16, 2)
     both(qew, np.array(L), F[kind], kind, given)
