@@ -34,6 +34,7 @@ static_assert(QEW_RF_GAUSS_LINEAR == kRF && QEW_RB_UNIFORM_CATMULLROM == kRB && 
               "the C ABI's disorder kinds index the kernels' kind table");
 constexpr int32_t kBlockTile = 1024;   // sites per block tile (FP64 path, init, conversions)
 constexpr int64_t kMaxSites = int64_t(1) << 40;
+constexpr size_t kSqKeep = size_t(256) << 20;
 
 struct DeviceGuard {
     int prev = -1;
@@ -140,6 +141,10 @@ struct qew_ctx {
     // structure factor: cuFFT plan of the handle's chain length and batch (made on first use)
     cufftHandle sq_plan = 0;
     bool sq_plan_made = false;
+    // its work area, kept between calls up to kSqKeep bytes
+    double* d_sq_rows = nullptr;
+    double* d_sq_S = nullptr;
+    int32_t sq_S_cap = 0;
 
     // stream owned by the handle (used unless the caller sets one) and the captured observation graph
     cudaStream_t own_stream = nullptr;
@@ -261,6 +266,8 @@ void free_all(qew_ctx* h)
     if (h->h_obs)
         cudaFreeHost(h->h_obs);
     h->h_obs = nullptr;
+    dev_free(h->d_sq_rows);
+    dev_free(h->d_sq_S);
     if (h->sq_plan_made)
         cufftDestroy(h->sq_plan);
     h->sq_plan_made = false;
@@ -1438,7 +1445,11 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
     const int32_t B = h->n_chains;
     if (!h->sq_plan_made) {
         int n = Li, inembed = 2 * (Li / 2 + 1), onembed = Li / 2 + 1;
-        const cufftResult r = cufftPlanMany(&h->sq_plan, 1, &n, &inembed, 1, inembed, &onembed, 1, onembed, CUFFT_D2Z, B);
+        const bool half = sq_half(Li);
+        if (half)
+            n = inembed = onembed = Li / 2;
+        const cufftResult r = cufftPlanMany(&h->sq_plan, 1, &n, &inembed, 1, inembed, &onembed, 1, onembed,
+                                            half ? CUFFT_Z2Z : CUFFT_D2Z, B);
         if (r != CUFFT_SUCCESS)
             return fail(h, r == CUFFT_ALLOC_FAILED ? QEW_ENOMEM : QEW_ECUDA,
                         "cuFFT plan of the structure factor failed (status " + std::to_string(static_cast<int>(r)) + ")");
@@ -1446,13 +1457,20 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
     }
     if (cufftSetStream(h->sq_plan, h->stream) != CUFFT_SUCCESS)
         return fail(h, QEW_ECUDA, "cuFFT could not take the handle's stream");
-    const size_t rows_n = static_cast<size_t>(B) * 2 * (static_cast<size_t>(Li) / 2 + 1);
-    double* d_rows = nullptr;
-    double* d_S = nullptr;
+    const size_t rows_n = static_cast<size_t>(B) * sq_row(Li);
     int rc = QEW_OK;
-    cudaError_t e = dev_alloc(&d_rows, rows_n);
-    if (e == cudaSuccess)
-        e = dev_alloc(&d_S, static_cast<size_t>(n_modes));
+    cudaError_t e = cudaSuccess;
+    if (!h->d_sq_rows)
+        e = dev_alloc(&h->d_sq_rows, rows_n);
+    if (e == cudaSuccess && n_modes > h->sq_S_cap) {
+        dev_free(h->d_sq_S);
+        h->sq_S_cap = 0;
+        e = dev_alloc(&h->d_sq_S, static_cast<size_t>(n_modes));
+        if (e == cudaSuccess)
+            h->sq_S_cap = n_modes;
+    }
+    double* d_rows = h->d_sq_rows;
+    double* d_S = h->d_sq_S;
     if (e != cudaSuccess) {
         rc = cuda_fail(h, e, "allocating the structure-factor work area");
     } else {
@@ -1461,7 +1479,8 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
         else
             e = sq_rows(h->d_chains, B, Li, nullptr, h->u64[h->cur], d_rows, h->stream);
         if (e == cudaSuccess) {
-            const cufftResult r = cufftExecD2Z(h->sq_plan, d_rows, reinterpret_cast<cufftDoubleComplex*>(d_rows));
+            cufftDoubleComplex* z = reinterpret_cast<cufftDoubleComplex*>(d_rows);
+            const cufftResult r = sq_half(Li) ? cufftExecZ2Z(h->sq_plan, z, z, CUFFT_FORWARD) : cufftExecD2Z(h->sq_plan, d_rows, z);
             if (r != CUFFT_SUCCESS)
                 rc = fail(h, QEW_ECUDA, "cuFFT transform failed (status " + std::to_string(static_cast<int>(r)) + ")");
         }
@@ -1475,8 +1494,11 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
         if (rc == QEW_OK && e != cudaSuccess)
             rc = cuda_fail(h, e, "computing the structure factor");
     }
-    dev_free(d_rows);
-    dev_free(d_S);
+    if (rc != QEW_OK || rows_n * sizeof(double) > kSqKeep) {
+        dev_free(h->d_sq_rows);
+        dev_free(h->d_sq_S);
+        h->sq_S_cap = 0;
+    }
     return rc;
 }
 

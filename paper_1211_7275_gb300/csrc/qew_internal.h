@@ -129,9 +129,12 @@ struct ObsList {
 cudaError_t reduce_chains(const ChainDesc* chains, int32_t n_chains, const double* partial, int64_t partial_stride,
                           double* shift, double* obs, const ObsList& list, cudaStream_t stream);
 
-// Structure factor (Eq. 6): rows of u(x) - c0 per chain in the padded layout of an in-place
-// real-to-complex FFT (row stride 2 (L/2 + 1) doubles), from the split state (split != NULL) or
-// the FP64 state; then the mean over chains of |Z(n)|^2 / L^2 for n = 1 .. n_modes.
+// Structure factor (Eq. 6): rows of u(x) - c0 per chain, sq_row(L) doubles apart (with sq_half(L), L of them,
+// read as L/2 complex numbers; else the padded layout of an in-place real-to-complex FFT), from the split state
+// (split != NULL) or the FP64 state; then, from the transforms, the mean over chains of |Z(n)|^2 / L^2 for
+// n = 1 .. n_modes.
+bool sq_half(int32_t L);
+int64_t sq_row(int32_t L);
 cudaError_t sq_rows(const ChainDesc* chains, int32_t n_chains, int32_t L, const SplitState* split, const double* u64,
                     double* rows, cudaStream_t stream);
 cudaError_t sq_power(const void* Z, int32_t L, int32_t n_chains, int32_t n_modes, double* S, cudaStream_t stream);
