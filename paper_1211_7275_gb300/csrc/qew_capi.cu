@@ -18,6 +18,7 @@
 #include <new>
 #include <string>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "qew.h"
@@ -110,6 +111,7 @@ struct qew_ctx {
     int32_t n_btiles = 0;
 
     SplitState sp[2] = {};
+    char* slab[2] = {nullptr, nullptr};   // the state's arrays: one allocation per buffer
     int cur = 0;
     F64State f64[2] = {};            // disorder caches: two copies when a launch takes several steps
     F64Shape f64s = {256, 4, 1, false};
@@ -200,28 +202,13 @@ void dev_free(T*& p)
     p = nullptr;
 }
 
-void free_split(qew_ctx* h)
+void free_state(qew_ctx* h)
 {
     for (int b = 0; b < 2; ++b) {
-        dev_free(h->sp[b].cell);
-        dev_free(h->sp[b].off);
-        dev_free(h->sp[b].rf);
-        dev_free(h->sp[b].qn);
-        dev_free(h->sp[b].q3);
-        dev_free(h->sp[b].qab);
-        dev_free(h->sp[b].qc);
-    }
-}
-
-void free_f64(qew_ctx* h)
-{
-    dev_free(h->u64[0]);
-    dev_free(h->u64[1]);
-    for (int b = 0; b < 2; ++b) {
-        dev_free(h->f64[b].ncache);
-        for (double*& c : h->f64[b].c)
-            dev_free(c);
-        h->f64[b].u = nullptr;
+        dev_free(h->slab[b]);
+        h->sp[b] = SplitState{};
+        h->f64[b] = F64State{};
+        h->u64[b] = nullptr;
     }
 }
 
@@ -251,8 +238,7 @@ void free_all(qew_ctx* h)
     free_events(h);
     dev_free(h->d_crossings);
     dev_free(h->d_error);
-    free_split(h);
-    free_f64(h);
+    free_state(h);
     dev_free(h->d_chains);
     for (int k = 0; k < kNumKinds; ++k) {
         dev_free(h->d_tiles[k]);
@@ -273,36 +259,51 @@ void free_all(qew_ctx* h)
     h->sq_plan_made = false;
 }
 
+// The state's arrays, one allocation per buffer (a handle made and freed per trial paid for up to
+// fourteen).
 int alloc_state(qew_ctx* h)
 {
-    const size_t N = static_cast<size_t>(h->precision == QEW_FP32_SPLIT ? h->n_state : h->n_sites);
-    if (h->precision == QEW_FP32_SPLIT) {
-        free_f64(h);
-        if (h->sp[0].cell)
-            return QEW_OK;
-        for (int b = 0; b < 2; ++b) {
-            QEW_CUDA(h, dev_alloc(&h->sp[b].cell, N), "allocating the cell array");
-            QEW_CUDA(h, dev_alloc(&h->sp[b].off, N), "allocating the offset array");
-            if (h->kinds_mask & kPairMask)
-                QEW_CUDA(h, dev_alloc(&h->sp[b].rf, N), "allocating the two-node disorder cache");
-            if (h->kinds_mask & (kQuadMask | 1 << kRBGLinear))
-                QEW_CUDA(h, dev_alloc(&h->sp[b].q3, N), "allocating the third disorder value");
-            if (h->kinds_mask & kQuadMask) {
-                QEW_CUDA(h, dev_alloc(&h->sp[b].qn, N), "allocating the cubic disorder cache");
-                QEW_CUDA(h, dev_alloc(&h->sp[b].qab, N), "allocating the cubic disorder cache");
-                QEW_CUDA(h, dev_alloc(&h->sp[b].qc, N), "allocating the cubic disorder cache");
+    const bool split = h->precision == QEW_FP32_SPLIT;
+    if (split ? h->sp[0].cell != nullptr : h->u64[0] != nullptr)
+        return QEW_OK;
+    free_state(h);
+    const size_t N = static_cast<size_t>(split ? h->n_state : h->n_sites);
+    for (int b = 0; b < 2; ++b) {
+        size_t size = 0;
+        char* base = nullptr;
+        auto take = [&](auto*& p, size_t count) {   // first pass: sizes; second: addresses
+            using E = std::remove_reference_t<decltype(*p)>;
+            if (base)
+                p = reinterpret_cast<E*>(base + size);
+            size += (count * sizeof(E) + 255) & ~size_t(255);
+        };
+        for (int pass = 0; pass < 2; ++pass) {
+            size = 0;
+            if (split) {
+                SplitState& s = h->sp[b];
+                take(s.cell, N);
+                take(s.off, N);
+                if (h->kinds_mask & kPairMask)
+                    take(s.rf, N);
+                if (h->kinds_mask & (kQuadMask | 1 << kRBGLinear))
+                    take(s.q3, N);
+                if (h->kinds_mask & kQuadMask) {
+                    take(s.qn, N);
+                    take(s.qab, N);
+                    take(s.qc, N);
+                }
+            } else {
+                take(h->u64[b], N);
+                if (b == 0 || h->f64s.K > 1) {
+                    take(h->f64[b].ncache, N);
+                    for (int c = 0; c < h->n_cache; ++c)
+                        take(h->f64[b].c[c], N);
+                }
             }
-        }
-    } else {
-        free_split(h);
-        if (h->u64[0])
-            return QEW_OK;
-        QEW_CUDA(h, dev_alloc(&h->u64[0], N), "allocating the FP64 state");
-        QEW_CUDA(h, dev_alloc(&h->u64[1], N), "allocating the FP64 state");
-        for (int b = 0; b < (h->f64s.K > 1 ? 2 : 1); ++b) {
-            QEW_CUDA(h, dev_alloc(&h->f64[b].ncache, N), "allocating the FP64 cache cells");
-            for (int c = 0; c < h->n_cache; ++c)
-                QEW_CUDA(h, dev_alloc(&h->f64[b].c[c], N), "allocating the FP64 disorder cache");
+            if (pass == 0) {
+                QEW_CUDA(h, dev_alloc(&h->slab[b], size), "allocating the state");
+                base = h->slab[b];
+            }
         }
     }
     return QEW_OK;
