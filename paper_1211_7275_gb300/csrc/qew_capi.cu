@@ -115,6 +115,7 @@ struct qew_ctx {
     int cur = 0;
     F64State f64[2] = {};            // disorder caches: two copies when a launch takes several steps
     F64Shape f64s = {256, 4, 1, false};
+    bool f64_in_place = false;       // no memory for the second copy
     TileDesc* d_ftiles = nullptr;    // tiles of the FP64 step kernel
     int32_t n_ftiles = 0;
     double* u64[2] = {nullptr, nullptr};
@@ -261,7 +262,7 @@ void free_all(qew_ctx* h)
 
 // The state's arrays, one allocation per buffer (a handle made and freed per trial paid for up to
 // fourteen).
-int alloc_state(qew_ctx* h)
+int alloc_buffers(qew_ctx* h)
 {
     const bool split = h->precision == QEW_FP32_SPLIT;
     if (split ? h->sp[0].cell != nullptr : h->u64[0] != nullptr)
@@ -307,6 +308,23 @@ int alloc_state(qew_ctx* h)
         }
     }
     return QEW_OK;
+}
+
+int build_layout(qew_ctx* h);
+
+int alloc_state(qew_ctx* h)
+{
+    int rc = alloc_buffers(h);
+    if (rc == QEW_ENOMEM && h->precision == QEW_FP64 && h->f64s.K > 1) {
+        // several steps per launch take a second copy of the disorder caches: without room for it, one
+        // step per launch updates them in place
+        free_state(h);
+        h->f64_in_place = true;
+        rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = alloc_buffers(h);
+    }
+    return rc;
 }
 
 // Sites per lane that chains of `kind` use under the requested S: the largest width the kind
@@ -395,7 +413,7 @@ int build_layout(qew_ctx* h)
     std::vector<int32_t> first(h->n_chains), step_first(h->n_chains);
     int64_t n_list[kNumKinds] = {}, n_step_list[kNumKinds] = {};
     std::vector<TileDesc> blocks, ftiles;
-    h->f64s = f64_shape(h->n_sites);
+    h->f64s = f64_shape(h->f64_in_place ? INT64_MAX : h->n_sites);
     h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
                  h->f64s.look ? ((h->kinds_mask >> kRBGLinear & 1) ? 4 : 3) : 2;
     h->h_chains.assign(h->n_chains, ChainDesc{});
