@@ -512,7 +512,7 @@ def main() -> None:
             S = relax.structure_factor()
             times.append(1e3 * (time.perf_counter() - t0))
         sq = {"ms_first": times[0], "ms": times[1], "modes": int(S.size), "chains": int(wl["n_chains"]),
-              "includes": "state to FP64 rows, batched real-to-complex cuFFT, mean |u_q|^2 over chains, "
+              "includes": "state to FP64 rows, batched half-length cuFFT, mean |u_q|^2 over chains, "
                           "copy to host (work area allocated and freed in the call); the first call also "
                           "builds the plan"}
 

@@ -15,7 +15,7 @@
 //   bond (Case 3)          one, and the node above them.  79% of the moves at the threshold go back
 //                          where the site came from (it chatters across a jump of its force): they flip
 //                          one bit of a lane mask and draw nothing (0.05 instead of 0.17 draws per
-//                          site-update; 4 x 2^25 sites 4.7e11 -> 8.9e11 su/s late in a relaxation)
+//                          site-update; 736-site tiles late in a relaxation 4.7e11 -> 9.3e11 su/s)
 //   cubic random bond      the coefficients A, B, C of F_p + f = A + d (B + d C) over the cell (from the
 //                          spline nodes V(n-1 .. n+2)) and the nodes V(n), V(n+1), V(n+2) that a move up
 //                          reuses
@@ -31,16 +31,17 @@
 // What bounds it, and the shape of a step.  The kernel is bound by instruction issue and by the
 // latency of a step's serial parts at 12 to 16 warps per SM, not by memory.  So
 //   - the update loop works on register pairs with packed FP32 instructions (half the issue slots; the
-//     FP32 pipe itself is as busy as with scalar ones, 59% at 992-site tiles) and reads both sites'
+//     FP32 pipe itself is as busy as with scalar ones, 61% at 992-site tiles) and reads both sites'
 //     cache values with one 16-byte load;
 //   - renormalisation is branch-free (n += floor(d), d -= floor(d)), with the floor by two packed
 //     additions: as a conversion it took the conversion pipe 7.6 clocks per site;
 //   - a funnel shift per site collects what moved how far (MoveCodes), so that moves by one cell need
 //     no copy of the cells for the consumers; a rare path takes moves by more;
 //   - requests are queued by ballots, without a prefix sum, and the Philox values evaluated 32 lanes at
-//     a time, straight into the shared-memory cache of the requesting sites.
-// 16 x 2^20 random-field chains at the threshold, 992-site tiles, K = 32: 0.94 -> 0.62 warp-instructions
-// per site-update, 75% -> 67% issue, 560 -> 425 us per launch (1.03e12 -> 1.26e12 su/s).
+//     a time, straight into the shared-memory cache of the requesting sites;
+//   - what is the same in all lanes is kept in uniform registers (see uniform()).
+// 16 x 2^20 random-field chains at the threshold, 992-site tiles, K = 32: 0.94 -> 0.59 warp-instructions
+// per site-update, 75% -> 67% issue, 560 -> 400 us per launch (1.03e12 -> 1.33e12 su/s).
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -300,9 +301,10 @@ struct Force {
 __device__ __forceinline__ int mask_top(unsigned m) { return 31 - __clz(m); }
 __device__ __forceinline__ int mask_top(unsigned long long m) { return 63 - __clzll(static_cast<long long>(m)); }
 
-// Registers per thread allowed to the kernel, the fastest measured of 80 .. 184 on each shape.  Both
-// ways cost: at 992-site random-field tiles 120 (and the same 16 warps per SM) instead of 128 lost 3%,
-// 96 lost 23%, and 144 (14 warps) lost 8%; Case 3 redraws less often and gains 1 to 6% from 144 and 168.
+// Registers per thread allowed to the kernel, the fastest measured of 96 .. 184 on each shape.  Both
+// ways cost: at 992-site random-field tiles 120 (and the same 16 warps per SM) instead of 128 lost 2%,
+// 104 with a shorter queue and 18 warps also 2%, 160 (12 warps) 9%; Case 3 at 736-site tiles gains 4%
+// from 144 over 112.
 template <int KIND, int S>
 struct MaxRegs {
     static constexpr int value = quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
