@@ -672,6 +672,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             if (!obs_marked) {
                 // the sums are relative to the cell, at this step, of the site `len` before the tile
                 obs_ref = cell_at<KIND, S>(s_cell, pad - a.obs_len[obs], lane, N0, c, cT, upper);
+                __syncwarp();   // read by every lane before the slot is written again
                 obs_marked = true;
             } else {
                 observe_tile<KIND, S>(a, f, tile, wt.chain, obs, obs_ref, owned, pad, N0, lane, c, d, cT, dT, upper, s_cell,
