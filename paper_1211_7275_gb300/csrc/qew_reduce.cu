@@ -102,10 +102,10 @@ __global__ void bounded_wait_probe(int32_t* error, int limit)
 }
 
 // Range guard of the FP32-split state, run at every observation: the fused kernel carries cells as
-// exact small floats relative to a cell of its tile window and (compact layout) decodes a step's
-// move from 16 bits of the cell.  Both hold while neighbouring cells differ by less than 2^12: then
+// exact small floats relative to a cell of its tile window and takes the floor of a displacement by an
+// addition that holds below 2^22.  Both hold while neighbouring cells differ by less than 2^12: then
 // no Euler step moves a site by 2^15 cells (the Euler map grows a neighbour difference by at most
-// 2 dt max|F_p| per step) and a 992-site window spans less than 2^22 cells.  A violation sets the
+// 2 dt max|F_p| per step) and a 1248-site window spans less than 2^23 cells.  A violation sets the
 // error flag to 2.  Blocks (x, y) stride over the sites of chains y, y + gridDim.y, ...; the
 // chain descriptor is read once per chain, so a thread's loads are independent of one another.
 __global__ void __launch_bounds__(256) split_range_guard_kernel(const ChainDesc* chains, int32_t n_chains,
