@@ -521,6 +521,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             if constexpr (T::has_quad || KIND == kRBGLinear)
                 tma_load_1d(s_top, a.in.q3 + p0, TW * 4, bar);
         }
+        __syncwarp();   // no lane polls the barrier before it is initialised
     }
     int32_t cells[T::early_cells ? S : 1];
     if constexpr (T::early_cells) {
