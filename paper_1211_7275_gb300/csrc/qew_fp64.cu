@@ -438,11 +438,12 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                 const unsigned h = static_cast<unsigned>(__double2hiint(d));
                 if (h >= 0x3FF00000u) {   // not in [0, 1)
                     // (1, 2) is one cell up and (-1, 0) one down, exactly; else the floor decides (u - floor
-                    // may have rounded up to 1)
+                    // may have rounded up to 1; -0 is in cell 0)
+                    const bool edge = (h == 0x3FF00000u || h == 0x80000000u) && __double2loint(d) == 0;   // 1 or -0
                     int32_t move;
-                    if (h < 0x40000000u && !(h == 0x3FF00000u && __double2loint(d) == 0))
+                    if (h < 0x40000000u && !edge)
                         move = 1;
-                    else if (h >= 0x80000000u && h < 0xBFF00000u)
+                    else if (h >= 0x80000000u && h < 0xBFF00000u && !edge)
                         move = -1;
                     else
                         move = __double2int_rd(u) - n;
