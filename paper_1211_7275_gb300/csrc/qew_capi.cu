@@ -119,6 +119,7 @@ struct qew_ctx {
     TileDesc* d_ftiles = nullptr;    // tiles of the FP64 step kernel
     int32_t n_ftiles = 0;
     double* u64[2] = {nullptr, nullptr};
+    bool layout_made = false;        // tile lists, descriptors and partials as the fields above say
 
     double* d_shift = nullptr;
     double* d_partial = nullptr;
@@ -260,12 +261,27 @@ void free_all(qew_ctx* h)
     h->sq_plan_made = false;
 }
 
+// Whether the state's buffers are there, both of them.
+bool have_buffers(const qew_ctx* h)
+{
+    return h->precision == QEW_FP32_SPLIT ? h->sp[0].cell && h->sp[1].cell : h->u64[0] && h->u64[1];
+}
+
+// An allocation that failed in an earlier call leaves a handle without some of the arrays that the
+// kernels write: every call that launches one on the state asks here first.
+int check_arrays(qew_ctx* h)
+{
+    if (!h->layout_made || !have_buffers(h))
+        return fail(h, QEW_ESTATE, "an earlier call on this handle ran out of memory: repeat it, or destroy the handle");
+    return QEW_OK;
+}
+
 // The state's arrays, one allocation per buffer (a handle made and freed per trial paid for up to
-// fourteen).
+// fourteen).  Both buffers or, after a failure, none.
 int alloc_buffers(qew_ctx* h)
 {
     const bool split = h->precision == QEW_FP32_SPLIT;
-    if (split ? h->sp[0].cell != nullptr : h->u64[0] != nullptr)
+    if (have_buffers(h))
         return QEW_OK;
     free_state(h);
     const size_t N = static_cast<size_t>(split ? h->n_state : h->n_sites);
@@ -302,7 +318,11 @@ int alloc_buffers(qew_ctx* h)
                 }
             }
             if (pass == 0) {
-                QEW_CUDA(h, dev_alloc(&h->slab[b], size), "allocating the state");
+                const cudaError_t e = dev_alloc(&h->slab[b], size);
+                if (e != cudaSuccess) {
+                    free_state(h);
+                    return cuda_fail(h, e, "allocating the state");
+                }
                 base = h->slab[b];
             }
         }
@@ -318,7 +338,6 @@ int alloc_state(qew_ctx* h)
     if (rc == QEW_ENOMEM && h->precision == QEW_FP64 && h->f64s.K > 1) {
         // several steps per launch take a second copy of the disorder caches: without room for it, one
         // step per launch updates them in place
-        free_state(h);
         h->f64_in_place = true;
         rc = build_layout(h);
         if (rc == QEW_OK)
@@ -403,6 +422,7 @@ void step_shape(qew_ctx* h)
 int build_layout(qew_ctx* h)
 {
     drop_graph(h);   // captured launches point at the descriptors rebuilt here
+    h->layout_made = false;
     step_shape(h);
     const bool own_step = h->precision == QEW_FP32_SPLIT && !h->shape_given;
     for (int k = 0; k < kNumKinds; ++k) {
@@ -523,6 +543,7 @@ int build_layout(qew_ctx* h)
         QEW_CUDA(h, dev_alloc(&h->d_partial, need), "allocating partial sums");
         h->partial_cap = need;
     }
+    h->layout_made = true;
     return QEW_OK;
 }
 
@@ -530,6 +551,8 @@ int build_layout(qew_ctx* h)
 // reference shifts to `shift0`.
 int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shift0)
 {
+    if (int rc = check_arrays(h))
+        return rc;
     h->cur = 0;
     h->step = 0;
     if (h->precision == QEW_FP32_SPLIT) {
@@ -1042,6 +1065,7 @@ int ensure_obs(qew_ctx* h, size_t n)
         drop_graph(h);   // the captured copy-out targets these buffers
     if (n > h->obs_cap) {
         dev_free(h->d_obs);
+        h->obs_cap = 0;
         QEW_CUDA(h, dev_alloc(&h->d_obs, n), "allocating observation buffer");
         h->obs_cap = n;
     }
@@ -1049,6 +1073,7 @@ int ensure_obs(qew_ctx* h, size_t n)
         if (h->h_obs)
             cudaFreeHost(h->h_obs);
         h->h_obs = nullptr;
+        h->h_obs_cap = 0;
         QEW_CUDA(h, cudaMallocHost(reinterpret_cast<void**>(&h->h_obs), n * sizeof(double)),
                  "allocating pinned observation buffer");
         h->h_obs_cap = n;
@@ -1065,6 +1090,8 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
         return QEW_OK;
     if (!steps)
         return fail(h, QEW_EINVAL, "steps must not be NULL");
+    if (int rc = check_arrays(h))
+        return rc;
     if (steps[0] < h->step)
         return fail(h, QEW_EINVAL, "steps[0] = " + std::to_string(steps[0]) + " lies before the current step " +
                                        std::to_string(h->step));
@@ -1188,6 +1215,8 @@ int get_state_impl(qew_ctx* h, double* u_out, int32_t* cells_out, int64_t* step_
         *step_out = h->step;
     if (!u_out && !cells_out)
         return QEW_OK;
+    if (int rc = check_arrays(h))
+        return rc;
     double* d_u = nullptr;
     int32_t* d_c = nullptr;
     int rc = QEW_OK;
@@ -1287,6 +1316,10 @@ int qew_set_precision(qew_handle h, int32_t precision)
     if (h->step != 0)
         return fail(h, QEW_ESTATE, "precision can only change before the first step");
     DeviceGuard g(h->device);
+    if (h->f64_in_place) {   // caches of the one-step shape: there may be room for the others by now
+        free_state(h);
+        h->f64_in_place = false;
+    }
     h->precision = precision;
     int rc = build_layout(h);
     if (rc == QEW_OK)
@@ -1389,6 +1422,8 @@ int qew_advance(qew_handle h, int64_t n_steps)
         return rc;
     if (n_steps < 0)
         return fail(h, QEW_EINVAL, "n_steps must be >= 0");
+    if (int rc = check_arrays(h))
+        return rc;
     DeviceGuard g(h->device);
     const int64_t target = h->step + n_steps;
     int rc = run_through(h, &target, 1, nullptr);
@@ -1459,6 +1494,8 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
             return fail(h, QEW_EINVAL, "the structure factor needs chains of one length");
     if (n_modes < 1 || n_modes > L / 2)
         return fail(h, QEW_EINVAL, "n_modes must lie in [1, L/2]");
+    if (int rc = check_arrays(h))
+        return rc;
     DeviceGuard g(h->device);
     const int32_t Li = static_cast<int32_t>(L);
     const int32_t B = h->n_chains;
