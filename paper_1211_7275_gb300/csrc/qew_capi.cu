@@ -100,12 +100,12 @@ struct qew_ctx {
 
     std::vector<ChainDesc> h_chains;
     ChainDesc* d_chains = nullptr;
-    WarpTile* d_tiles[kNumKinds] = {};
-    int32_t n_tiles[kNumKinds] = {};
-    int32_t tile_base[kNumKinds] = {};
+    WarpTile* d_tiles[kNumClasses] = {};   // per class of chains
+    int32_t n_tiles[kNumClasses] = {};
+    int32_t tile_base[kNumClasses] = {};
     int32_t w_own[kNumKinds] = {};   // sites a warp tile owns, per disorder kind
-    WarpTile* d_step_tiles[kNumKinds] = {};   // the same of the step shape, where it is another one
-    int32_t n_step_tiles[kNumKinds] = {};
+    WarpTile* d_step_tiles[kNumClasses] = {};   // the same of the step shape, where it is another one
+    int32_t n_step_tiles[kNumClasses] = {};
     int32_t step_w_own[kNumKinds] = {};
     TileDesc* d_btiles = nullptr;
     int32_t n_btiles = 0;
@@ -132,7 +132,7 @@ struct qew_ctx {
     size_t h_obs_cap = 0;
 
     // statistics (qew_enable_stats / qew_get_stats)
-    int64_t sites_of_kind[kNumKinds] = {};
+    int64_t sites_of_class[kNumClasses] = {};
     bool stats_on = false;
     int64_t n_launches = 0;
     int64_t n_fused = 0;
@@ -242,7 +242,7 @@ void free_all(qew_ctx* h)
     dev_free(h->d_error);
     free_state(h);
     dev_free(h->d_chains);
-    for (int k = 0; k < kNumKinds; ++k) {
+    for (int k = 0; k < kNumClasses; ++k) {
         dev_free(h->d_tiles[k]);
         dev_free(h->d_step_tiles[k]);
     }
@@ -429,9 +429,9 @@ int build_layout(qew_ctx* h)
         h->w_own[k] = 32 * kind_S(k, h->S) - 2 * h->K;
         h->step_w_own[k] = 32 * kind_S(k, h->step_S) - 2 * h->step_K;
     }
-    // first tile of each chain in its kind's list, and the lists' lengths, in both shapes
+    // first tile of each chain in its class's list, and the lists' lengths, in both shapes
     std::vector<int32_t> first(h->n_chains), step_first(h->n_chains);
-    int64_t n_list[kNumKinds] = {}, n_step_list[kNumKinds] = {};
+    int64_t n_list[kNumClasses] = {}, n_step_list[kNumClasses] = {};
     std::vector<TileDesc> blocks, ftiles;
     h->f64s = f64_shape(h->f64_in_place ? INT64_MAX : h->n_sites);
     h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
@@ -450,12 +450,13 @@ int build_layout(qew_ctx* h)
         for (int64_t st = 0; st < d.L; st += kBlockTile)   // 64-bit: L may reach 2^31 - 1
             blocks.push_back(TileDesc{c, static_cast<int32_t>(st)});
         if (h->precision == QEW_FP32_SPLIT) {
-            first[c] = static_cast<int32_t>(n_list[d.kind]);
+            const int cls = chain_class(d.kind, d.f32);
+            first[c] = static_cast<int32_t>(n_list[cls]);
             d.ntiles = static_cast<int32_t>((int64_t(d.L) + h->w_own[d.kind] - 1) / h->w_own[d.kind]);
-            n_list[d.kind] += d.ntiles;
+            n_list[cls] += d.ntiles;
             if (own_step) {
-                step_first[c] = static_cast<int32_t>(n_step_list[d.kind]);
-                n_step_list[d.kind] += (int64_t(d.L) + h->step_w_own[d.kind] - 1) / h->step_w_own[d.kind];
+                step_first[c] = static_cast<int32_t>(n_step_list[cls]);
+                n_step_list[cls] += (int64_t(d.L) + h->step_w_own[d.kind] - 1) / h->step_w_own[d.kind];
             }
         } else {
             for (int64_t st = 0; st < d.L; st += h->f64s.w_own())
@@ -465,13 +466,13 @@ int build_layout(qew_ctx* h)
     size_t slots = 0;
     if (h->precision == QEW_FP32_SPLIT) {
         int32_t base = 0;
-        for (int k = 0; k < kNumKinds; ++k) {
+        for (int k = 0; k < kNumClasses; ++k) {
             h->tile_base[k] = base;
             h->n_tiles[k] = static_cast<int32_t>(n_list[k]);
             base += h->n_tiles[k];
         }
         for (int32_t c = 0; c < h->n_chains; ++c) {
-            h->h_chains[c].tile0 = h->tile_base[h->kind[c]] + first[c];
+            h->h_chains[c].tile0 = h->tile_base[chain_class(h->kind[c], h->h_chains[c].f32)] + first[c];
         }
         slots = static_cast<size_t>(base);
     } else {
@@ -483,11 +484,11 @@ int build_layout(qew_ctx* h)
             b += nb;
         }
         slots = static_cast<size_t>(b);
-        for (int k = 0; k < kNumKinds; ++k)
+        for (int k = 0; k < kNumClasses; ++k)
             h->n_tiles[k] = 0;
     }
     dev_free(h->d_chains);
-    for (int k = 0; k < kNumKinds; ++k) {
+    for (int k = 0; k < kNumClasses; ++k) {
         dev_free(h->d_tiles[k]);
         dev_free(h->d_step_tiles[k]);
     }
@@ -502,16 +503,17 @@ int build_layout(qew_ctx* h)
         std::vector<int32_t> both(first);
         both.insert(both.end(), step_first.begin(), step_first.end());
         cudaError_t e = cudaMemcpyAsync(d_first, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
-        for (int k = 0; k < kNumKinds; ++k) {
+        for (int k = 0; k < kNumClasses; ++k) {
+            const int kind = class_kind(k);
             h->n_step_tiles[k] = static_cast<int32_t>(n_step_list[k]);
             if (e == cudaSuccess && n_list[k] > 0)
                 e = dev_alloc(&h->d_tiles[k], n_list[k]);
             if (e == cudaSuccess && n_list[k] > 0)
-                e = split_tiles(h->d_chains, h->n_chains, k, h->w_own[k], d_first, h->d_tiles[k], h->stream);
+                e = split_tiles(h->d_chains, h->n_chains, k, h->w_own[kind], d_first, h->d_tiles[k], h->stream);
             if (e == cudaSuccess && n_step_list[k] > 0)
                 e = dev_alloc(&h->d_step_tiles[k], n_step_list[k]);
             if (e == cudaSuccess && n_step_list[k] > 0)
-                e = split_tiles(h->d_chains, h->n_chains, k, h->step_w_own[k], d_first + h->n_chains, h->d_step_tiles[k], h->stream);
+                e = split_tiles(h->d_chains, h->n_chains, k, h->step_w_own[kind], d_first + h->n_chains, h->d_step_tiles[k], h->stream);
         }
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(h->stream);
@@ -570,7 +572,7 @@ int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shif
     return QEW_OK;
 }
 
-// One launch of the fused kernel (per disorder kind): K steps and the observations among them.
+// One launch of the fused kernel (per class of chains): K steps and the observations among them.
 struct Segment {
     int K = 0;
     bool step_only = false;        // in the step shape (no observations)
@@ -580,13 +582,15 @@ struct Segment {
     int32_t index[kMaxLaunchObs];  // and its place in the call's list
 };
 
-SplitLaunch split_args(qew_ctx* h, int kind, const Segment& s, SplitState in, SplitState out)
+SplitLaunch split_args(qew_ctx* h, int cls, const Segment& s, SplitState in, SplitState out)
 {
     SplitLaunch a{};
     const bool other = s.step_only && !h->shape_given;
-    a.tiles = other ? h->d_step_tiles[kind] : h->d_tiles[kind];
-    a.n_tiles = other ? h->n_step_tiles[kind] : h->n_tiles[kind];
-    a.tile_base = h->tile_base[kind];
+    const int kind = class_kind(cls);
+    a.tiles = other ? h->d_step_tiles[cls] : h->d_tiles[cls];
+    a.n_tiles = other ? h->n_step_tiles[cls] : h->n_tiles[cls];
+    a.neg = cls != kind;
+    a.tile_base = h->tile_base[cls];
     a.in = in;
     a.out = out;
     a.K = s.K;
@@ -622,7 +626,7 @@ int next_event(qew_ctx* h, cudaEvent_t* ev)
 
 int launch_split_all(qew_ctx* h, const Segment& s, SplitState in, SplitState out)
 {
-    for (int k = 0; k < kNumKinds; ++k) {
+    for (int k = 0; k < kNumClasses; ++k) {
         if (h->n_tiles[k] == 0)
             continue;
         const SplitLaunch a = split_args(h, k, s, in, out);
@@ -635,13 +639,13 @@ int launch_split_all(qew_ctx* h, const Segment& s, SplitState in, SplitState out
                 return rc;
             QEW_CUDA(h, cudaEventRecord(e0, h->stream), "recording a timing event");
         }
-        QEW_CUDA(h, split_step(k, kind_S(k, s.step_only ? h->step_S : h->S), s.step_only ? h->step_tpc : h->tpc, a, h->stream),
+        QEW_CUDA(h, split_step(class_kind(k), kind_S(class_kind(k), s.step_only ? h->step_S : h->S), s.step_only ? h->step_tpc : h->tpc, a, h->stream),
                  "launching the fused step kernel");
         if (h->stats_on)
             QEW_CUDA(h, cudaEventRecord(e1, h->stream), "recording a timing event");
         h->n_launches += 1;
         h->n_fused += 1;
-        h->n_site_updates += h->sites_of_kind[k] * s.K;
+        h->n_site_updates += h->sites_of_class[k] * s.K;
     }
     return QEW_OK;
 }
@@ -1001,7 +1005,7 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
             h->soffset[c] = h->n_state;
             h->n_state += (L[c] + 31) & ~int64_t(31);
             h->kinds_mask |= 1 << kind[c];
-            h->sites_of_kind[kind[c]] += L[c];
+            h->sites_of_class[chain_class(kind[c], static_cast<float>(f[c]))] += L[c];
         }
         h->n_sites = off;
         h->dt = dt;

@@ -29,6 +29,12 @@ __host__ __device__ constexpr bool quad_kind(int k) { return k == kRB || k == kR
 constexpr int kPairMask = (1 << kRF) | (1 << kRBGLinear);
 constexpr int kQuadMask = (1 << kRB) | (1 << kRBGCubic);
 
+// Chains that the fused kernel takes in one launch: of one kind and, where there is disorder, one sign of
+// the drive.
+constexpr int kNumClasses = 2 * kNumKinds;
+__host__ __device__ constexpr int chain_class(int kind, float f) { return kind + (f < 0.0f && kind != kNone ? kNumKinds : 0); }
+constexpr int class_kind(int c) { return c % kNumKinds; }
+
 constexpr uint32_t kTagRF = 0u;   // counter word 3 of random-field force values
 constexpr uint32_t kTagRB = 1u;   // counter word 3 of uniform random-bond potential values
 constexpr uint32_t kTagRBG = 2u;  // counter word 3 of Gaussian random-bond potential values (Cases 1, 3)

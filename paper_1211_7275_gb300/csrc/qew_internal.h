@@ -39,8 +39,9 @@ struct F64State {
 constexpr int kMaxLaunchObs = 24;
 
 struct SplitLaunch {
-    const WarpTile* tiles;   // tiles of one disorder kind
+    const WarpTile* tiles;   // tiles of one class
     int32_t n_tiles;
+    int32_t neg;             // the class's drives are negative
     int32_t tile_base;       // partial-sum slot of tiles[0]
     SplitState in, out;
     int32_t K;               // Euler steps in this launch (0: observe only)
@@ -59,8 +60,8 @@ struct SplitLaunch {
     PhiloxKeys keys;         // round keys of `seed`
 };
 
-// Writes the warp tiles of the chains of one kind: chain c's, w_own sites each, at tiles[first[c]].
-cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int kind, int32_t w_own, const int32_t* first,
+// Writes the warp tiles of the chains of one class: chain c's, w_own sites each, at tiles[first[c]].
+cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int cls, int32_t w_own, const int32_t* first,
                         WarpTile* tiles, cudaStream_t stream);
 // Sites per lane of the fused kernel for each supported tile width (tile_w = 32 * S).
 bool split_supported(int kind, int sites_per_lane);

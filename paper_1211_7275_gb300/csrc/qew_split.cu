@@ -12,7 +12,7 @@
 //   random field           the nodes of the cell, (R(n) + f, R(n+1) + f): the drive f is folded in, so
 //                          F_p + f is one subtraction and one FMA
 //   linear-spline random   the forces F_p = G - G(+1) of two neighbouring cells, of which the site is in
-//   bond (Case 3)          one, and the node above them.  79% of the moves at the threshold go back
+//   bond (Case 3)          one, and the node beyond them in the direction of the drive (above for f >= 0).  79% of the moves at the threshold go back
 //                          where the site came from (it chatters across a jump of its force): they flip
 //                          one bit of a lane mask and draw nothing (0.05 instead of 0.17 draws per
 //                          site-update; 736-site tiles late in a relaxation 4.7e11 -> 9.3e11 su/s)
@@ -131,7 +131,7 @@ __device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c)
 //           the last site): one conflict-free 16-byte load per pair and step.  (first, second) value
 //           of both sites: RF (R(n) + f, R(n+1) + f); linear-spline random bond the force F_p of
 //           two neighbouring cells; cubic kinds the coefficients (A, B), and C in rows of float2
-//   nodes   what only a cell move reads, linear: the node above the two cells (linear-spline random
+//   nodes   what only a cell move reads, linear: the node beyond the two cells (linear-spline random
 //           bond), V(n), V(n+1) and V(n+2) (cubic kinds)
 //   queue   kQueue requests of 2 B
 // RF takes 12 B per site and so 16 warps per SM at 992-site tiles, the register limit.
@@ -153,8 +153,8 @@ struct Tile {
     static constexpr int nodes = top + (has_quad || KIND == kRBGLinear ? 4 * TW : 0);   // one float2 per site
     static constexpr int queue = nodes + (has_quad ? 8 * TW : 0);
     static constexpr int kQueue = 256;
-    // whether a single cell downwards is an ordinary move (else it takes the rare path of far moves):
-    // a fifth of the linear-spline random bond's moves, a few in 10^4 of the other kinds'
+    // whether a single cell against the drive is an ordinary move (else it takes the rare path of far
+    // moves): a fifth of the linear-spline random bond's moves, a few in 10^4 of the other kinds'
     static constexpr bool kDown = KIND == kRBGLinear || KIND == kRBGCubic;
     // KIND none stages offsets and cells side by side: it has no cache to make room for
     static constexpr int slot2 = has_cache ? slot : 4 * TW;
@@ -212,14 +212,18 @@ struct MoveCodes {
     __device__ __forceinline__ void put_last(float fl) { last = __float_as_uint(fl); }
 
     // moved: sites that changed cell; down: of those, by one cell downwards (when nothing is far);
-    // far: some site of the lane moved two cells or more, or, unless DOWN, moved downwards
-    template <bool DOWN>
+    // far: some site of the lane moved two cells or more, or, unless DOWN, moved against the drive
+    // (downwards, with NEG upwards)
+    template <bool DOWN, bool NEG>
     __device__ __forceinline__ void masks(typename Moves<S>::mask& moved, typename Moves<S>::mask& down, bool& far) const
     {
         using mask = typename Moves<S>::mask;
-        constexpr unsigned kFar = DOWN ? kOnes << 1 : (kOnes << 1) | (kOnes << 2);
+        constexpr unsigned kFar = (DOWN || NEG) ? kOnes << 1 : (kOnes << 1) | (kOnes << 2);
+        auto against = [](unsigned c) -> unsigned { return (!DOWN && NEG) ? c & ~(c >> 2) & kOnes : 0u; };
         unsigned mv[2] = {0u, 0u}, dn[2] = {0u, 0u};
-        unsigned any = last & (DOWN ? 0x40000000u : 0xC0000000u);
+        unsigned any = last & ((DOWN || NEG) ? 0x40000000u : 0xC0000000u);
+        if (!DOWN && NEG)
+            any |= static_cast<unsigned>(static_cast<int>(last) > 0);
 #pragma unroll
         for (int w = 0; w < 3; ++w) {
             const int n = (H - w + 2) / 3;       // codes in word w
@@ -230,14 +234,14 @@ struct MoveCodes {
                 const unsigned c[2] = {b[w], a[w]};
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
-                    any |= c[r] & kFar;
+                    any |= (c[r] & kFar) | against(c[r]);
                     mv[r] |= ((c[r] | (c[r] >> 1)) & kOnes) << sh;
                     if (DOWN)
                         dn[r] |= ((c[r] >> 2) & kOnes) << sh;
                 }
             } else {
                 const unsigned c = (a[w] << Moves<S>::D) + b[w];
-                any |= c & kFar;
+                any |= (c & kFar) | against(c);
                 mv[0] += ((c | (c >> 1)) & kOnes) << sh;
                 if (DOWN)
                     dn[0] += ((c >> 2) & kOnes) << sh;
@@ -456,7 +460,12 @@ __device__ __forceinline__ unsigned uniform(unsigned v)
 
 // OBS: whether the launch observes at all.  The observation code in the step loop takes registers
 // from it, so that launches without any (nearly all of a long relaxation's) have a kernel of their own.
-template <int KIND, int S, bool OBS>
+// NEG: chains of a negative drive, whose ordinary moves go downwards.  As one kernel for both signs, by a
+// branch or by selecting at the moves, the random field lost 3% to 12%; without the distinction 16 x 2^20
+// sites at -f_c, -3 f_c took, ms per 512 steps (random field, uniform cubic, Case 3; at f_c, 3 f_c):
+// 10.8 27.2 (8.2 18.5), 16.0 39.9 (10.7 21.0), 18.0 74.6 (12.2 39.3); with it 8.4 18.9,
+// 12.3 26.7, 12.2 39.3.
+template <int KIND, int S, bool OBS, bool NEG>
 __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLaunch a)
 {
     using T = Tile<KIND, S>;
@@ -721,7 +730,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
         mask moved = 0, down = 0;
         bool lane_far = false;
         if (T::has_cache || a.crossings)
-            codes.template masks<T::kDown>(moved, down, lane_far);
+            codes.template masks<T::kDown, NEG>(moved, down, lane_far);
         if (a.crossings)
             n_cross += __reduce_add_sync(kFull, static_cast<unsigned>(mask_popc(moved)));
         if constexpr (T::has_cache) {
@@ -735,21 +744,23 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                     req = (up & upper) | (down & ~upper);
                     upper = (upper | up) & ~down;
                 } else {
-                    upper &= ~moved;   // redrawn with the new cell as the lower one
+                    // redrawn with the new cell as the lower one (NEG: upper one)
+                    upper = NEG ? (upper | moved) : (upper & ~moved);
                 }
             }
             if (far) {
                 // some site moved two cells or more: the lanes leave their new cells in the slot,
                 // and every site that moved redraws all of its nodes
+                const int32_t base = (KIND == kRBGLinear && NEG) ? N0 - 1 : N0;
 #pragma unroll
                 for (int p = 0; p < H; ++p) {
                     if (KIND != kRBGLinear || (moved & M::first(p)))
-                        s_cell[lane * S + p] = N0 + __float2int_rn(lo(c[p]));
+                        s_cell[lane * S + p] = base + __float2int_rn(lo(c[p]));
                     if (KIND != kRBGLinear || (moved & M::second(p)))
-                        s_cell[lane * S + H + p] = N0 + __float2int_rn(hi(c[p]));
+                        s_cell[lane * S + H + p] = base + __float2int_rn(hi(c[p]));
                 }
                 if (KIND != kRBGLinear || (moved & M::last))
-                    s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
+                    s_cell[lane * S + 2 * H] = base + __float2int_rn(cT);
             }
             // Queue the requests, one per lane and pass: a lane's slot is its rank in the ballot of the
             // lanes that still have one (no prefix sum; three or four passes empty the masks)
@@ -781,40 +792,45 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                             const int t = first ? b - M::D : b;            // row of the pair
                             const int x = src * S + (H - 1 - t) + (first ? 0 : H) + (t == H ? S : 0);
                             float* row = s_loop + 4 * (32 * t + src) + (first ? 0 : 1);
-                            const int step = far ? 0 : (T::kDown && (e & 64)) ? -1 : 1;
+                            const int step = far ? 0 : (T::kDown ? (e & 64) != 0 : NEG) ? -1 : 1;
                             const int32_t i = contiguous ? static_cast<int32_t>(wstart) + x
                                                          : site_index(wstart, x, contiguous, L);
                             const int32_t slot = s_cell[x];
                             if constexpr (KIND == kRF) {
-                                // an up move keeps R(n) and draws R(n+1); a far move draws both
+                                // a move keeps the node between the two cells and draws the one beyond
+                                // the new cell; a far move draws both
+                                constexpr int beyond = NEG ? 0 : 1;
                                 const int32_t nn = slot + step;
-                                const float old = row[2];
-                                const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 1, period), f);
-                                row[0] = far ? pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn, period), f) : old;
-                                row[2] = v;
+                                const float old = row[2 * beyond];
+                                const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn + beyond, period), f);
+                                row[2 - 2 * beyond] = far ? pair_node_f32<KIND>(a.keys, s, i, wrap_node(nn + 1 - beyond, period), f) : old;
+                                row[2 * beyond] = v;
                                 if (!far)
                                     s_cell[x] = nn;
                             } else if constexpr (KIND == kRBGLinear) {
-                                // the pair of cells moves up (n = slot + 2 is the new upper cell, one new
-                                // node), down or, after a far move, starts anew at n = slot: three nodes
-                                const bool up = step > 0;
-                                const int32_t base_n = up ? slot + 3 : slot + step;
-                                const int trips = up ? 1 : 3;
-                                float g0 = row[2], g1 = 0.0f, prev = s_top[x];
+                                // The pair of cells moves on by one, in the direction of the drive with one
+                                // new node beyond it.  Against it, or anew after a far move (then the slot
+                                // holds the new lower cell), its three nodes are drawn in the drive's order.
+                                constexpr int behind = NEG ? 2 : 0, front = NEG ? 0 : 2;   // F_p of the two cells, in that order
+                                const bool ahead = NEG ? step < 0 : step > 0;
+                                const int32_t lower = slot + step;
+                                const int32_t n0 = lower + (ahead != NEG ? 2 : 0);
+                                const int trips = ahead ? 1 : 3;
+                                float gb = row[front], gf = 0.0f, prev = s_top[x];
 #pragma unroll 1
                                 for (int r = 0; r < trips; ++r) {
-                                    const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(base_n + r, period), f);
-                                    const float g = prev - v;   // F_p of the cell between the two nodes
-                                    if (!up && r == 1)
-                                        g0 = g;
+                                    const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(n0 + (NEG ? -r : r), period), f);
+                                    const float g = NEG ? v - prev : prev - v;   // F_p of the cell between the two nodes
+                                    if (!ahead && r == 1)
+                                        gb = g;
                                     else
-                                        g1 = g;
+                                        gf = g;
                                     prev = v;
                                 }
-                                row[0] = g0;
-                                row[2] = g1;
+                                row[behind] = gb;
+                                row[front] = gf;
                                 s_top[x] = prev;
-                                s_cell[x] = slot + step;
+                                s_cell[x] = lower;
                             } else {
                                 // The spline over the new cell n needs V(n-1 .. n+2).  The cache holds
                                 // V, V(+1), V(+2) of the old cell: an up move draws V(n+2), a down move
@@ -974,11 +990,11 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
     }
 }
 
-template <int KIND, int S, bool OBS>
+template <int KIND, int S, bool OBS, bool NEG>
 cudaError_t launch_split_as(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
 {
     const size_t smem = static_cast<size_t>(tiles_per_cta) * Tile<KIND, S>::bytes;
-    auto kern = split_step_kernel<KIND, S, OBS>;
+    auto kern = split_step_kernel<KIND, S, OBS, NEG>;
     // raise the dynamic shared-memory limit of this kernel on this device to the largest shape in
     // use; under a lock, so that two threads raising it at once cannot leave the smaller value
     static std::mutex s_mu;
@@ -1008,14 +1024,19 @@ cudaError_t launch_split_as(int tiles_per_cta, const SplitLaunch& a, cudaStream_
 template <int KIND, int S>
 cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
 {
-    return a.n_obs > 0 ? launch_split_as<KIND, S, true>(tiles_per_cta, a, st) : launch_split_as<KIND, S, false>(tiles_per_cta, a, st);
+    if constexpr (KIND != kNone)
+        if (a.neg)
+            return a.n_obs > 0 ? launch_split_as<KIND, S, true, true>(tiles_per_cta, a, st) :
+                                 launch_split_as<KIND, S, false, true>(tiles_per_cta, a, st);
+    return a.n_obs > 0 ? launch_split_as<KIND, S, true, false>(tiles_per_cta, a, st) :
+                         launch_split_as<KIND, S, false, false>(tiles_per_cta, a, st);
 }
 
-__global__ void split_tiles_kernel(const ChainDesc* chains, int kind, int32_t w_own, const int32_t* first, WarpTile* tiles)
+__global__ void split_tiles_kernel(const ChainDesc* chains, int cls, int32_t w_own, const int32_t* first, WarpTile* tiles)
 {
     const int32_t c = blockIdx.x;
     const ChainDesc ch = chains[c];
-    if (ch.kind != kind)
+    if (chain_class(ch.kind, ch.f32) != cls)
         return;
     WarpTile* mine = tiles + first[c];
     for (int64_t k = threadIdx.x; k * w_own < ch.L; k += blockDim.x) {
@@ -1058,9 +1079,14 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
             st.rf[p] = make_float2(rf_plus_f32(seed, ch.s, i, m1, ch.f32), rf_plus_f32(seed, ch.s, i, m2, ch.f32));
         else if (ch.kind == kRBGLinear)
         {
-            const float g1 = rbg_f32(seed, ch.s, i, m1), g2 = rbg_f32(seed, ch.s, i, m2), g3 = rbg_f32(seed, ch.s, i, m3);
-            st.rf[p] = make_float2(g1 - g2, g2 - g3);
+            // the site's cell and the next one in the direction of the drive; the sign of the offset says
+            // that the site is in the upper one
+            const bool neg = ch.f32 < 0.0f;
+            const float g1 = rbg_f32(seed, ch.s, i, m1), g2 = rbg_f32(seed, ch.s, i, m2);
+            const float g3 = rbg_f32(seed, ch.s, i, neg ? m0 : m3);
+            st.rf[p] = neg ? make_float2(g3 - g1, g1 - g2) : make_float2(g1 - g2, g2 - g3);
             st.q3[p] = g3;
+            st.off[p] = neg ? -d : d;
         }
         else if (ch.kind == kRB || ch.kind == kRBGCubic) {
             const bool uni = ch.kind == kRB;
@@ -1164,10 +1190,10 @@ cudaError_t split_step(int kind, int S, int tiles_per_cta, const SplitLaunch& a,
     return cudaErrorInvalidValue;
 }
 
-cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int kind, int32_t w_own, const int32_t* first,
+cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int cls, int32_t w_own, const int32_t* first,
                         WarpTile* tiles, cudaStream_t stream)
 {
-    split_tiles_kernel<<<n_chains, 256, 0, stream>>>(chains, kind, w_own, first, tiles);
+    split_tiles_kernel<<<n_chains, 256, 0, stream>>>(chains, cls, w_own, first, tiles);
     return cudaGetLastError();
 }
 
