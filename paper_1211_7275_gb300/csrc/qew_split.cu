@@ -260,6 +260,28 @@ struct MoveCodes {
         }
         far = any != 0;
     }
+    // The sites that moved two cells or more.
+    __device__ __forceinline__ typename Moves<S>::mask far_ones() const
+    {
+        unsigned m[2] = {0u, 0u};
+#pragma unroll
+        for (int w = 0; w < 3; ++w) {
+            const int n = (H - w + 2) / 3;
+            if (n <= 0)
+                continue;
+            const int sh = H - 1 - w - 3 * (n - 1);
+            if constexpr (Moves<S>::wide) {
+                m[0] |= ((b[w] >> 1) & kOnes) << sh;
+                m[1] |= ((a[w] >> 1) & kOnes) << sh;
+            } else {
+                m[0] += ((((a[w] << Moves<S>::D) + b[w]) >> 1) & kOnes) << sh;
+            }
+        }
+        typename Moves<S>::mask r = m[0];
+        if constexpr (Moves<S>::wide)
+            r |= static_cast<typename Moves<S>::mask>(m[1]) << 32;
+        return (last & 0x40000000u) ? r | Moves<S>::last : r;
+    }
 };
 
 // F_p + f of a lane's pair (row t = H - 1 - p) and of its last site, at offsets d, from shared memory.
@@ -312,11 +334,11 @@ __device__ __forceinline__ int mask_top(unsigned long long m) { return 63 - __cl
 // Registers per thread allowed to the kernel, the fastest measured of 96 .. 184 on each shape.  Both
 // ways cost: at 992-site random-field tiles 120 (and the same 16 warps per SM) instead of 128 lost 2%,
 // 104 with a shorter queue and 18 warps also 2%, 160 (12 warps) 9%; Case 3 at 736-site tiles gains 4%
-// from 144 over 112.
+// from 144 over 112, at 480-site tiles 2% from 104 over 112.
 template <int KIND, int S>
 struct MaxRegs {
     static constexpr int value = quad_kind(KIND) ? (S <= 8 ? 80 : 128) :
-                                 KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 112 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
+                                 KIND == kRBGLinear ? (S <= 8 ? 64 : S <= 16 ? 104 : S <= 23 ? 144 : S <= 31 ? 168 : 184) :
                                                       (S <= 8 ? 64 : S <= 16 ? 112 : S <= 31 ? 128 : 160);
 };
 
@@ -464,7 +486,7 @@ __device__ __forceinline__ unsigned uniform(unsigned v)
 // branch or by selecting at the moves, the random field lost 3% to 12%; without the distinction 16 x 2^20
 // sites at -f_c, -3 f_c took, ms per 512 steps (random field, uniform cubic, Case 3; at f_c, 3 f_c):
 // 10.8 27.2 (8.2 18.5), 16.0 39.9 (10.7 21.0), 18.0 74.6 (12.2 39.3); with it 8.4 18.9,
-// 12.3 26.7, 12.2 39.3.
+// 12.3 26.7, 12.1 37.6.
 template <int KIND, int S, bool OBS, bool NEG>
 __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLaunch a)
 {
@@ -735,32 +757,61 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             n_cross += __reduce_add_sync(kFull, static_cast<unsigned>(mask_popc(moved)));
         if constexpr (T::has_cache) {
             const bool far = __any_sync(kFull, lane_far);
-            // requests: sites whose cache has to change
-            mask req = moved;
+            mask req = moved;   // requests: sites whose cache has to change
             if constexpr (KIND == kRBGLinear) {
+                if (far) {
+                    // Some site moved two cells or more.  Each lane redraws those of its own, the new cell
+                    // being the lower (NEG: upper) of the two in the cache, and the others take the queue.
+                    // 16 x 2^20 sites driven at 8 f_c, where most steps of a tile have a far move, ms per 512
+                    // steps: 147 with all moved sites redrawn, 117 with the far ones in the queue among
+                    // the others, 110 so.
+                    const mask m = codes.far_ones();
+                    const int32_t base = NEG ? N0 - 1 : N0;
+#pragma unroll
+                    for (int p = 0; p < H; ++p) {
+                        if (m & M::first(p))
+                            s_cell[lane * S + p] = base + __float2int_rn(lo(c[p]));
+                        if (m & M::second(p))
+                            s_cell[lane * S + H + p] = base + __float2int_rn(hi(c[p]));
+                    }
+                    if (m & M::last)
+                        s_cell[lane * S + 2 * H] = base + __float2int_rn(cT);
+                    moved &= ~m;
+                    upper = NEG ? (upper | m) : (upper & ~m);
+                    for (mask left = m; left != 0;) {
+                        const int b = mask_top(left);
+                        left = mask_drop(left, b);
+                        const bool first = b >= M::D;
+                        const int t = first ? b - M::D : b;
+                        const int x = lane * S + (H - 1 - t) + (first ? 0 : H) + (t == H ? S : 0);
+                        float* row = s_loop + 4 * (32 * t + lane) + (first ? 0 : 1);
+                        const int32_t i = contiguous ? static_cast<int32_t>(wstart) + x : site_index(wstart, x, contiguous, L);
+                        const int32_t lower = s_cell[x];
+                        float g = 0.0f, prev = 0.0f;
+#pragma unroll 1
+                        for (int r = 0; r < 3; ++r) {
+                            const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(lower + (NEG ? 2 - r : r), period), f);
+                            row[NEG ? 2 : 0] = g;
+                            g = NEG ? v - prev : prev - v;
+                            prev = v;
+                        }
+                        row[NEG ? 0 : 2] = g;
+                        s_top[x] = prev;
+                    }
+                }
                 down &= moved;
                 const mask up = moved & ~down;
-                if (!far) {
-                    req = (up & upper) | (down & ~upper);
-                    upper = (upper | up) & ~down;
-                } else {
-                    // redrawn with the new cell as the lower one (NEG: upper one)
-                    upper = NEG ? (upper | moved) : (upper & ~moved);
-                }
-            }
-            if (far) {
-                // some site moved two cells or more: the lanes leave their new cells in the slot,
-                // and every site that moved redraws all of its nodes
-                const int32_t base = (KIND == kRBGLinear && NEG) ? N0 - 1 : N0;
+                req = (up & upper) | (down & ~upper);
+                upper = (upper | up) & ~down;
+            } else if (far) {
+                // the lanes leave their new cells in the slot, and every site that moved redraws all of
+                // its nodes
 #pragma unroll
                 for (int p = 0; p < H; ++p) {
-                    if (KIND != kRBGLinear || (moved & M::first(p)))
-                        s_cell[lane * S + p] = base + __float2int_rn(lo(c[p]));
-                    if (KIND != kRBGLinear || (moved & M::second(p)))
-                        s_cell[lane * S + H + p] = base + __float2int_rn(hi(c[p]));
+                    s_cell[lane * S + p] = N0 + __float2int_rn(lo(c[p]));
+                    s_cell[lane * S + H + p] = N0 + __float2int_rn(hi(c[p]));
                 }
-                if (KIND != kRBGLinear || (moved & M::last))
-                    s_cell[lane * S + 2 * H] = base + __float2int_rn(cT);
+                s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
             }
             // Queue the requests, one per lane and pass: a lane's slot is its rank in the ballot of the
             // lanes that still have one (no prefix sum; three or four passes empty the masks)
@@ -792,7 +843,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                             const int t = first ? b - M::D : b;            // row of the pair
                             const int x = src * S + (H - 1 - t) + (first ? 0 : H) + (t == H ? S : 0);
                             float* row = s_loop + 4 * (32 * t + src) + (first ? 0 : 1);
-                            const int step = far ? 0 : (T::kDown ? (e & 64) != 0 : NEG) ? -1 : 1;
+                            const int step = KIND != kRBGLinear && far ? 0 : (T::kDown ? (e & 64) != 0 : NEG) ? -1 : 1;
                             const int32_t i = contiguous ? static_cast<int32_t>(wstart) + x
                                                          : site_index(wstart, x, contiguous, L);
                             const int32_t slot = s_cell[x];
@@ -809,23 +860,25 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                                     s_cell[x] = nn;
                             } else if constexpr (KIND == kRBGLinear) {
                                 // The pair of cells moves on by one, in the direction of the drive with one
-                                // new node beyond it.  Against it, or anew after a far move (then the slot
-                                // holds the new lower cell), its three nodes are drawn in the drive's order.
+                                // new node beyond it, against it with its three nodes drawn anew, in the
+                                // drive's order.  (The first draw inside the loop as well: 2% slower at f_c,
+                                // 5% at 3 f_c.)
                                 constexpr int behind = NEG ? 2 : 0, front = NEG ? 0 : 2;   // F_p of the two cells, in that order
                                 const bool ahead = NEG ? step < 0 : step > 0;
                                 const int32_t lower = slot + step;
                                 const int32_t n0 = lower + (ahead != NEG ? 2 : 0);
-                                const int trips = ahead ? 1 : 3;
-                                float gb = row[front], gf = 0.0f, prev = s_top[x];
+                                float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(n0, period), f);
+                                float gb = row[front], prev = s_top[x];
+                                float gf = NEG ? v - prev : prev - v;   // F_p of the cell between the two nodes
+                                prev = v;
+                                if (!ahead) {
 #pragma unroll 1
-                                for (int r = 0; r < trips; ++r) {
-                                    const float v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(n0 + (NEG ? -r : r), period), f);
-                                    const float g = NEG ? v - prev : prev - v;   // F_p of the cell between the two nodes
-                                    if (!ahead && r == 1)
-                                        gb = g;
-                                    else
-                                        gf = g;
-                                    prev = v;
+                                    for (int r = 1; r < 3; ++r) {
+                                        v = pair_node_f32<KIND>(a.keys, s, i, wrap_node(n0 + (NEG ? -r : r), period), f);
+                                        gb = gf;
+                                        gf = NEG ? v - prev : prev - v;
+                                        prev = v;
+                                    }
                                 }
                                 row[behind] = gb;
                                 row[front] = gf;
