@@ -45,16 +45,15 @@ __device__ __forceinline__ double node_f64(uint64_t seed, uint32_t s, int32_t i,
 //   - a small batch is spread over many SMs in small tiles and advanced K steps per launch.
 // Loop values of a site: RF R(n), R(n+1); linear spline F; cubic ca, 2 b, 3 c of the force.
 // Cached nodes of a site in cell n: V(n + lo) .. V(n + lo + n_nodes - 1), the force's.  With look-ahead
-// there are n_look of them, from V(n + lo_look): the one a move up will need, and for the linear spline,
-// whose sites move up and down across a node, also the one a move down will; the force's start at
-// `used`.
+// there are n_look of them, from V(n + lo - used): the one that a move in the direction of the drive will
+// need (neg: a negative drive's, downwards), and for the linear spline, whose sites move up and down
+// across a node, both; the force's start at `used`.
 template <int KIND>
 struct F64Site {
     static constexpr int n_nodes = pair_kind(KIND) ? 2 : quad_kind(KIND) ? 4 : 0;
     static constexpr int lo = quad_kind(KIND) ? -1 : 0;
     static constexpr int n_look = KIND == kRBGLinear ? 4 : n_nodes > 0 ? n_nodes + 1 : 0;
-    static constexpr int lo_look = KIND == kRBGLinear ? -1 : lo;
-    static constexpr int used = lo - lo_look;
+    static __host__ __device__ constexpr int used(bool neg) { return KIND == kRBGLinear || (neg && n_nodes > 0) ? 1 : 0; }
     static constexpr int n_loop = KIND == kRF ? 2 : KIND == kRBGLinear ? 1 : quad_kind(KIND) ? 3 : 0;
 };
 // A node that has not been drawn.
@@ -261,6 +260,7 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
     const TileDesc td = a.tiles[blockIdx.x];
     const ChainDesc ch = a.chains[td.chain];
     const double c = a.shift[td.chain];
+    const int used = a.look ? V::used(ch.f64 < 0.0) : 0;
     double tF = 0.0, t1 = 0.0, t2 = 0.0;
     for (int x = threadIdx.x; x < a.w_tile; x += blockDim.x) {
         const int32_t i = td.start + x;
@@ -272,7 +272,7 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
             double nodes[V::n_nodes], v[V::n_loop];
 #pragma unroll
             for (int k = 0; k < V::n_nodes; ++k)
-                nodes[k] = a.st.c[a.look ? V::used + k : k][p];
+                nodes[k] = a.st.c[used + k][p];
             loop_values<KIND>(nodes, v);
             tF = __dadd_rn(tF, force_f64<KIND>(__dsub_rn(u, static_cast<double>(a.st.ncache[p])), v));
         }
@@ -310,11 +310,11 @@ __device__ __forceinline__ void f64_observe_body(const F64Launch& a, double (*re
 
 template <int KIND>
 __device__ __forceinline__ void init_nodes(const F64State& st, int64_t p, uint64_t seed, uint32_t s, int32_t i, int32_t n,
-                                           int32_t period, int look)
+                                           int32_t period, int look, bool neg)
 {
     using V = F64Site<KIND>;
     const int count = look ? V::n_look : V::n_nodes;
-    const int lo = look ? V::lo_look : V::lo;
+    const int lo = V::lo - (look ? V::used(neg) : 0);
 #pragma unroll 1
     for (int c = 0; c < count; ++c)
         st.c[c][p] = node_f64<KIND>(seed, s, i, n + lo + c, period);
@@ -336,13 +336,13 @@ __global__ void f64_init_kernel(const ChainDesc* chains, const TileDesc* tiles, 
         st.ncache[p] = n;
         const int32_t M = ch.period;
         if (ch.kind == kRF)
-            init_nodes<kRF>(st, p, seed, ch.s, i, n, M, look);
+            init_nodes<kRF>(st, p, seed, ch.s, i, n, M, look, ch.f64 < 0.0);
         else if (ch.kind == kRBGLinear)
-            init_nodes<kRBGLinear>(st, p, seed, ch.s, i, n, M, look);
+            init_nodes<kRBGLinear>(st, p, seed, ch.s, i, n, M, look, ch.f64 < 0.0);
         else if (ch.kind == kRB)
-            init_nodes<kRB>(st, p, seed, ch.s, i, n, M, look);
+            init_nodes<kRB>(st, p, seed, ch.s, i, n, M, look, ch.f64 < 0.0);
         else if (ch.kind == kRBGCubic)
-            init_nodes<kRBGCubic>(st, p, seed, ch.s, i, n, M, look);
+            init_nodes<kRBGCubic>(st, p, seed, ch.s, i, n, M, look, ch.f64 < 0.0);
     }
 }
 
@@ -365,11 +365,11 @@ __global__ void f64_cells_kernel(const ChainDesc* chains, const TileDesc* tiles,
 // listed sites' missing nodes are drawn together once a warp of them has gathered, or at once when a
 // force needs one.  One 1024-site RF chain at f = 1, us per step: 22.7 with one launch per step on one
 // SM, 3.3 in small tiles with every draw in its own step, 1.47 so, 1.38 with the draws split in two.
-template <int KIND>
+template <int KIND, bool NEG>
 __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc td, const ChainDesc& ch, double* smem)
 {
     using V = F64Site<KIND>;
-    constexpr int NN = V::n_nodes, NX = V::n_look, NL = V::n_loop;
+    constexpr int NN = V::n_nodes, NX = V::n_look, NL = V::n_loop, used = V::used(NEG), lo_look = V::lo - used;
     const int NT = blockDim.x;
     // (the linear spline's sites keep listing outer nodes that they may never use: us per step at 1024,
     // 2^16 and 2^18 sites 2.84, 5.43, 19.4 gathering a quarter as for the others, 2.29, 5.12, 18.2 so)
@@ -412,7 +412,7 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                 s_p[c * NT + x] = nodes[c];
                 missing = missing || no_node(nodes[c]);
             }
-            loop_values<KIND>(nodes + V::used, v);
+            loop_values<KIND>(nodes + used, v);
         }
     }
     if (x < 2) {   // the window's outer neighbours, as they are at the start
@@ -464,11 +464,11 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
 #pragma unroll
                         for (int c = 0; c < NX; ++c) {
                             s_p[c * NT + x] = nodes[c];
-                            if (c >= V::used && c < V::used + NN)
+                            if (c >= used && c < used + NN)
                                 urgent = urgent || no_node(nodes[c]);
                         }
                         s_cell[x] = n;
-                        loop_values<KIND>(nodes + V::used, v);
+                        loop_values<KIND>(nodes + used, v);
                         if (slot < 0) {
                             slot = atomicAdd(&s_count[turn], 1);
                             s_q[slot] = static_cast<uint16_t>(x);
@@ -484,11 +484,16 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                 const int half = NT / 2;
                 const bool split = KIND != kRB && listed <= half;
                 const int part = split && x >= half ? 1 : 0;
+                // Of a site that lost all of its force's nodes (a move of several cells) only those are drawn,
+                // and it is listed again for the others: a steep line, whose sites move so in every step,
+                // would never use them (2^20 sites, 16 steps: random field 8.6 ms, Case 3 10.5, with all drawn).
+                auto lost = [&](int at) { return no_node(s_p[used * NT + at]) && no_node(s_p[(used + NN - 1) * NT + at]); };
                 for (int q = x - part * half; q < listed; q += NT) {
                     const int at = s_q[q];
-                    const int32_t i = site_of(at), base = s_cell[at] + V::lo_look;
+                    const int32_t i = site_of(at), base = s_cell[at] + lo_look;
+                    const bool all = !lost(at);
 #pragma unroll 1
-                    for (int c = 0; c < NX; ++c) {
+                    for (int c = all ? 0 : used; c < (all ? NX : used + NN); ++c) {
                         if (!no_node(s_p[c * NT + at]))
                             continue;
                         if (!split) {
@@ -503,9 +508,10 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                     __syncthreads();
                     if (x < listed) {
                         const int at = s_q[x];
+                        const bool all = !lost(at);
 #pragma unroll
                         for (int c = 0; c < NX; ++c)
-                            if (no_node(s_p[c * NT + at]))
+                            if ((all || (c >= used && c < used + NN)) && no_node(s_p[c * NT + at]))
                                 s_p[c * NT + at] = __dmul_rn(s_f[c * half + x], s_f[(NX + c) * half + x]);
                     }
                 }
@@ -518,8 +524,12 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                     double nodes[NN];
 #pragma unroll
                     for (int c = 0; c < NN; ++c)
-                        nodes[c] = s_p[(V::used + c) * NT + x];
+                        nodes[c] = s_p[(used + c) * NT + x];
                     loop_values<KIND>(nodes, v);
+                    if (no_node(s_p[(NEG ? 0 : NX - 1) * NT + x])) {
+                        slot = atomicAdd(&s_count[turn], 1);
+                        s_q[slot] = static_cast<uint16_t>(x);
+                    }
                 }
             }
         } else {
@@ -552,16 +562,17 @@ __global__ void __launch_bounds__(256, 1) f64_look_any(F64Step a)
     extern __shared__ double smem_f64[];
     const TileDesc td = a.tiles[blockIdx.x];
     const ChainDesc ch = a.chains[td.chain];
+    const bool neg = ch.f64 < 0.0;
     if (ch.kind == kRF)
-        f64_look_body<kRF>(a, td, ch, smem_f64);
+        neg ? f64_look_body<kRF, true>(a, td, ch, smem_f64) : f64_look_body<kRF, false>(a, td, ch, smem_f64);
     else if (ch.kind == kRB)
-        f64_look_body<kRB>(a, td, ch, smem_f64);
+        neg ? f64_look_body<kRB, true>(a, td, ch, smem_f64) : f64_look_body<kRB, false>(a, td, ch, smem_f64);
     else if (ch.kind == kRBGLinear)
-        f64_look_body<kRBGLinear>(a, td, ch, smem_f64);
+        f64_look_body<kRBGLinear, false>(a, td, ch, smem_f64);
     else if (ch.kind == kRBGCubic)
-        f64_look_body<kRBGCubic>(a, td, ch, smem_f64);
+        neg ? f64_look_body<kRBGCubic, true>(a, td, ch, smem_f64) : f64_look_body<kRBGCubic, false>(a, td, ch, smem_f64);
     else
-        f64_look_body<kNone>(a, td, ch, smem_f64);
+        f64_look_body<kNone, false>(a, td, ch, smem_f64);
 }
 
 // Tiles of mixed kinds share one launch: the kind is uniform per block (one chain).
