@@ -433,7 +433,7 @@ int build_layout(qew_ctx* h)
     std::vector<int32_t> first(h->n_chains), step_first(h->n_chains);
     int64_t n_list[kNumClasses] = {}, n_step_list[kNumClasses] = {};
     std::vector<TileDesc> blocks, ftiles;
-    h->f64s = f64_shape(h->f64_in_place ? INT64_MAX : h->n_sites);
+    h->f64s = f64_shape(h->f64_in_place ? INT64_MAX : h->n_sites, h->kinds_mask);
     h->n_cache = (h->kinds_mask & kQuadMask) ? (h->f64s.look ? 5 : 4) :
                  h->f64s.look ? ((h->kinds_mask >> kRBGLinear & 1) ? 4 : 3) : 2;
     h->h_chains.assign(h->n_chains, ChainDesc{});

@@ -625,16 +625,19 @@ size_t f64_step_smem(const F64Shape& s, int n_nodes)
 //   2^24 sites    128 threads of 4 sites x 8 steps without look-ahead 651 (Case 3 on half of them 367, against
 //                 550 with look-ahead, whose outer nodes its moves up and down keep discarding), 4 steps 669
 // Few sites are latency: 65 clocks per FP64 operation whatever a block does, so small tiles on as many
-// SMs as there are.  Then it is FP64 throughput, where a wide halo is work done twice.  One step per launch
+// SMs as there are.  Then it is FP64 throughput, where a wide halo is work done twice.  A batch of uniform
+// random-bond chains alone, whose draws are a few operations, gives up look-ahead at 3 x 2^18 sites (us per
+// step with it and without, at f_c, 3 f_c and from a steep line: 2^19 sites 33.3 34.0, 39.4 35.8, 80 54; 2^20
+// sites 63.2 59.0, 75.2 69.1, 151 98).  One step per launch
 // updates the cached disorder in place and takes no second copy of it, for batches beyond 2^29 sites (30 GB
 // with it for RF, 47 GB for the cubic kinds); at 2^27 RF sites it runs 9.1 ms per step against 5.2.
-F64Shape f64_shape(int64_t n_sites)
+F64Shape f64_shape(int64_t n_sites, int kinds_mask)
 {
     if (n_sites <= (int64_t(1) << 13))
         return F64Shape{128, 1, 32, true};
     if (n_sites <= (int64_t(1) << 15))
         return F64Shape{128, 1, 16, true};
-    if (n_sites <= (int64_t(1) << 20))
+    if (n_sites <= (int64_t(1) << 20) && (kinds_mask != 1 << kRB || n_sites < (int64_t(3) << 18)))
         return F64Shape{256, 1, 16, true};
     if (n_sites <= (int64_t(1) << 29))
         return F64Shape{128, 4, 8, false};

@@ -111,7 +111,7 @@ struct F64Step {
     uint64_t seed;
 };
 
-F64Shape f64_shape(int64_t n_sites);
+F64Shape f64_shape(int64_t n_sites, int kinds_mask);
 size_t f64_step_smem(const F64Shape& s, int n_nodes);
 cudaError_t f64_step(const F64Step& a, const F64Shape& s, cudaStream_t st);
 cudaError_t f64_observe(const F64Launch& a, cudaStream_t st);

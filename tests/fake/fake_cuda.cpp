@@ -223,7 +223,7 @@ cudaError_t split_range_guard(const ChainDesc* chains, int32_t, int64_t, const i
 }
 
 // (only the shapes that matter here: look-ahead, several steps, one step in place)
-F64Shape f64_shape(int64_t n_sites)
+F64Shape f64_shape(int64_t n_sites, int)
 {
     if (n_sites <= (int64_t(1) << 20))
         return F64Shape{256, 1, 16, true};

@@ -34,6 +34,11 @@ def test_driven_lines(kind, drive, L):
     both(L, f, kind, 0.7 * np.random.default_rng(3).standard_normal(sum(L)))
 
 
+@pytest.mark.parametrize("L", [(3 << 18) - 1, 3 << 18])
+def test_where_the_uniform_random_bond_changes_shape(L):
+    both([L], np.array([F[RB]]), RB, 0.7 * np.random.default_rng(3).standard_normal(L))
+
+
 @pytest.mark.parametrize("kind", [RF, RB, RBG_LINEAR, RBG_CUBIC])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 @pytest.mark.parametrize("L", [777, 9000, 60000])
