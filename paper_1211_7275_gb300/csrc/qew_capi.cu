@@ -96,6 +96,7 @@ struct qew_ctx {
     // Shape of the launches without observations; the same unless the handle has its default shape
     // (step_shape).  The sums of an observation follow the tiles of the shape above.
     int step_S = 23, step_K = 16, step_tpc = 2;
+    int short_K = 0;   // launches of up to so many steps take the shape above all the same
     bool shape_given = false;
 
     std::vector<ChainDesc> h_chains;
@@ -415,6 +416,72 @@ void step_shape(qew_ctx* h)
         if (h->kinds_mask & kQuadMask)
             h->step_tpc = 1;
     }
+    // A chain shorter than a tile takes a whole window all the same: narrower tiles where the windows
+    // then add up to less (each launch about four steps' worth of staging).  20000 chains, ms per 256
+    // steps: uniform cubic, 100 sites 3.3 by the number of sites alone (480 x 48), 2.2 so (224 x 48);
+    // 192 sites 3.3, 2.6; random field, 300 sites 5.5, 3.1.  The line at 3/4 leaves longer chains alone,
+    // where the best alternative has 1.0 of the windows.
+    if (*std::min_element(h->L.begin(), h->L.end()) < 4096) {
+        auto cost = [&](int S, int K) {
+            double windows = 0.0;
+            for (int32_t c = 0; c < h->n_chains; ++c) {
+                const int s = kind_S(h->kind[c], S);
+                windows += static_cast<double>((h->L[c] + 32 * s - 2 * K - 1) / (32 * s - 2 * K)) * s;
+            }
+            return windows * (K + 4) / K;
+        };
+        double best = 0.75 * cost(h->step_S, h->step_K);
+        const int limit = h->step_S;
+        const int shapes[][2] = {{7, 48}, {7, 32}, {7, 16}, {15, 48}, {15, 32}, {23, 48}};
+        for (const auto& s : shapes) {
+            const double c = s[0] <= limit ? cost(s[0], s[1]) : best;
+            if (c < best) {
+                best = c;
+                h->step_S = s[0];
+                h->step_K = s[1];
+            }
+        }
+    }
+}
+
+// Waves of the launches in a shape, in units of a site per lane, and their tiles.
+struct ShapeLoad {
+    int64_t tiles = 0, waves = 0, cost = 0;
+};
+ShapeLoad shape_load(const qew_ctx* h, int S, const int32_t* n_tiles)
+{
+    constexpr int kSMs = 152;
+    ShapeLoad r;
+    for (int k = 0; k < kNumClasses; ++k) {
+        if (n_tiles[k] == 0)
+            continue;
+        const int s = kind_S(class_kind(k), S);
+        const int64_t resident = static_cast<int64_t>(kSMs) * split_warps_per_sm(class_kind(k), s);
+        const int64_t w = (n_tiles[k] + resident - 1) / resident;
+        r.tiles += n_tiles[k];
+        r.waves = std::max(r.waves, w);
+        r.cost += w * s;
+    }
+    return r;
+}
+
+// Launches of a few steps are staging more than steps, which the deep tiles of the step shape only make
+// longer: they take the observing shape where its waves are cheaper.  Up to its K steps if there is one
+// wave, or the tiles are as wide and not more; else one or two.  us per call of qew_advance of 1 and 16
+// steps in the step shape and in the observing one, 4 chains: random field 2^20 sites 27.8 26.8, 41.9
+// 37.2, 2^21 sites (the observing shape has two waves, the step shape one) 30.6 31.5, 47.2 55.6; Case 3
+// 2^20 sites 32.3 28.8, 48.6 44.8; uniform cubic 2^18 sites 20.6 16.5, 28.9 26.5, 2^20 sites 24.5 20.8,
+// 44.1 46.0.
+void short_launches(qew_ctx* h)
+{
+    h->short_K = 0;
+    if (h->shape_given || h->precision != QEW_FP32_SPLIT || h->n_sites < (int64_t(1) << 17))
+        return;
+    const ShapeLoad obs = shape_load(h, h->S, h->n_tiles), step = shape_load(h, h->step_S, h->n_step_tiles);
+    if (min_kind_S(h, h->S) == min_kind_S(h, h->step_S) && obs.cost == step.cost && obs.tiles <= step.tiles)
+        h->short_K = h->K;
+    else if (5 * obs.cost < 4 * step.cost)
+        h->short_K = obs.waves == 1 ? h->K : 2;
 }
 
 // Tile lists for the current precision and launch shape; uploads chain descriptors and sizes
@@ -467,6 +534,7 @@ int build_layout(qew_ctx* h)
     if (h->precision == QEW_FP32_SPLIT) {
         int32_t base = 0;
         for (int k = 0; k < kNumClasses; ++k) {
+            h->n_step_tiles[k] = static_cast<int32_t>(n_step_list[k]);
             h->tile_base[k] = base;
             h->n_tiles[k] = static_cast<int32_t>(n_list[k]);
             base += h->n_tiles[k];
@@ -505,7 +573,6 @@ int build_layout(qew_ctx* h)
         cudaError_t e = cudaMemcpyAsync(d_first, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
         for (int k = 0; k < kNumClasses; ++k) {
             const int kind = class_kind(k);
-            h->n_step_tiles[k] = static_cast<int32_t>(n_step_list[k]);
             if (e == cudaSuccess && n_list[k] > 0)
                 e = dev_alloc(&h->d_tiles[k], n_list[k]);
             if (e == cudaSuccess && n_list[k] > 0)
@@ -533,6 +600,7 @@ int build_layout(qew_ctx* h)
                                     h->stream),
                  "uploading FP64 tiles");
     }
+    short_launches(h);
     // room for the partials of as many observations as 256 MB hold
     h->partial_slots = slots;
     h->launch_obs = 1;
@@ -771,7 +839,7 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
         while (n > 0) {
             const int64_t launches = (n + h->step_K - 1) / h->step_K;
             Segment b;
-            b.step_only = true;
+            b.step_only = n > h->short_K;
             b.K = static_cast<int>(std::min<int64_t>({n, h->step_K, ((n + launches - 1) / launches + 3) & ~int64_t(3)}));
             const int e = run_segment(h, b, nullptr);
             if (e != QEW_OK)

@@ -66,6 +66,7 @@ cudaError_t split_tiles(const ChainDesc* chains, int32_t n_chains, int cls, int3
 // Sites per lane of the fused kernel for each supported tile width (tile_w = 32 * S).
 bool split_supported(int kind, int sites_per_lane);
 size_t split_smem_bytes(int kind, int sites_per_lane, int tiles_per_cta);
+int split_warps_per_sm(int kind, int sites_per_lane);   // resident warps (tiles), by registers and shared memory
 cudaError_t split_step(int kind, int sites_per_lane, int tiles_per_cta, const SplitLaunch& a, cudaStream_t st);
 cudaError_t split_init(const ChainDesc* chains, int32_t n_chains, const TileDesc* tiles, int32_t n_tiles,
                        int32_t w_tile, SplitState st, uint64_t seed, int any_rb, const double* u_in,

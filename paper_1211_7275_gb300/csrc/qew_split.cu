@@ -42,6 +42,7 @@
 //   - what is the same in all lanes is kept in uniform registers (see uniform()).
 // 16 x 2^20 random-field chains at the threshold, 992-site tiles, K = 32: 0.94 -> 0.59 warp-instructions
 // per site-update, 75% -> 67% issue, 560 -> 400 us per launch (1.03e12 -> 1.33e12 su/s).
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -1202,6 +1203,24 @@ size_t split_smem_bytes(int kind, int S, int tiles_per_cta)
     const int b = kind == kRF ? tile_bytes<kRF>(S) : kind == kRBGLinear ? tile_bytes<kRBGLinear>(S) :
                   kind == kNone ? tile_bytes<kNone>(S) : tile_bytes<kRB>(S);
     return static_cast<size_t>(tiles_per_cta) * b;
+}
+
+template <int KIND>
+constexpr int max_regs(int S)
+{
+    switch (S) {
+    case 7: return MaxRegs<KIND, 7>::value;
+    case 15: return MaxRegs<KIND, 15>::value;
+    case 23: return MaxRegs<KIND, 23>::value;
+    case 31: return MaxRegs<KIND, 31>::value;
+    default: return MaxRegs<KIND, 39>::value;
+    }
+}
+
+int split_warps_per_sm(int kind, int S)
+{
+    const int regs = kind == kRBGLinear ? max_regs<kRBGLinear>(S) : quad_kind(kind) ? max_regs<kRB>(S) : max_regs<kRF>(S);
+    return std::min(65536 / (32 * regs), static_cast<int>(227 * 1024 / split_smem_bytes(kind, S, 1)));
 }
 
 cudaError_t split_step(int kind, int S, int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)

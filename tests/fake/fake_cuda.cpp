@@ -178,6 +178,7 @@ cudaError_t split_tiles(const ChainDesc* chains, int32_t, int, int32_t, const in
 }
 bool split_supported(int kind, int S) { return S == 7 || S == 15 || (!quad_kind(kind) && (S == 23 || S == 31 || (S == 39 && kind != kNone))); }
 size_t split_smem_bytes(int, int S, int tiles) { return static_cast<size_t>(tiles) * 32 * S * 28; }
+int split_warps_per_sm(int, int) { return 16; }
 cudaError_t split_step(int kind, int, int, const SplitLaunch& a, cudaStream_t s)
 {
     on_stream(s);
