@@ -444,9 +444,9 @@ void step_shape(qew_ctx* h)
     }
 }
 
-// Waves of the launches in a shape, in units of a site per lane, and their tiles.
+// Tiles of the launches in a shape, their windows and their waves, in sites per lane.
 struct ShapeLoad {
-    int64_t tiles = 0, waves = 0, cost = 0;
+    int64_t tiles = 0, windows = 0, waves = 0, cost = 0;
 };
 ShapeLoad shape_load(const qew_ctx* h, int S, const int32_t* n_tiles)
 {
@@ -459,6 +459,7 @@ ShapeLoad shape_load(const qew_ctx* h, int S, const int32_t* n_tiles)
         const int64_t resident = static_cast<int64_t>(kSMs) * split_warps_per_sm(class_kind(k), s);
         const int64_t w = (n_tiles[k] + resident - 1) / resident;
         r.tiles += n_tiles[k];
+        r.windows += static_cast<int64_t>(n_tiles[k]) * s;
         r.waves = std::max(r.waves, w);
         r.cost += w * s;
     }
@@ -467,11 +468,12 @@ ShapeLoad shape_load(const qew_ctx* h, int S, const int32_t* n_tiles)
 
 // Launches of a few steps are staging more than steps, which the deep tiles of the step shape only make
 // longer: they take the observing shape where its waves are cheaper.  Up to its K steps if there is one
-// wave, or the tiles are as wide and not more; else one or two.  us per call of qew_advance of 1 and 16
-// steps in the step shape and in the observing one, 4 chains: random field 2^20 sites 27.8 26.8, 41.9
-// 37.2, 2^21 sites (the observing shape has two waves, the step shape one) 30.6 31.5, 47.2 55.6; Case 3
-// 2^20 sites 32.3 28.8, 48.6 44.8; uniform cubic 2^18 sites 20.6 16.5, 28.9 26.5, 2^20 sites 24.5 20.8,
-// 44.1 46.0.
+// wave, or the tiles are as wide and not more; else a few, and half of K for the two-node kinds in many
+// waves, where the sum of the windows counts.  us per call of qew_advance of 1, 4 and 16 steps in the step
+// shape and in the observing one, 4 chains: random field 2^20 sites 27.8 26.8, 30.8 28.8, 41.9 37.2, 2^21
+// sites (the observing shape has two waves, the step shape one) 30.6 31.5, 33.0 36.1, 47.2 55.6, 2^22 sites
+// 59.8 53.7, 65.3 59.1, 90 90; Case 3 2^20 sites 32.3 28.8, 35.1 31.9, 48.6 44.8; uniform cubic 2^18 sites
+// 20.6 16.5, 22.6 18.5, 28.9 26.5, 2^20 sites 24.5 20.8, 28.0 25.0, 44.1 46.0.
 void short_launches(qew_ctx* h)
 {
     h->short_K = 0;
@@ -481,7 +483,9 @@ void short_launches(qew_ctx* h)
     if (min_kind_S(h, h->S) == min_kind_S(h, h->step_S) && obs.cost == step.cost && obs.tiles <= step.tiles)
         h->short_K = h->K;
     else if (5 * obs.cost < 4 * step.cost)
-        h->short_K = obs.waves == 1 ? h->K : 2;
+        h->short_K = obs.waves == 1 ? h->K : 2 * obs.cost <= step.cost ? h->K / 4 : 2;
+    else if (step.waves > 1 && obs.windows < step.windows && !(h->kinds_mask & kQuadMask))
+        h->short_K = h->K / 2;
 }
 
 // Tile lists for the current precision and launch shape; uploads chain descriptors and sizes

@@ -157,9 +157,13 @@ struct Tile {
     // whether a single cell against the drive is an ordinary move (else it takes the rare path of far
     // moves): a fifth of the linear-spline random bond's moves, a few in 10^4 of the other kinds'
     static constexpr bool kDown = KIND == kRBGLinear || KIND == kRBGCubic;
-    // KIND none stages offsets and cells side by side: it has no cache to make room for
-    static constexpr int slot2 = has_cache ? slot : 4 * TW;
-    static constexpr int bytes = has_cache ? queue + 2 * kQueue : 8 * TW;
+    // KIND none stages offsets and cells side by side, having no cache to make room for, and so does the
+    // random field up to 736-site tiles, where the room does not cost a warp: one wait instead of two at
+    // each end of a launch.  A launch of one step on 2^20 sites, 736-site tiles: 27 -> 22 us.  (Case 3 so
+    // only at 224-site tiles, 32768 sites 4.9 -> 4.6 ms per 5000 steps; wider ones lost 2% to 4%.)
+    static constexpr bool side_by_side = !has_cache || (KIND == kRF && S <= 23) || (KIND == kRBGLinear && S <= 7);
+    static constexpr int slot2 = !has_cache ? 4 * TW : side_by_side ? queue + 2 * kQueue : slot;
+    static constexpr int bytes = !has_cache ? 8 * TW : queue + 2 * kQueue + (side_by_side ? 4 * TW : 0);
 };
 
 // Per-lane mask of the sites that moved in a step.  Bit t is pair H - 1 - t's second site, bit D + t
@@ -539,9 +543,9 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
         if (lane == 0) {
             mbar_init(bar, 1);
             fence_mbar_init();
-            mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::has_cache ? 0 : 4)));
+            mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::side_by_side ? 4 : 0)));
             tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
-            if constexpr (!T::has_cache)
+            if constexpr (T::side_by_side)
                 tma_load_1d(s_cell, a.in.cell + p0, TW * 4, bar);
             if constexpr (T::has_pair)
                 tma_load_1d(s_loop, a.in.rf + p0, TW * 8, bar);
@@ -576,7 +580,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
         for (int x = lane; x < TW; x += 32) {
             const int64_t p = chain0 + site_index(wstart, x, contiguous, L);
             s_off[x] = __ldg(a.in.off + p);
-            if constexpr (!T::has_cache)
+            if constexpr (T::side_by_side)
                 s_cell[x] = __ldg(a.in.cell + p);
             if constexpr (T::has_pair)
                 reinterpret_cast<float2*>(s_loop)[x] = __ldg(a.in.rf + p);
@@ -641,7 +645,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             for (int j = 0; j < S; ++j)
                 s_cell[32 * j + lane] = cells[j];
             __syncwarp();
-        } else {
+        } else if constexpr (!T::side_by_side) {
             fence_proxy_async_shared();
             __syncwarp();
             if (tma_in) {
@@ -949,6 +953,21 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
         }
         s_cell[lane * S + 2 * H] = N0 + __float2int_rn(cT);
     }
+    // offsets, into the slot: side by side at once, else once the cells have left it
+    auto put_offsets = [&]() {
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
+            float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
+            if constexpr (KIND == kRBGLinear) {
+                if (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last))
+                    dj = -dj;
+            }
+            s_off[lane * S + j] = dj;
+        }
+    };
+    if constexpr (T::side_by_side)
+        put_offsets();
     if constexpr (T::has_cache) {
         // the cache back to linear order
         float2 q[S];
@@ -981,6 +1000,8 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             if (lane == 0) {
                 const uint32_t cnt = static_cast<uint32_t>(owned);
                 tma_store_1d(a.out.cell + out0, s_cell + pad, cnt * 4);
+                if constexpr (T::side_by_side)
+                    tma_store_1d(a.out.off + out0, s_off + pad, cnt * 4);
                 if constexpr (T::has_pair)
                     tma_store_1d(a.out.rf + out0, reinterpret_cast<float2*>(s_loop) + pad, cnt * 8);
                 if constexpr (T::has_quad) {
@@ -1000,6 +1021,8 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                 const int x = o + pad;
                 const int64_t p = out0 + o;
                 a.out.cell[p] = s_cell[x];
+                if constexpr (T::side_by_side)
+                    a.out.off[p] = s_off[x];
                 if constexpr (T::has_pair)
                     a.out.rf[p] = reinterpret_cast<float2*>(s_loop)[x];
                 if constexpr (T::has_quad) {
@@ -1013,16 +1036,10 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
             __syncwarp();
         }
     }
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-        const int p = (j < H) ? j : (j < 2 * H) ? j - H : 0;
-        float dj = (j < H) ? lo(d[p]) : (j < 2 * H) ? hi(d[p]) : dT;
-        if constexpr (KIND == kRBGLinear) {
-            if (upper & ((j < H) ? M::first(p) : (j < 2 * H) ? M::second(p) : M::last))
-                dj = -dj;
-        }
-        s_off[lane * S + j] = dj;
-    }
+    if constexpr (T::has_cache && T::side_by_side)
+        return;
+    if constexpr (!T::side_by_side)
+        put_offsets();
     if (tma_out) {
         fence_proxy_async_shared();
         __syncwarp();
