@@ -1121,7 +1121,7 @@ __global__ void split_tiles_kernel(const ChainDesc* chains, int cls, int32_t w_o
 // Block tiles of w_tile sites, one thread per site.
 // ---------------------------------------------------------------------------------------
 __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles, int32_t w_tile, SplitState st,
-                                  uint64_t seed, const double* u_in)
+                                  PhiloxKeys keys, const double* u_in)
 {
     const TileDesc td = tiles[blockIdx.x];
     const ChainDesc ch = chains[td.chain];
@@ -1147,24 +1147,24 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
         const int32_t M = ch.period;
         const int32_t m0 = wrap_node(n - 1, M), m1 = wrap_node(n, M), m2 = wrap_node(n + 1, M), m3 = wrap_node(n + 2, M);
         if (ch.kind == kRF)
-            st.rf[p] = make_float2(rf_plus_f32(seed, ch.s, i, m1, ch.f32), rf_plus_f32(seed, ch.s, i, m2, ch.f32));
+            st.rf[p] = make_float2(pair_node_f32<kRF>(keys, ch.s, i, m1, ch.f32), pair_node_f32<kRF>(keys, ch.s, i, m2, ch.f32));
         else if (ch.kind == kRBGLinear)
         {
             // the site's cell and the next one in the direction of the drive; the sign of the offset says
             // that the site is in the upper one
             const bool neg = ch.f32 < 0.0f;
-            const float g1 = rbg_f32(seed, ch.s, i, m1), g2 = rbg_f32(seed, ch.s, i, m2);
-            const float g3 = rbg_f32(seed, ch.s, i, neg ? m0 : m3);
+            const float g1 = rbg_f32(keys, ch.s, i, m1), g2 = rbg_f32(keys, ch.s, i, m2);
+            const float g3 = rbg_f32(keys, ch.s, i, neg ? m0 : m3);
             st.rf[p] = neg ? make_float2(g3 - g1, g1 - g2) : make_float2(g1 - g2, g2 - g3);
             st.q3[p] = g3;
             st.off[p] = neg ? -d : d;
         }
         else if (ch.kind == kRB || ch.kind == kRBGCubic) {
             const bool uni = ch.kind == kRB;
-            const float p0 = uni ? rb_f32(seed, ch.s, i, m0) : rbg_f32(seed, ch.s, i, m0);
-            const float p1 = uni ? rb_f32(seed, ch.s, i, m1) : rbg_f32(seed, ch.s, i, m1);
-            const float p2 = uni ? rb_f32(seed, ch.s, i, m2) : rbg_f32(seed, ch.s, i, m2);
-            const float p3 = uni ? rb_f32(seed, ch.s, i, m3) : rbg_f32(seed, ch.s, i, m3);
+            const float p0 = uni ? rb_f32(keys, ch.s, i, m0) : rbg_f32(keys, ch.s, i, m0);
+            const float p1 = uni ? rb_f32(keys, ch.s, i, m1) : rbg_f32(keys, ch.s, i, m1);
+            const float p2 = uni ? rb_f32(keys, ch.s, i, m2) : rbg_f32(keys, ch.s, i, m2);
+            const float p3 = uni ? rb_f32(keys, ch.s, i, m3) : rbg_f32(keys, ch.s, i, m3);
             float A, B, C;
             rb_coefficients(p0, p1, p2, p3, ch.f32, A, B, C);
             st.qn[p] = make_float2(p1, p2);
@@ -1291,7 +1291,7 @@ cudaError_t split_init(const ChainDesc* chains, int32_t, const TileDesc* tiles, 
 {
     if (n_tiles == 0)
         return cudaSuccess;
-    split_init_kernel<<<n_tiles, 256, 0, stream>>>(chains, tiles, w_tile, st, seed, u_in);
+    split_init_kernel<<<n_tiles, 256, 0, stream>>>(chains, tiles, w_tile, st, philox_key_schedule(seed), u_in);
     return cudaGetLastError();
 }
 
