@@ -78,7 +78,12 @@ enum qew_precision {
  * disorder `disorder_kind`, time step `dt`, flat start, precision QEW_FP32_SPLIT.
  * Requirements: 1 <= L < 2^31, batch >= 1, L * batch < 2^40, 0 < dt < 0.5, |f| < 2^12 (so that,
  * with neighbouring displacements below 2^12, no Euler step moves a site by 2^15 cells or more).
- * Allocates the state on the current CUDA device (QEW_ENOMEM if it does not fit).
+ * Allocates the state on the current CUDA device (QEW_ENOMEM if it does not fit): two buffers of 16 bytes
+ * per site (QEW_RF_GAUSS_LINEAR), 20 (QEW_RB_GAUSS_LINEAR; 16 if there is not enough memory for 20), 32
+ * (cubic kinds) or 8 (QEW_NONE), chains of 224 sites and more rounded up to 4 or 32 sites, and up to 256 MB
+ * of partial sums.  QEW_FP64: 16 bytes per site and two copies of 4 + 8 k, k = 2 (two-node kinds) or 4
+ * (cubic kinds), one more or two below 2^20 sites; one copy beyond 2^29 sites or if there is not enough
+ * memory for two, at about half the speed.
  * On success *out receives the handle; on failure *out is set to NULL.
  */
 int qew_create(qew_handle* out, int64_t L, int32_t batch, double f, double dt, int32_t disorder_kind,
@@ -324,6 +329,14 @@ int qew_observe_state_noalloc(const int32_t* cell, const float* off, int64_t L, 
  * Any other status means the failure path is broken.  The handle stays usable afterwards.
  */
 int qew_selftest_bounded_wait(qew_handle h, int32_t spin_limit);
+
+/*
+ * qew_selftest_lean -- put the handle into the form that it takes by itself when device memory is short,
+ * and reset it to the flat start: FP64 with one step per launch and one copy of the disorder caches,
+ * FP32-split with one launch shape, one observation per launch and, for QEW_RB_GAUSS_LINEAR, a cache of
+ * two values per site instead of three.  Results are the same; setting the precision ends it.
+ */
+int qew_selftest_lean(qew_handle h);
 
 /* qew_last_error -- message of the last failed call on `h` (NULL: of the last failed creation
  * or handle-less call on this thread).  Never NULL; "" if there was no error. */

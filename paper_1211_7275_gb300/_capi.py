@@ -61,6 +61,7 @@ SIGNATURES = {
     "qew_critical_force_rf": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int64, _P, ctypes.c_double, ctypes.c_double,
                                              _P, _P, _P, _P]),
     "qew_selftest_bounded_wait": (ctypes.c_int, [_H, ctypes.c_int32]),
+    "qew_selftest_lean": (ctypes.c_int, [_H]),
     "qew_last_error": (ctypes.c_char_p, [_H]),
     "qew_destroy": (None, [_H]),
 }

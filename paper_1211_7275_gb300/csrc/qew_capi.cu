@@ -79,7 +79,7 @@ struct qew_ctx {
     std::vector<int32_t> kind;
     std::vector<uint32_t> sample;   // sample index s of each chain (counter word 2)
     std::vector<int64_t> offset;    // first site of each chain in the caller's arrays (no gaps)
-    std::vector<int64_t> soffset;   // and in the FP32-split state, whose chains start on 128-byte boundaries
+    std::vector<int64_t> soffset;   // and in the FP32-split state (state_align)
     int64_t n_state = 0;            // sites of the FP32-split state arrays
     double dt = 0.1;
     uint64_t seed = 0;
@@ -117,6 +117,7 @@ struct qew_ctx {
     F64State f64[2] = {};            // disorder caches: two copies when a launch takes several steps
     F64Shape f64s = {256, 4, 1, false};
     bool f64_in_place = false;       // no memory for the second copy
+    bool lean = false;               // FP32-split: no memory for what only makes it faster
     TileDesc* d_ftiles = nullptr;    // tiles of the FP64 step kernel
     int32_t n_ftiles = 0;
     double* u64[2] = {nullptr, nullptr};
@@ -303,7 +304,7 @@ int alloc_buffers(qew_ctx* h)
                 take(s.off, N);
                 if (h->kinds_mask & kPairMask)
                     take(s.rf, N);
-                if (h->kinds_mask & (kQuadMask | 1 << kRBGLinear))
+                if (h->kinds_mask & kQuadMask || (h->kinds_mask >> kRBGLinear & 1 && !h->lean))
                     take(s.q3, N);
                 if (h->kinds_mask & kQuadMask) {
                     take(s.qn, N);
@@ -343,6 +344,13 @@ int alloc_state(qew_ctx* h)
         rc = build_layout(h);
         if (rc == QEW_OK)
             rc = alloc_buffers(h);
+    } else if (rc == QEW_ENOMEM && h->precision == QEW_FP32_SPLIT && !h->lean) {
+        // one shape for all launches, one observation per launch, and the linear-spline random bond's
+        // third node drawn by each launch: 16 instead of 20 bytes per site and buffer for that kind
+        h->lean = true;
+        rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = alloc_buffers(h);
     }
     return rc;
 }
@@ -379,6 +387,12 @@ size_t max_kind_smem(const qew_ctx* h, int S, int tiles_per_cta)
     return m;
 }
 
+// Whether launches without observations may take a shape of their own.
+bool own_step_shape(const qew_ctx* h)
+{
+    return !h->shape_given && !h->lean;
+}
+
 // Step shape of a handle in its default shape, by the number of sites.  Few sites are latency: a
 // launch costs some 7 us beside its steps, so deep launches, and a step of a warp of 7 or 15 sites per
 // lane takes half the time of one of 23.  More sites fill the SMs better with wider tiles (less halo,
@@ -394,7 +408,7 @@ void step_shape(qew_ctx* h)
     h->step_S = h->S;
     h->step_K = h->K;
     h->step_tpc = h->tpc;
-    if (h->shape_given)
+    if (!own_step_shape(h))
         return;
     const int64_t n = h->n_sites;
     const bool case1 = h->kinds_mask >> kRBGCubic & 1, case3 = h->kinds_mask >> kRBGLinear & 1;
@@ -421,26 +435,25 @@ void step_shape(qew_ctx* h)
     // steps: uniform cubic, 100 sites 3.3 by the number of sites alone (480 x 48), 2.2 so (224 x 48);
     // 192 sites 3.3, 2.6; random field, 300 sites 5.5, 3.1.  The line at 3/4 leaves longer chains alone,
     // where the best alternative has 1.0 of the windows.
-    if (*std::min_element(h->L.begin(), h->L.end()) < 4096) {
-        auto cost = [&](int S, int K) {
-            double windows = 0.0;
-            for (int32_t c = 0; c < h->n_chains; ++c) {
-                const int s = kind_S(h->kind[c], S);
-                windows += static_cast<double>((h->L[c] + 32 * s - 2 * K - 1) / (32 * s - 2 * K)) * s;
-            }
-            return windows * (K + 4) / K;
-        };
-        double best = 0.75 * cost(h->step_S, h->step_K);
-        const int limit = h->step_S;
-        const int shapes[][2] = {{7, 48}, {7, 32}, {7, 16}, {15, 48}, {15, 32}, {23, 48}};
-        for (const auto& s : shapes) {
-            const double c = s[0] <= limit ? cost(s[0], s[1]) : best;
-            if (c < best) {
-                best = c;
-                h->step_S = s[0];
-                h->step_K = s[1];
+    if (h->precision == QEW_FP32_SPLIT && *std::min_element(h->L.begin(), h->L.end()) < 4096) {
+        const int shapes[7][2] = {{h->step_S, h->step_K}, {7, 48}, {7, 32}, {7, 16}, {15, 48}, {15, 32}, {23, 48}};
+        double cost[7] = {};
+        for (int32_t c = 0, end; c < h->n_chains; c = end) {   // runs of equal chains
+            for (end = c + 1; end < h->n_chains && h->L[end] == h->L[c] && h->kind[end] == h->kind[c];)
+                ++end;
+            for (int k = 0; k < 7; ++k) {
+                const int s = kind_S(h->kind[c], shapes[k][0]), own = 32 * s - 2 * shapes[k][1];
+                cost[k] += static_cast<double>((h->L[c] + own - 1) / own) * (end - c) * s;
             }
         }
+        int best = 0;
+        for (int k = 0; k < 7; ++k) {
+            cost[k] *= (k == 0 ? 0.75 : 1.0) * (shapes[k][1] + 4) / shapes[k][1];
+            if (shapes[k][0] <= shapes[0][0] && cost[k] < cost[best])
+                best = k;
+        }
+        h->step_S = shapes[best][0];
+        h->step_K = shapes[best][1];
     }
 }
 
@@ -477,7 +490,7 @@ ShapeLoad shape_load(const qew_ctx* h, int S, const int32_t* n_tiles)
 void short_launches(qew_ctx* h)
 {
     h->short_K = 0;
-    if (h->shape_given || h->precision != QEW_FP32_SPLIT || h->n_sites < (int64_t(1) << 17))
+    if (!own_step_shape(h) || h->precision != QEW_FP32_SPLIT || h->n_sites < (int64_t(1) << 17))
         return;
     const ShapeLoad obs = shape_load(h, h->S, h->n_tiles), step = shape_load(h, h->step_S, h->n_step_tiles);
     if (min_kind_S(h, h->S) == min_kind_S(h, h->step_S) && obs.cost == step.cost && obs.tiles <= step.tiles)
@@ -495,7 +508,7 @@ int build_layout(qew_ctx* h)
     drop_graph(h);   // captured launches point at the descriptors rebuilt here
     h->layout_made = false;
     step_shape(h);
-    const bool own_step = h->precision == QEW_FP32_SPLIT && !h->shape_given;
+    const bool own_step = h->precision == QEW_FP32_SPLIT && own_step_shape(h);
     for (int k = 0; k < kNumKinds; ++k) {
         h->w_own[k] = 32 * kind_S(k, h->S) - 2 * h->K;
         h->step_w_own[k] = 32 * kind_S(k, h->step_S) - 2 * h->step_K;
@@ -605,16 +618,23 @@ int build_layout(qew_ctx* h)
                  "uploading FP64 tiles");
     }
     short_launches(h);
-    // room for the partials of as many observations as 256 MB hold
+    // room for the partials of as many observations as 256 MB hold, or of one where that is too much
     h->partial_slots = slots;
     h->launch_obs = 1;
-    if (h->precision == QEW_FP32_SPLIT)
+    if (h->precision == QEW_FP32_SPLIT && !h->lean)
         h->launch_obs = static_cast<int>(std::min<size_t>(kMaxLaunchObs, std::max<size_t>(1, (size_t(256) << 20) / (slots * 32))));
-    const size_t need = slots * 4 * h->launch_obs;
-    if (need > h->partial_cap) {
+    size_t need = slots * 4 * h->launch_obs;
+    if (need > h->partial_cap || h->lean) {
         dev_free(h->d_partial);
         h->partial_cap = 0;
-        QEW_CUDA(h, dev_alloc(&h->d_partial, need), "allocating partial sums");
+        cudaError_t e = dev_alloc(&h->d_partial, need);
+        if (e == cudaErrorMemoryAllocation && h->launch_obs > 1) {
+            cudaGetLastError();
+            h->launch_obs = 1;
+            need = slots * 4;
+            e = dev_alloc(&h->d_partial, need);
+        }
+        QEW_CUDA(h, e, "allocating partial sums");
         h->partial_cap = need;
     }
     h->layout_made = true;
@@ -657,7 +677,7 @@ struct Segment {
 SplitLaunch split_args(qew_ctx* h, int cls, const Segment& s, SplitState in, SplitState out)
 {
     SplitLaunch a{};
-    const bool other = s.step_only && !h->shape_given;
+    const bool other = s.step_only && own_step_shape(h);
     const int kind = class_kind(cls);
     a.tiles = other ? h->d_step_tiles[cls] : h->d_tiles[cls];
     a.n_tiles = other ? h->n_step_tiles[cls] : h->n_tiles[cls];
@@ -868,7 +888,7 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
                 end = std::min<int64_t>(end, kTuneAfterSteps);
             // Where launches without observations have their own shape, all steps but the segment of an
             // observation at `end` take it (the segment is what is left over whole K steps).
-            if (!h->shape_given && at < end) {
+            if (own_step_shape(h) && at < end) {
                 const bool observed = d_obs && end == targets[k];
                 const int64_t bulk = observed ? (end - at - 1) / h->K * h->K : end - at;
                 if (bulk > 0) {
@@ -1017,6 +1037,14 @@ int autotune(qew_ctx* h)
     return build_layout(h);
 }
 
+// Sites on whose multiples a chain starts in the FP32-split state: bulk copies need four (16 bytes) for
+// windows inside a chain, whole 128-byte lines are worth their room in long ones, and chains shorter than
+// a window, which has to wrap around them, follow one another.
+int64_t state_align(int64_t L)
+{
+    return L >= 4096 ? 32 : L >= 224 ? 4 : 1;
+}
+
 int validate_common(double dt, uint64_t)
 {
     if (!(dt > 0.0 && dt < 0.5))
@@ -1074,8 +1102,9 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
         for (int32_t c = 0; c < n_chains; ++c) {
             h->offset[c] = off;
             off += L[c];
-            h->soffset[c] = h->n_state;
-            h->n_state += (L[c] + 31) & ~int64_t(31);
+            const int64_t align = state_align(L[c]);
+            h->soffset[c] = (h->n_state + align - 1) / align * align;
+            h->n_state = h->soffset[c] + L[c];
             h->kinds_mask |= 1 << kind[c];
             h->sites_of_class[chain_class(kind[c], static_cast<float>(f[c]))] += L[c];
         }
@@ -1392,9 +1421,9 @@ int qew_set_precision(qew_handle h, int32_t precision)
     if (h->step != 0)
         return fail(h, QEW_ESTATE, "precision can only change before the first step");
     DeviceGuard g(h->device);
-    if (h->f64_in_place) {   // caches of the one-step shape: there may be room for the others by now
+    if (h->f64_in_place || h->lean) {   // there may be room for the rest by now
         free_state(h);
-        h->f64_in_place = false;
+        h->f64_in_place = h->lean = false;
     }
     h->precision = precision;
     int rc = build_layout(h);
@@ -1773,6 +1802,22 @@ int qew_selftest_bounded_wait(qew_handle h, int32_t spin_limit)
     QEW_CUDA(h, bounded_wait_selftest(h->d_error, spin_limit, h->stream), "launching the bounded-wait probe");
     QEW_CUDA(h, cudaStreamSynchronize(h->stream), "running the bounded-wait probe");
     return check_device_error(h);
+}
+
+int qew_selftest_lean(qew_handle h)
+{
+    if (int rc = check_handle(h))
+        return rc;
+    DeviceGuard g(h->device);
+    cudaStreamSynchronize(h->stream);
+    free_state(h);
+    h->f64_in_place = h->lean = true;
+    int rc = build_layout(h);
+    if (rc == QEW_OK)
+        rc = alloc_buffers(h);
+    if (rc == QEW_OK)
+        rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+    return rc;
 }
 
 const char* qew_last_error(qew_handle h)

@@ -12,10 +12,12 @@
 namespace qew {
 
 // FP32-split state: cell n (int32), in-cell offset d (float, [0,1)) and the disorder cache
-// of each site.  The two-node kinds keep (R(n) + f, R(n+1) + f) or (G(n), G(n+1)) in rf.  The
-// cubic kinds keep the nodes V(n), V(n+1) in qn, V(n+2) in q3, and the coefficients of
-// F_p + f = A + d (B + d C) over cell n (from V(n-1) .. V(n+2)) in qab (A, B) and qc (C).  A
-// chain of kind NONE uses none of them.
+// of each site.  The random field keeps (R(n) + f, R(n+1) + f) in rf.  The linear-spline random bond
+// keeps F_p = G - G(+1) of two neighbouring cells in rf, the sign of d saying that the site is in the
+// upper one, and in q3 the node beyond them in the direction of the drive; where memory is short q3 is
+// NULL and each launch draws that node anew.  The cubic kinds keep the nodes V(n), V(n+1) in qn, V(n+2)
+// in q3, and the coefficients of F_p + f = A + d (B + d C) over cell n (from V(n-1) .. V(n+2)) in qab
+// (A, B) and qc (C).  A chain of kind NONE uses none of them.
 struct SplitState {
     int32_t* cell;
     float* off;

@@ -69,10 +69,10 @@ __device__ __forceinline__ int32_t site_index(int64_t wstart, int x, bool contig
     return wrap_site(g, L);
 }
 
-// Bytes of disorder cache per site in HBM.
+// Bytes of disorder cache per site in HBM, beside the third node.
 template <int KIND>
 struct CacheBytes {
-    static constexpr int hbm = KIND == kRF ? 8 : KIND == kRBGLinear ? 12 : quad_kind(KIND) ? 24 : 0;
+    static constexpr int hbm = pair_kind(KIND) ? 8 : quad_kind(KIND) ? 20 : 0;
 };
 
 // ---- two sites at a time ----
@@ -537,13 +537,14 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
     // coalesced read-only loads.  Offsets come first, with the cache, and then the cells through
     // the same slot, where they stay.
     const int64_t p0 = wt.p - pad;
+    const bool has_top = T::has_quad || (KIND == kRBGLinear && a.in.q3 != nullptr);   // see SplitState
     const bool tma_in = contiguous && (p0 & 3) == 0;
     uint64_t* bar = &s_bar[warp];
     if (tma_in) {
         if (lane == 0) {
             mbar_init(bar, 1);
             fence_mbar_init();
-            mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::side_by_side ? 4 : 0)));
+            mbar_arrive_expect_tx(bar, TW * (4 + CacheBytes<KIND>::hbm + (T::side_by_side ? 4 : 0) + (has_top ? 4 : 0)));
             tma_load_1d(s_off, a.in.off + p0, TW * 4, bar);
             if constexpr (T::side_by_side)
                 tma_load_1d(s_cell, a.in.cell + p0, TW * 4, bar);
@@ -554,7 +555,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                 tma_load_1d(s_loop, a.in.qab + p0, TW * 8, bar);
                 tma_load_1d(s_loopc, a.in.qc + p0, TW * 4, bar);
             }
-            if constexpr (T::has_quad || KIND == kRBGLinear)
+            if (has_top)
                 tma_load_1d(s_top, a.in.q3 + p0, TW * 4, bar);
         }
         __syncwarp();   // no lane polls the barrier before it is initialised
@@ -589,7 +590,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                 reinterpret_cast<float2*>(s_loop)[x] = __ldg(a.in.qab + p);
                 s_loopc[x] = __ldg(a.in.qc + p);
             }
-            if constexpr (T::has_quad || KIND == kRBGLinear)
+            if (has_top)
                 s_top[x] = __ldg(a.in.q3 + p);
         }
         __syncwarp();
@@ -688,6 +689,13 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
         if (upper & M::last)
             s_cell[lane * S + 2 * H] -= 1;
         __syncwarp();
+        if (!has_top) {
+#pragma unroll 1
+            for (int x = lane; x < TW; x += 32)
+                s_top[x] = pair_node_f32<KIND>(a.keys, s, site_index(wstart, x, contiguous, L),
+                                               wrap_node(s_cell[x] + (NEG ? 0 : 2), period), f);
+            __syncwarp();
+        }
     }
 
     Force<KIND, S> force;
@@ -1009,7 +1017,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                     tma_store_1d(a.out.qab + out0, reinterpret_cast<float2*>(s_loop) + pad, cnt * 8);
                     tma_store_1d(a.out.qc + out0, s_loopc + pad, cnt * 4);
                 }
-                if constexpr (T::has_quad || KIND == kRBGLinear)
+                if (has_top)
                     tma_store_1d(a.out.q3 + out0, s_top + pad, cnt * 4);
                 tma_store_commit();
                 tma_store_wait_read_all();   // the slot may be overwritten
@@ -1030,7 +1038,7 @@ __global__ void __maxnreg__((MaxRegs<KIND, S>::value)) split_step_kernel(SplitLa
                     a.out.qab[p] = reinterpret_cast<float2*>(s_loop)[x];
                     a.out.qc[p] = s_loopc[x];
                 }
-                if constexpr (T::has_quad || KIND == kRBGLinear)
+                if (has_top)
                     a.out.q3[p] = s_top[x];
             }
             __syncwarp();
@@ -1156,7 +1164,8 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
             const float g1 = rbg_f32(keys, ch.s, i, m1), g2 = rbg_f32(keys, ch.s, i, m2);
             const float g3 = rbg_f32(keys, ch.s, i, neg ? m0 : m3);
             st.rf[p] = neg ? make_float2(g3 - g1, g1 - g2) : make_float2(g1 - g2, g2 - g3);
-            st.q3[p] = g3;
+            if (st.q3)
+                st.q3[p] = g3;
             st.off[p] = neg ? -d : d;
         }
         else if (ch.kind == kRB || ch.kind == kRBGCubic) {

@@ -172,3 +172,31 @@ def test_fp64_batch_with_room_for_one_copy_of_the_caches(lib, kind, per_site):
     assert lib.fake_bad() == 0, lib.fake_first_bad()
     assert lib.fake_last_K() == 8 and lib.fake_last_in_place() == 0
     lib.qew_destroy(h)
+
+
+@pytest.mark.parametrize("kind,L,per_site,per_chain", [
+    (0, [(1 << 22) + 5], 32, 0), (3, [(1 << 22) + 5], 32, 0), (1, [(1 << 22) + 5], 64, 0), (2, [(1 << 22) + 5], 16, 0),
+    (0, [1] * 50000, 32, 200), (3, [37] * 50000, 32, 200), (4, [101] * 20000, 64, 200)])
+def test_fp32_batch_with_room_for_the_state(lib, kind, L, per_site, per_chain):
+    """Two buffers of cells, offsets and caches and little beside them: what only makes a relaxation faster
+    (tile lists of a second shape, the partials of many observations, Case 3's third node) gives way."""
+    n = sum(L)
+    lib.fake_reset()
+    lib.fake_capacity(lib.fake_held() + int(1.015 * per_site * n) + per_chain * len(L))
+    rc, h = create(lib, L, kind, FP32)
+    assert rc == OK
+    assert lib.qew_advance(h, 100) == OK
+    lib.fake_capacity(2 ** 62)
+    v = np.empty(30 * len(L))
+    t = np.arange(100, 130, dtype=np.int64)
+    assert lib.qew_observe(h, _p(t), 30, _p(v), None) == OK
+    assert lib.fake_max_n_obs() == 1 and lib.fake_bad() == 0, lib.fake_first_bad()
+    if kind == 3:
+        assert lib.fake_last_has_q3() == 0
+    # with the memory back, setting the precision again takes the rest
+    assert lib.qew_reset(h) == OK and lib.qew_set_precision(h, FP32) == OK
+    assert lib.qew_observe(h, _p(t), 30, _p(v), None) == OK
+    assert lib.fake_max_n_obs() > 1 and lib.fake_bad() == 0, lib.fake_first_bad()
+    if kind == 3:
+        assert lib.fake_last_has_q3() == 1
+    lib.qew_destroy(h)
