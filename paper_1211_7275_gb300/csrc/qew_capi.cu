@@ -1122,7 +1122,7 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
             if (e == cudaSuccess)
                 e = dev_alloc(&h->d_error, 1);
             if (e == cudaSuccess)
-                e = cudaMemset(h->d_error, 0, sizeof(int32_t));
+                e = cudaMemsetAsync(h->d_error, 0, sizeof(int32_t), h->stream);
             if (e != cudaSuccess)
                 rc = cuda_fail(h, e, "allocating reference shifts");
         }
@@ -1155,7 +1155,7 @@ int check_device_error(qew_ctx* h)
     int32_t flag = 0;
     QEW_CUDA(h, cudaMemcpy(&flag, h->d_error, sizeof(flag), cudaMemcpyDeviceToHost), "reading the error flag");
     if (flag) {
-        cudaMemset(h->d_error, 0, sizeof(int32_t));
+        cudaMemsetAsync(h->d_error, 0, sizeof(int32_t), h->stream);
         if (flag == 2)
             return fail(h, QEW_ESTATE, "neighbouring displacements reached 2^12 cells, outside the range the "
                                        "FP32-split kernel represents exactly; the state is no longer valid");
@@ -1377,7 +1377,7 @@ int set_state_impl(qew_ctx* h, const double* u_in)
     cudaError_t e = dev_alloc(&d_u, N);
     if (e != cudaSuccess)
         return cuda_fail(h, e, "allocating a state copy");
-    e = cudaMemcpy(d_u, u_in, N * sizeof(double), cudaMemcpyHostToDevice);
+    e = cudaMemcpyAsync(d_u, u_in, N * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     int rc = (e == cudaSuccess) ? init_state(h, d_u, shift0) : cuda_fail(h, e, "uploading the state");
     dev_free(d_u);
     return rc;
@@ -1752,7 +1752,7 @@ int qew_enable_stats(qew_handle h, int32_t enable)
     if (enable && !h->d_crossings)
         QEW_CUDA(h, dev_alloc(&h->d_crossings, 1), "allocating the crossing counter");
     if (h->d_crossings)
-        QEW_CUDA(h, cudaMemset(h->d_crossings, 0, sizeof(unsigned long long)), "clearing the crossing counter");
+        QEW_CUDA(h, cudaMemsetAsync(h->d_crossings, 0, sizeof(unsigned long long), h->stream), "clearing the crossing counter");
     h->stats_on = enable != 0;
     h->n_launches = h->n_fused = h->n_site_updates = 0;
     h->ev_used = 0;
@@ -1775,7 +1775,7 @@ int qew_get_stats(qew_handle h, int64_t* launches, int64_t* fused_launches, doub
     unsigned long long cr = 0;
     if (h->stats_on && h->d_crossings) {
         QEW_CUDA(h, cudaMemcpy(&cr, h->d_crossings, sizeof(cr), cudaMemcpyDeviceToHost), "reading crossings");
-        QEW_CUDA(h, cudaMemset(h->d_crossings, 0, sizeof(cr)), "clearing the crossing counter");
+        QEW_CUDA(h, cudaMemsetAsync(h->d_crossings, 0, sizeof(cr), h->stream), "clearing the crossing counter");
     }
     if (launches)
         *launches = h->n_launches;

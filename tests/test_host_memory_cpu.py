@@ -131,6 +131,20 @@ def test_creation_fails_cleanly(lib, kind, precision, L):
 
 
 @pytest.mark.parametrize("precision", [FP32, FP64])
+def test_uploads_and_fills_are_ordered_with_the_kernels(lib, precision):
+    """The handle's stream does not wait for the legacy default stream, where a copy from pageable memory
+    may still be under way when the call returns: nothing but reads of finished results goes there."""
+    lib.fake_reset()
+    rc, h = create(lib, [3000, 3000], 0, precision)
+    assert rc == OK and calls(lib, h, 6000) == [OK] * 7
+    assert lib.qew_enable_stats(h, 1) == OK and calls(lib, h, 6000) == [OK] * 7
+    assert lib.qew_get_stats(h, None, None, None, None, None) == OK
+    assert lib.qew_set_precision(h, 1 - precision) == OK and calls(lib, h, 6000) == [OK] * 7
+    assert lib.fake_off_stream() == 0
+    lib.qew_destroy(h)
+
+
+@pytest.mark.parametrize("precision", [FP32, FP64])
 def test_allocations_inside_the_calls(lib, precision):
     L = 5000
     lib.fake_reset()
