@@ -175,6 +175,17 @@ int fail(qew_ctx* h, int code, const std::string& msg)
     return code;
 }
 
+// No exception leaves a C entry: those whose work allocates on the host run it through this.
+template <class F>
+int guarded(qew_ctx* h, F&& work)
+{
+    try {
+        return work();
+    } catch (const std::bad_alloc&) {
+        return fail(h, QEW_ENOMEM, "host allocation failed");
+    }
+}
+
 int cuda_fail(qew_ctx* h, cudaError_t e, const char* where)
 {
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
@@ -584,9 +595,9 @@ int build_layout(qew_ctx* h)
     // the warp tiles are written on the device, from the chains and these
     int32_t* d_first = nullptr;
     if (h->precision == QEW_FP32_SPLIT) {
-        QEW_CUDA(h, dev_alloc(&d_first, 2 * static_cast<size_t>(h->n_chains)), "allocating tile lists");
         std::vector<int32_t> both(first);
         both.insert(both.end(), step_first.begin(), step_first.end());
+        QEW_CUDA(h, dev_alloc(&d_first, 2 * static_cast<size_t>(h->n_chains)), "allocating tile lists");
         cudaError_t e = cudaMemcpyAsync(d_first, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream);
         for (int k = 0; k < kNumClasses; ++k) {
             const int kind = class_kind(k);
@@ -1238,8 +1249,10 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
         const int cur0 = h->cur;
         const int64_t l0 = h->n_launches, f0 = h->n_fused, s0 = h->n_site_updates;
         bool capturing = false;
+        std::vector<int64_t> key;
         if (graphable) {
             drop_graph(h);
+            key.assign(steps, steps + n_times);
             capturing = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
             if (!capturing)
                 cudaGetLastError();
@@ -1258,7 +1271,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
                     cudaGraphDestroy(graph);
                 h->step = step0;   // nothing ran: undo the host-side bookkeeping
                 h->cur = cur0;
-                        if (rc != QEW_OK)
+                if (rc != QEW_OK)
                     return rc;
                 return cuda_fail(h, ce != cudaSuccess ? ce : ee, "capturing the observation graph");
             }
@@ -1268,9 +1281,9 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
                 h->gexec = nullptr;
                 h->step = step0;
                 h->cur = cur0;
-                        return cuda_fail(h, ce, "instantiating the observation graph");
+                return cuda_fail(h, ce, "instantiating the observation graph");
             }
-            h->g_steps.assign(steps, steps + n_times);
+            h->g_steps.swap(key);
             h->g_step0 = step0;
             h->g_cur0 = cur0;
             h->g_step1 = h->step;
@@ -1421,17 +1434,19 @@ int qew_set_precision(qew_handle h, int32_t precision)
     if (h->step != 0)
         return fail(h, QEW_ESTATE, "precision can only change before the first step");
     DeviceGuard g(h->device);
-    if (h->f64_in_place || h->lean) {   // there may be room for the rest by now
-        free_state(h);
-        h->f64_in_place = h->lean = false;
-    }
-    h->precision = precision;
-    int rc = build_layout(h);
-    if (rc == QEW_OK)
-        rc = alloc_state(h);
-    if (rc == QEW_OK)
-        rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
-    return rc;
+    return guarded(h, [&]() -> int {
+        if (h->f64_in_place || h->lean) {   // there may be room for the rest by now
+            free_state(h);
+            h->f64_in_place = h->lean = false;
+        }
+        h->precision = precision;
+        int rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = alloc_state(h);
+        if (rc == QEW_OK)
+            rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+        return rc;
+    });
 }
 
 int qew_set_disorder_period(qew_handle h, int64_t period)
@@ -1441,12 +1456,14 @@ int qew_set_disorder_period(qew_handle h, int64_t period)
     if (period < 0 || period >= (int64_t(1) << 31))
         return fail(h, QEW_EINVAL, "period must lie in [0, 2^31)");
     DeviceGuard g(h->device);
-    cudaStreamSynchronize(h->stream);
-    h->period = static_cast<int32_t>(period);
-    int rc = build_layout(h);
-    if (rc == QEW_OK)
-        rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
-    return rc;
+    return guarded(h, [&]() -> int {
+        cudaStreamSynchronize(h->stream);
+        h->period = static_cast<int32_t>(period);
+        int rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+        return rc;
+    });
 }
 
 int qew_set_samples(qew_handle h, const uint32_t* s)
@@ -1456,12 +1473,14 @@ int qew_set_samples(qew_handle h, const uint32_t* s)
     if (!s)
         return fail(h, QEW_EINVAL, "s must not be NULL");
     DeviceGuard g(h->device);
-    cudaStreamSynchronize(h->stream);
-    h->sample.assign(s, s + h->n_chains);
-    int rc = build_layout(h);
-    if (rc == QEW_OK)
-        rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
-    return rc;
+    return guarded(h, [&]() -> int {
+        cudaStreamSynchronize(h->stream);
+        h->sample.assign(s, s + h->n_chains);
+        int rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+        return rc;
+    });
 }
 
 int qew_set_stream(qew_handle h, void* stream)
@@ -1500,7 +1519,7 @@ int qew_set_tuning(qew_handle h, int32_t tile_w, int32_t K, int32_t tiles_per_ct
     h->tpc = tiles_per_cta;
     h->shape_given = true;
     h->autotune_pending = false;
-    return build_layout(h);
+    return guarded(h, [&] { return build_layout(h); });
 }
 
 int qew_get_tuning(qew_handle h, int32_t* tile_w, int32_t* K, int32_t* tiles_per_cta)
@@ -1530,16 +1549,18 @@ int qew_advance(qew_handle h, int64_t n_steps)
     if (int rc = check_arrays(h))
         return rc;
     DeviceGuard g(h->device);
-    const int64_t target = h->step + n_steps;
-    int rc = run_through(h, &target, 1, nullptr);
-    if (rc == QEW_OK && n_steps > 0)
-        rc = guard_range(h);
-    if (rc == QEW_OK) {
-        cudaError_t e = cudaPeekAtLastError();
-        if (e != cudaSuccess)
-            return cuda_fail(h, e, "advancing");
-    }
-    return rc;
+    return guarded(h, [&]() -> int {
+        const int64_t target = h->step + n_steps;
+        int rc = run_through(h, &target, 1, nullptr);
+        if (rc == QEW_OK && n_steps > 0)
+            rc = guard_range(h);
+        if (rc == QEW_OK) {
+            cudaError_t e = cudaPeekAtLastError();
+            if (e != cudaSuccess)
+                return cuda_fail(h, e, "advancing");
+        }
+        return rc;
+    });
 }
 
 int qew_observe(qew_handle h, const int64_t* steps, int32_t n_times, double* v_out, double* w2_out)
@@ -1547,7 +1568,7 @@ int qew_observe(qew_handle h, const int64_t* steps, int32_t n_times, double* v_o
     if (int rc = check_handle(h))
         return rc;
     DeviceGuard g(h->device);
-    return observe_impl(h, steps, n_times, v_out, nullptr, w2_out);
+    return guarded(h, [&] { return observe_impl(h, steps, n_times, v_out, nullptr, w2_out); });
 }
 
 int qew_observe_ex(qew_handle h, const int64_t* steps, int32_t n_times, double* v_out, double* ubar_out,
@@ -1556,7 +1577,7 @@ int qew_observe_ex(qew_handle h, const int64_t* steps, int32_t n_times, double* 
     if (int rc = check_handle(h))
         return rc;
     DeviceGuard g(h->device);
-    return observe_impl(h, steps, n_times, v_out, ubar_out, w2_out);
+    return guarded(h, [&] { return observe_impl(h, steps, n_times, v_out, ubar_out, w2_out); });
 }
 
 int qew_get_state(qew_handle h, double* u_out, int64_t* step_out)
@@ -1584,7 +1605,7 @@ int qew_set_state(qew_handle h, const double* u_in)
     if (!u_in)
         return fail(h, QEW_EINVAL, "u_in must not be NULL");
     DeviceGuard g(h->device);
-    return set_state_impl(h, u_in);
+    return guarded(h, [&] { return set_state_impl(h, u_in); });
 }
 
 int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
@@ -1668,7 +1689,7 @@ int qew_reset(qew_handle h)
     if (int rc = check_handle(h))
         return rc;
     DeviceGuard g(h->device);
-    return init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+    return guarded(h, [&] { return init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0)); });
 }
 
 int qew_num_sites(qew_handle h, int64_t* n_sites)
@@ -1809,15 +1830,17 @@ int qew_selftest_lean(qew_handle h)
     if (int rc = check_handle(h))
         return rc;
     DeviceGuard g(h->device);
-    cudaStreamSynchronize(h->stream);
-    free_state(h);
-    h->f64_in_place = h->lean = true;
-    int rc = build_layout(h);
-    if (rc == QEW_OK)
-        rc = alloc_buffers(h);
-    if (rc == QEW_OK)
-        rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
-    return rc;
+    return guarded(h, [&]() -> int {
+        cudaStreamSynchronize(h->stream);
+        free_state(h);
+        h->f64_in_place = h->lean = true;
+        int rc = build_layout(h);
+        if (rc == QEW_OK)
+            rc = alloc_buffers(h);
+        if (rc == QEW_OK)
+            rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
+        return rc;
+    });
 }
 
 const char* qew_last_error(qew_handle h)

@@ -22,7 +22,6 @@ size_t held = 0, peak = 0, capacity = ~size_t(0);
 int64_t until_failure = -1;   // allocations until one fails (-1: none does)
 int64_t launches = 0, bad = 0;
 std::string first_bad;
-cudaStream_t expected = nullptr;
 int64_t off_stream = 0;       // copies and fills that other work does not wait for
 int32_t last_K = 0, last_in_place = 0, last_n_obs = 0, max_n_obs = 0, last_has_q3 = 0;
 
@@ -35,9 +34,8 @@ void need(const void* p, const char* what)
     }
 }
 
-void on_stream(cudaStream_t s)
+void on_stream(cudaStream_t)
 {
-    expected = s;
     ++launches;
 }
 

@@ -23,10 +23,11 @@ FP32, FP64 = 0, 1
 def lib(tmp_path_factory):
     tmp = tmp_path_factory.mktemp("fake")
     cc, procs, objs = _build.nvcc(), [], []
-    for src in (os.path.join(_build.CSRC, "qew_capi.cu"), os.path.join(HERE, "fake", "fake_cuda.cpp")):
+    for src, lang in ((os.path.join(_build.CSRC, "qew_capi.cu"), "cu"), (os.path.join(HERE, "fake", "fake_cuda.cpp"), "cu"),
+                      (os.path.join(HERE, "fake", "fake_new.cpp"), "c++")):
         objs.append(str(tmp / (os.path.basename(src) + ".o")))
         procs.append(subprocess.Popen([cc, "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-I", _build.INCLUDE, "-I", _build.CSRC,
-                                       *_build.ARCH, "-x", "cu", "-c", src, "-o", objs[-1]]))
+                                       *_build.ARCH, "-x", lang, "-c", src, "-o", objs[-1]]))
     assert all(p.wait() == 0 for p in procs)
     out = str(tmp / "libqew_fake.so")
     wrap = [x for n in WRAPPED for x in ("-Xlinker", f"--wrap=cuda{n}")]
@@ -36,6 +37,7 @@ def lib(tmp_path_factory):
         if hasattr(lib, name):
             getattr(lib, name).restype, getattr(lib, name).argtypes = res, args
     lib.fake_fail_after.argtypes = [ctypes.c_int64]
+    lib.fake_throw_after.argtypes = [ctypes.c_int64]
     lib.fake_capacity.argtypes = [ctypes.c_size_t]
     for n in ("fake_held", "fake_peak"):
         getattr(lib, n).restype = ctypes.c_size_t
@@ -108,6 +110,33 @@ def test_a_handle_whose_reconfiguration_fails(lib, what, kind, L):
         lib.qew_destroy(h)
         if rc == OK and fail > 20:
             break
+
+
+@pytest.mark.parametrize("what", sorted(RECONFIGURE))
+def test_host_allocations_that_fail(lib, what):
+    """No exception leaves a C entry: QEW_ENOMEM, and the handle is as after a failed device allocation."""
+    precision, change = RECONFIGURE[what]
+    L = 5000
+    v, zero = np.empty(8), np.zeros(2 * L)
+    others = [lambda h: lib.qew_reset(h), lambda h: lib.qew_set_state(h, _p(zero)), lambda h: lib.qew_advance(h, 40),
+              lambda h: lib.qew_observe(h, _p(np.array([2000, 2001], dtype=np.int64)), 2, _p(v), None)]
+    lib.fake_reset()
+    rc, h = create(lib, [L, L], 3, precision)
+    assert rc == OK
+    assert lib.qew_enable_stats(h, 1) == OK
+    for fail in range(40):
+        for call in [lambda h: change(lib, h)] + others:
+            lib.qew_reset(h)
+            lib.fake_throw_after(fail)
+            rc = call(h)
+            lib.fake_throw_after(-1)
+            assert rc in (OK, ENOMEM)
+            assert set(calls(lib, h, 2 * L)) <= ({OK} if rc == OK else {OK, ESTATE})
+            assert lib.fake_bad() == 0, lib.fake_first_bad()
+            lib.qew_reset(h)
+            assert change(lib, h) == OK
+            assert lib.qew_set_precision(h, precision) in (OK, ESTATE)
+    lib.qew_destroy(h)
 
 
 @pytest.mark.parametrize("kind", [0, 1, 2, 3, 4])
