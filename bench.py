@@ -39,11 +39,17 @@ UNIT = "site-updates/s"
 # Algorithmic lane operations per site-update of the fused kernel, per disorder kind (0 RF,
 # 1 uniform RB cubic, 2 none, 3 Gaussian RB linear, 4 Gaussian RB cubic): elastic force 6,
 # pinning 2 (linear) / 8 (cubic) / 0 (none), Euler 3, renormalisation and cell test 3; plus, per
-# cell crossing, one Philox4x32-10 block (~90 integer operations with its key schedule) and the
+# disorder draw, one Philox4x32-10 block (~90 integer operations with its key schedule) and the
 # value transform (Box-Muller ~13, uniform ~2).
 OPS_BASE = {0: 14, 1: 20, 2: 12, 3: 14, 4: 20}
-OPS_PER_CROSSING = {0: 103, 1: 92, 2: 0, 3: 103, 4: 103}
-QUAD_KINDS = (1, 4)
+OPS_PER_DRAW = {0: 103, 1: 92, 2: 0, 3: 103, 4: 103}
+# Draws per cell crossing.  One, but for the Gaussian RB linear kind, whose cache of two cells draws nothing
+# when a site moves back where it came from: counted in the kernel at the preset's drive, 0.33 over the first
+# 256 steps, 0.27 over 1024, 0.22 over 4096.  (The counter itself slows the kernel by up to 10%, so that the
+# figure over 1024 steps stands here.)
+DRAWS_PER_CROSSING = {0: 1.0, 1: 1.0, 2: 0.0, 3: 0.27, 4: 1.0}
+# bytes of a site's state in memory: cell, offset and disorder cache
+STATE_BYTES = {0: 16, 1: 32, 2: 8, 3: 20, 4: 32}
 LANES_PER_SM = 128
 
 
@@ -70,6 +76,11 @@ def parse():
     p.add_argument("--no-cpu-baseline", action="store_true")
     p.add_argument("--no-e2e", action="store_true")
     return p.parse_args()
+
+
+def ops_per_site_update(kind_share: dict, crossings: float) -> float:
+    """Lane operations per site-update at `crossings` per site-update, weighted by each kind's share of sites."""
+    return sum(w * (OPS_BASE[k] + OPS_PER_DRAW[k] * DRAWS_PER_CROSSING[k] * crossings) for k, w in kind_share.items())
 
 
 def rank_seed(rank: int) -> int:
@@ -329,7 +340,7 @@ def other_kernel(q, name: str, stream, sms: int, clk_mhz: float, n_steps: int = 
     sites = np.broadcast_to(np.asarray(wl["L"], dtype=np.float64), (wl["n_chains"],))
     wk = {int(k): float(sites[kinds == k].sum() / sites.sum()) for k in set(kinds.tolist())}
     rx = st["crossings"] / max(1, st["site_updates"])
-    ops = sum(w * (OPS_BASE[k] + OPS_PER_CROSSING[k] * rx) for k, w in wk.items())
+    ops = ops_per_site_update(wk, rx)
     peak = sms * LANES_PER_SM * clk_mhz * 1e6 / 1e12
     ach = ops * st["site_updates"] / (st["fused_ms"] / 1e3) / 1e12 if st["fused_ms"] > 0 else None
     return {"value": n_sites * n_steps / (ms / 1e3), "unit": UNIT, "relax_steps": n_steps,
@@ -416,11 +427,12 @@ def main() -> None:
     kinds = np.broadcast_to(np.asarray(wl["kind"]), (wl["n_chains"],))
     sites = np.broadcast_to(np.asarray(wl["L"], dtype=np.float64), (wl["n_chains"],))
     wk = {int(k): float(sites[kinds == k].sum() / sites.sum()) for k in set(kinds.tolist())}
-    ops_per_su = sum(w * (OPS_BASE[k] + OPS_PER_CROSSING[k] * r_cross) for k, w in wk.items())
+    ops_per_su = ops_per_site_update(wk, r_cross)
+    r_draw = r_cross * sum(w * DRAWS_PER_CROSSING[k] for k, w in wk.items())
     achieved = ops_per_su * su_per_launch / (per_launch_ms / 1e3) / 1e12
     peak = sms * LANES_PER_SM * clk * 1e6 / 1e12
     tile_w, K, tpc = tuning
-    bytes_per_su = sum(w * 2 * (8 + 4 * (6 if k in QUAD_KINDS else 2 if k != 2 else 0)) for k, w in wk.items()) / K
+    bytes_per_su = sum(w * 2 * STATE_BYTES[k] for k, w in wk.items()) / K
     hbm_achieved = bytes_per_su * su_per_launch / (per_launch_ms / 1e3) / 1e9
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     traffic = profiled_traffic()
@@ -442,7 +454,7 @@ def main() -> None:
         "fp32_fma_tops": alu["fp32_fma_per_s"] / 1e12, "sm_mhz": alu["sm_mhz"],
         "frac_of_measured_fp32_fma": achieved / (alu["fp32_fma_per_s"] / 1e12),
         "philox_blocks_per_s": alu["philox_blocks_per_s"],
-        "regeneration_bound_su_per_s": alu["philox_blocks_per_s"] / r_cross if r_cross > 0 else None,
+        "regeneration_bound_su_per_s": alu["philox_blocks_per_s"] / r_draw if r_draw > 0 else None,
         "fp64_fma_tops": alu["fp64_fma_per_s"] / 1e12,
         "basis": "qew_measure_alu_peaks: best of 3 event-timed launches of independent FMA chains / Philox4x32-10 "
                  "blocks on a grid filling every SM"}
@@ -479,7 +491,7 @@ def main() -> None:
 
         def leg_fields(ms_leg, hst, steps):
             rx = hst["crossings"] / max(1, hst["site_updates"])
-            ops = sum(w * (OPS_BASE[k] + OPS_PER_CROSSING[k] * rx) for k, w in wk.items())
+            ops = ops_per_site_update(wk, rx)
             ach = ops * hst["site_updates"] / (hst["fused_ms"] / 1e3) / 1e12 if hst["fused_ms"] > 0 else None
             return {"steps": int(steps), "ms": ms_leg, "value": n_sites * steps / (ms_leg / 1e3),
                     "crossings_per_site_update": rx, "ops_per_site_update": ops,
@@ -572,7 +584,7 @@ def main() -> None:
         cpu = oracle_sample(wl, *cpu_sample_shape(wl["cpu"]["L"]))
         cpu.pop("seconds", None)
 
-    state_gib = sum(w * (8 + 4 * (4 if k in QUAD_KINDS else 2 if k != 2 else 0)) for k, w in wk.items()) * n_sites / 2 ** 30
+    state_gib = sum(w * STATE_BYTES[k] for k, w in wk.items()) * n_sites / 2 ** 30
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
