@@ -35,6 +35,11 @@ static_assert(QEW_RF_GAUSS_LINEAR == kRF && QEW_RB_UNIFORM_CATMULLROM == kRB && 
               "the C ABI's disorder kinds index the kernels' kind table");
 constexpr int32_t kBlockTile = 1024;   // sites per block tile (FP64 path, init, conversions)
 constexpr int64_t kMaxSites = int64_t(1) << 40;
+// Batches of both signs of the drive take a launch for each sign from so many sites on; below, two launches
+// one after the other cost more than the rare moves do.  Half the chains at f_c and half at -f_c, ms per 512
+// steps in one launch and in two: random field 2^19 sites 0.95 1.29, 2^21 1.79 1.88, 2^22 3.01 2.90, 2^24 9.8
+// 9.0; uniform cubic 0.97 1.16, 2.50 2.48, 4.5 4.1, 16.1 14.0; Case 3 1.33 1.76, 2.74 2.45, 4.6 4.6, 15.4 13.0.
+constexpr int64_t kSplitSigns = int64_t(3) << 20;
 constexpr size_t kSqKeep = size_t(256) << 20;
 
 struct DeviceGuard {
@@ -77,6 +82,7 @@ struct qew_ctx {
     std::vector<int64_t> L;
     std::vector<double> f;
     std::vector<int32_t> kind;
+    std::vector<char> neg;          // relaxed by the fused kernel of negative drives
     std::vector<uint32_t> sample;   // sample index s of each chain (counter word 2)
     std::vector<int64_t> offset;    // first site of each chain in the caller's arrays (no gaps)
     std::vector<int64_t> soffset;   // and in the FP32-split state (state_align)
@@ -540,12 +546,13 @@ int build_layout(qew_ctx* h)
         d.s = h->sample[c];
         d.kind = h->kind[c];
         d.f32 = static_cast<float>(h->f[c]);
+        d.neg = h->neg[c];
         d.period = h->period;
         d.f64 = h->f[c];
         for (int64_t st = 0; st < d.L; st += kBlockTile)   // 64-bit: L may reach 2^31 - 1
             blocks.push_back(TileDesc{c, static_cast<int32_t>(st)});
         if (h->precision == QEW_FP32_SPLIT) {
-            const int cls = chain_class(d.kind, d.f32);
+            const int cls = chain_class(d.kind, d.neg);
             first[c] = static_cast<int32_t>(n_list[cls]);
             d.ntiles = static_cast<int32_t>((int64_t(d.L) + h->w_own[d.kind] - 1) / h->w_own[d.kind]);
             n_list[cls] += d.ntiles;
@@ -568,7 +575,7 @@ int build_layout(qew_ctx* h)
             base += h->n_tiles[k];
         }
         for (int32_t c = 0; c < h->n_chains; ++c) {
-            h->h_chains[c].tile0 = h->tile_base[chain_class(h->kind[c], h->h_chains[c].f32)] + first[c];
+            h->h_chains[c].tile0 = h->tile_base[chain_class(h->kind[c], h->neg[c])] + first[c];
         }
         slots = static_cast<size_t>(base);
     } else {
@@ -1117,9 +1124,16 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
             h->soffset[c] = (h->n_state + align - 1) / align * align;
             h->n_state = h->soffset[c] + L[c];
             h->kinds_mask |= 1 << kind[c];
-            h->sites_of_class[chain_class(kind[c], static_cast<float>(f[c]))] += L[c];
         }
         h->n_sites = off;
+        bool positive = false;   // some chain of the kinds that tell the signs apart is not driven downwards
+        for (int32_t c = 0; c < n_chains; ++c)
+            positive = positive || (signed_kind(kind[c]) && !(static_cast<float>(f[c]) < 0.0f));
+        h->neg.resize(n_chains);
+        for (int32_t c = 0; c < n_chains; ++c) {
+            h->neg[c] = signed_kind(kind[c]) && static_cast<float>(f[c]) < 0.0f && (!positive || h->n_sites >= kSplitSigns);
+            h->sites_of_class[chain_class(kind[c], h->neg[c])] += L[c];
+        }
         h->dt = dt;
         h->seed = seed;
         h->precision = precision;

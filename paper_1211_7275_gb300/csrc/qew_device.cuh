@@ -29,10 +29,11 @@ __host__ __device__ constexpr bool quad_kind(int k) { return k == kRB || k == kR
 constexpr int kPairMask = (1 << kRF) | (1 << kRBGLinear);
 constexpr int kQuadMask = (1 << kRB) | (1 << kRBGCubic);
 
-// Chains that the fused kernel takes in one launch: of one kind and, where there is disorder, one sign of
-// the drive.
+// Chains that the fused kernel takes in one launch: of one kind and, where a launch for each sign pays
+// (ChainDesc::neg), one sign of the drive.  (The Gaussian cubic kind treats both directions alike.)
+__host__ __device__ constexpr bool signed_kind(int k) { return pair_kind(k) || k == kRB; }
 constexpr int kNumClasses = 2 * kNumKinds;
-__host__ __device__ constexpr int chain_class(int kind, float f) { return kind + (f < 0.0f && kind != kNone ? kNumKinds : 0); }
+__host__ __device__ constexpr int chain_class(int kind, bool neg) { return kind + (neg ? kNumKinds : 0); }
 constexpr int class_kind(int c) { return c % kNumKinds; }
 
 constexpr uint32_t kTagRF = 0u;   // counter word 3 of random-field force values
@@ -49,6 +50,7 @@ struct ChainDesc {
     int32_t tile0;    // first partial-sum slot of this chain (tiles of its list)
     int32_t ntiles;   // number of tiles (partial-sum slots) of this chain
     float f32;        // drive f, FP32
+    int32_t neg;      // FP32-split: relaxed by the fused kernel of negative drives
     int32_t period;   // disorder period M in u (node index taken mod M); 0: aperiodic
     double f64;       // drive f, FP64
 };

@@ -487,7 +487,7 @@ __device__ __forceinline__ unsigned uniform(unsigned v)
 
 // OBS: whether the launch observes at all.  The observation code in the step loop takes registers
 // from it, so that launches without any (nearly all of a long relaxation's) have a kernel of their own.
-// NEG: chains of a negative drive, whose ordinary moves go downwards.  As one kernel for both signs, by a
+// NEG: chains of a negative drive, whose ordinary moves go downwards (signed_kind).  As one kernel for both signs, by a
 // branch or by selecting at the moves, the random field lost 3% to 12%; without the distinction 16 x 2^20
 // sites at -f_c, -3 f_c took, ms per 512 steps (random field, uniform cubic, Case 3; at f_c, 3 f_c):
 // 10.8 27.2 (8.2 18.5), 16.0 39.9 (10.7 21.0), 18.0 74.6 (12.2 39.3); with it 8.4 18.9,
@@ -1103,7 +1103,7 @@ cudaError_t launch_split_as(int tiles_per_cta, const SplitLaunch& a, cudaStream_
 template <int KIND, int S>
 cudaError_t launch_split(int tiles_per_cta, const SplitLaunch& a, cudaStream_t st)
 {
-    if constexpr (KIND != kNone)
+    if constexpr (signed_kind(KIND))
         if (a.neg)
             return a.n_obs > 0 ? launch_split_as<KIND, S, true, true>(tiles_per_cta, a, st) :
                                  launch_split_as<KIND, S, false, true>(tiles_per_cta, a, st);
@@ -1115,7 +1115,7 @@ __global__ void split_tiles_kernel(const ChainDesc* chains, int cls, int32_t w_o
 {
     const int32_t c = blockIdx.x;
     const ChainDesc ch = chains[c];
-    if (chain_class(ch.kind, ch.f32) != cls)
+    if (chain_class(ch.kind, ch.neg) != cls)
         return;
     WarpTile* mine = tiles + first[c];
     for (int64_t k = threadIdx.x; k * w_own < ch.L; k += blockDim.x) {
@@ -1160,7 +1160,7 @@ __global__ void split_init_kernel(const ChainDesc* chains, const TileDesc* tiles
         {
             // the site's cell and the next one in the direction of the drive; the sign of the offset says
             // that the site is in the upper one
-            const bool neg = ch.f32 < 0.0f;
+            const bool neg = ch.neg;
             const float g1 = rbg_f32(keys, ch.s, i, m1), g2 = rbg_f32(keys, ch.s, i, m2);
             const float g3 = rbg_f32(keys, ch.s, i, neg ? m0 : m3);
             st.rf[p] = neg ? make_float2(g3 - g1, g1 - g2) : make_float2(g1 - g2, g2 - g3);

@@ -59,3 +59,23 @@ def test_forces_of_fresh_caches(qew, kind, sign):
         u, _ = r.state()
     np.testing.assert_allclose(u, ref["u"], atol=2e-6)
     np.testing.assert_allclose(obs["v"][0], ref["v"][0], atol=2e-5)
+
+
+@pytest.mark.parametrize("kind", [RF, RB, RBG_LINEAR, RBG_CUBIC])
+@pytest.mark.parametrize("sites", [(3 << 20) - 64, 3 << 20])
+def test_signs_in_one_launch_and_in_two(qew, kind, sites):
+    """A chain of either sign beside others, below and above the size from which each sign has a launch of
+    its own, against the same chain alone."""
+    n = np.array([5000, 7001])
+    f = F_C[kind] * np.array([1.5, -1.5])
+    lines = []
+    with qew.Relaxation(np.append(n, sites - n.sum()), np.append(f, -f[0]), kind, dt=0.1, seed=SEED) as r:
+        r.advance(60)
+        lines.append(r.state()[0][:n.sum()])
+    alone = []
+    for c in range(2):
+        with qew.Relaxation([n[c]], f[c], kind, dt=0.1, seed=SEED) as r:
+            r.set_samples([c])
+            r.advance(60)
+            alone.append(r.state()[0])
+    assert np.array_equal(lines[0], np.concatenate(alone))
