@@ -306,7 +306,7 @@ def run_reference(args, rank: int, world: int) -> None:
 
 # Launch shapes the autotuner picks for the other presets on a GB300 (their own relaxations, at
 # step 1024); the short measurement below uses them directly instead of tuning again.
-OTHER_SHAPES = {"rb_1024x2^16": (480, 16, 1), "uneven_256": (736, 32, 1), "rbg_linear_4x2^25": (480, 8, 1),
+OTHER_SHAPES = {"rb_1024x2^16": (480, 16, 1), "uneven_256": (736, 32, 1), "rbg_linear_4x2^25": (736, 32, 1),
                 "none_16x2^20": (736, 32, 2), "rf_16x2^20": (992, 32, 2), "rf_4x2^25": (992, 32, 2)}
 
 

@@ -1121,7 +1121,7 @@ int create_impl(qew_handle* out, int32_t n_chains, const int64_t* L, const doubl
             h->offset[c] = off;
             off += L[c];
             const int64_t align = state_align(L[c]);
-            h->soffset[c] = (h->n_state + align - 1) / align * align;
+            h->soffset[c] = (h->n_state + align - 1) & ~(align - 1);
             h->n_state = h->soffset[c] + L[c];
             h->kinds_mask |= 1 << kind[c];
         }

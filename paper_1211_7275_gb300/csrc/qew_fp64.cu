@@ -1,6 +1,6 @@
-// qew_fp64.cu -- the plain FP64 path of the qEW relaxation: FP64 state in HBM (ping-pong), one thread
-// per site and Euler step, and each site's disorder values cached for the cell they were drawn for
-// (regenerated when the site changes cell).
+// qew_fp64.cu -- the plain FP64 path of the qEW relaxation: FP64 state in HBM (ping-pong), a tile of sites
+// per block advanced by several Euler steps in shared memory, and each site's disorder values cached for
+// the cell they were drawn for (regenerated when the site changes cell).
 //
 // Method: Eq. 1 of arXiv:1211.7275 with eta = c = 1, periodic in x, explicit Euler with all
 // forces from the old state (Sec. III.B); pinning force by linear interpolation of R (RF), as
@@ -484,35 +484,40 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                 const int half = NT / 2;
                 const bool split = KIND != kRB && listed <= half;
                 const int part = split && x >= half ? 1 : 0;
-                // Of a site that lost all of its force's nodes (a move of several cells) only those are drawn,
-                // and it is listed again for the others: a steep line, whose sites move so in every step,
-                // would never use them (2^20 sites, 16 steps: random field 8.6 ms, Case 3 10.5, with all drawn).
-                auto lost = [&](int at) { return no_node(s_p[used * NT + at]) && no_node(s_p[(used + NN - 1) * NT + at]); };
-                for (int q = x - part * half; q < listed; q += NT) {
-                    const int at = s_q[q];
-                    const int32_t i = site_of(at), base = s_cell[at] + lo_look;
-                    const bool all = !lost(at);
+                if (split) {
+                    const int q = x - part * half;
+                    if (q < listed) {
+                        const int at = s_q[q];
+                        const int32_t i = site_of(at), base = s_cell[at] + lo_look;
 #pragma unroll 1
-                    for (int c = all ? 0 : used; c < (all ? NX : used + NN); ++c) {
-                        if (!no_node(s_p[c * NT + at]))
-                            continue;
-                        if (!split) {
-                            s_p[c * NT + at] = node_f64<KIND>(a.seed, ch.s, i, base + c, ch.period);
-                        } else {
+                        for (int c = 0; c < NX; ++c) {
+                            if (!no_node(s_p[c * NT + at]))
+                                continue;
                             const uint4 w = disorder_words(a.seed, ch.s, i, wrap_node(base + c, ch.period), KIND == kRF ? kTagRF : kTagRBG);
                             s_f[part * NX * half + c * half + q] = part ? gauss_angle_f64(w) : gauss_radius_f64(w);
                         }
                     }
-                }
-                if (split) {
                     __syncthreads();
                     if (x < listed) {
                         const int at = s_q[x];
-                        const bool all = !lost(at);
 #pragma unroll
                         for (int c = 0; c < NX; ++c)
-                            if ((all || (c >= used && c < used + NN)) && no_node(s_p[c * NT + at]))
+                            if (no_node(s_p[c * NT + at]))
                                 s_p[c * NT + at] = __dmul_rn(s_f[c * half + x], s_f[(NX + c) * half + x]);
+                    }
+                } else {
+                    // In a crowded round a site that lost all of its force's nodes (a move of several cells)
+                    // draws only those, and is listed again for the others: a steep line, whose sites move so
+                    // in every step, would never use them (2^20 sites, 16 steps: random field 8.6 ms, Case 3
+                    // 10.5, with all drawn, 7.3 and 7.7 so).
+                    for (int q = x; q < listed; q += NT) {
+                        const int at = s_q[q];
+                        const int32_t i = site_of(at), base = s_cell[at] + lo_look;
+                        const bool lost = no_node(s_p[used * NT + at]) && no_node(s_p[(used + NN - 1) * NT + at]);
+#pragma unroll 1
+                        for (int c = lost ? used : 0; c < (lost ? used + NN : NX); ++c)
+                            if (no_node(s_p[c * NT + at]))
+                                s_p[c * NT + at] = node_f64<KIND>(a.seed, ch.s, i, base + c, ch.period);
                     }
                 }
                 turn ^= 1;
@@ -526,7 +531,7 @@ __device__ __forceinline__ void f64_look_body(const F64Step& a, const TileDesc t
                     for (int c = 0; c < NN; ++c)
                         nodes[c] = s_p[(used + c) * NT + x];
                     loop_values<KIND>(nodes, v);
-                    if (no_node(s_p[(NEG ? 0 : NX - 1) * NT + x])) {
+                    if (!split && no_node(s_p[(NEG ? 0 : NX - 1) * NT + x])) {
                         slot = atomicAdd(&s_count[turn], 1);
                         s_q[slot] = static_cast<uint16_t>(x);
                     }
