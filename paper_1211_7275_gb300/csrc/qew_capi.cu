@@ -128,6 +128,7 @@ struct qew_ctx {
     int32_t n_ftiles = 0;
     double* u64[2] = {nullptr, nullptr};
     bool layout_made = false;        // tile lists, descriptors and partials as the fields above say
+    bool state_made = false;         // the state's caches are of the handle's disorder
 
     double* d_shift = nullptr;
     double* d_partial = nullptr;
@@ -292,6 +293,17 @@ int check_arrays(qew_ctx* h)
 {
     if (!h->layout_made || !have_buffers(h))
         return fail(h, QEW_ESTATE, "an earlier call on this handle ran out of memory: repeat it, or destroy the handle");
+    return QEW_OK;
+}
+
+// The same for calls that go on from the state: a change of precision or disorder that failed half-way has
+// left it behind.
+int check_state(qew_ctx* h)
+{
+    if (int rc = check_arrays(h))
+        return rc;
+    if (!h->state_made)
+        return fail(h, QEW_ESTATE, "an earlier call on this handle failed: repeat it, or reset the handle");
     return QEW_OK;
 }
 
@@ -679,6 +691,7 @@ int init_state(qew_ctx* h, const double* d_u_in, const std::vector<double>& shif
     QEW_CUDA(h, cudaMemcpyAsync(h->d_shift, shift0.data(), shift0.size() * sizeof(double), cudaMemcpyHostToDevice,
                                 h->stream), "setting reference shifts");
     QEW_CUDA(h, cudaStreamSynchronize(h->stream), "initialising the state");
+    h->state_made = true;
     return QEW_OK;
 }
 
@@ -969,6 +982,8 @@ int autotune(qew_ctx* h)
             return build_layout(h);
         }
     }
+    const int S0 = h->S, K0 = h->K, tpc0 = h->tpc;
+    const bool given0 = h->shape_given;
     h->shape_given = true;
     const int S_all[] = {7, 15, 23, 31, 39};
     const int K_all[] = {4, 8, 16, 32};
@@ -1043,8 +1058,15 @@ int autotune(qew_ctx* h)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc != QEW_OK)
-        return rc;
+    if (rc != QEW_OK) {   // back to the shape there was
+        const std::string why = h->err;
+        h->S = S0;
+        h->K = K0;
+        h->tpc = tpc0;
+        h->shape_given = given0;
+        build_layout(h);
+        return fail(h, rc, why);
+    }
     h->S = bS;
     h->K = bK;
     h->tpc = bT;
@@ -1220,7 +1242,7 @@ int observe_impl(qew_ctx* h, const int64_t* steps, int32_t n_times, double* v_ou
         return QEW_OK;
     if (!steps)
         return fail(h, QEW_EINVAL, "steps must not be NULL");
-    if (int rc = check_arrays(h))
+    if (int rc = check_state(h))
         return rc;
     if (steps[0] < h->step)
         return fail(h, QEW_EINVAL, "steps[0] = " + std::to_string(steps[0]) + " lies before the current step " +
@@ -1347,7 +1369,7 @@ int get_state_impl(qew_ctx* h, double* u_out, int32_t* cells_out, int64_t* step_
         *step_out = h->step;
     if (!u_out && !cells_out)
         return QEW_OK;
-    if (int rc = check_arrays(h))
+    if (int rc = check_state(h))
         return rc;
     double* d_u = nullptr;
     int32_t* d_c = nullptr;
@@ -1454,6 +1476,7 @@ int qew_set_precision(qew_handle h, int32_t precision)
             h->f64_in_place = h->lean = false;
         }
         h->precision = precision;
+        h->state_made = false;
         int rc = build_layout(h);
         if (rc == QEW_OK)
             rc = alloc_state(h);
@@ -1473,6 +1496,7 @@ int qew_set_disorder_period(qew_handle h, int64_t period)
     return guarded(h, [&]() -> int {
         cudaStreamSynchronize(h->stream);
         h->period = static_cast<int32_t>(period);
+        h->state_made = false;
         int rc = build_layout(h);
         if (rc == QEW_OK)
             rc = init_state(h, nullptr, std::vector<double>(h->n_chains, 0.0));
@@ -1489,6 +1513,7 @@ int qew_set_samples(qew_handle h, const uint32_t* s)
     DeviceGuard g(h->device);
     return guarded(h, [&]() -> int {
         cudaStreamSynchronize(h->stream);
+        h->state_made = false;
         h->sample.assign(s, s + h->n_chains);
         int rc = build_layout(h);
         if (rc == QEW_OK)
@@ -1560,7 +1585,7 @@ int qew_advance(qew_handle h, int64_t n_steps)
         return rc;
     if (n_steps < 0)
         return fail(h, QEW_EINVAL, "n_steps must be >= 0");
-    if (int rc = check_arrays(h))
+    if (int rc = check_state(h))
         return rc;
     DeviceGuard g(h->device);
     return guarded(h, [&]() -> int {
@@ -1634,7 +1659,7 @@ int qew_structure_factor(qew_handle h, int32_t n_modes, double* S_out)
             return fail(h, QEW_EINVAL, "the structure factor needs chains of one length");
     if (n_modes < 1 || n_modes > L / 2)
         return fail(h, QEW_EINVAL, "n_modes must lie in [1, L/2]");
-    if (int rc = check_arrays(h))
+    if (int rc = check_state(h))
         return rc;
     DeviceGuard g(h->device);
     const int32_t Li = static_cast<int32_t>(L);
@@ -1847,6 +1872,7 @@ int qew_selftest_lean(qew_handle h)
     return guarded(h, [&]() -> int {
         cudaStreamSynchronize(h->stream);
         free_state(h);
+        h->state_made = false;
         h->f64_in_place = h->lean = true;
         int rc = build_layout(h);
         if (rc == QEW_OK)

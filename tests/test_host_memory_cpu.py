@@ -112,6 +112,43 @@ def test_a_handle_whose_reconfiguration_fails(lib, what, kind, L):
             break
 
 
+@pytest.mark.parametrize("what", ["period", "period64", "samples"])
+def test_a_new_layout_is_not_a_new_state(lib, what):
+    """After a failed change of the disorder the caches are of the old one: another call that makes a layout
+    does not let the chains go on with them, a reset does."""
+    precision, change = RECONFIGURE[what]
+    for fail in range(12):
+        lib.fake_reset()
+        rc, h = create(lib, [5000, 5000], 0, precision)
+        assert rc == OK and lib.qew_advance(h, 10) == OK
+        lib.fake_fail_after(fail)
+        rc = change(lib, h)
+        lib.fake_fail_after(-1)
+        assert rc in (OK, ENOMEM)
+        assert lib.qew_set_tuning(h, 224, 8, 1) == OK
+        assert lib.qew_advance(h, 10) == (OK if rc == OK else ESTATE)
+        assert lib.qew_reset(h) == OK
+        assert calls(lib, h, 10000) == [OK] * 7
+        assert lib.fake_bad() == 0, lib.fake_first_bad()
+        lib.qew_destroy(h)
+
+
+def test_autotuning_that_runs_out_of_memory(lib):
+    for fail in range(0, 400, 7):
+        lib.fake_reset()
+        rc, h = create(lib, [5003 + fail] * 2, 0, FP32)   # (the shape found is remembered by size)
+        assert rc == OK and lib.qew_advance(h, 1100) == OK
+        assert lib.qew_set_tuning(h, 0, 0, 0) == OK
+        lib.fake_fail_after(fail)
+        v = np.empty(2)
+        rc = lib.qew_observe(h, _p(np.array([1200], dtype=np.int64)), 1, _p(v), None)
+        lib.fake_fail_after(-1)
+        assert rc in (OK, ENOMEM)
+        assert calls(lib, h, 2 * (5003 + fail)) == [OK] * 7   # in the shape it had
+        assert lib.fake_bad() == 0, lib.fake_first_bad()
+        lib.qew_destroy(h)
+
+
 @pytest.mark.parametrize("what", sorted(RECONFIGURE))
 def test_host_allocations_that_fail(lib, what):
     """No exception leaves a C entry: QEW_ENOMEM, and the handle is as after a failed device allocation."""
