@@ -971,6 +971,19 @@ int run_through(qew_ctx* h, const int64_t* targets, int32_t n_targets, double* d
 int autotune(qew_ctx* h)
 {
     h->autotune_pending = false;
+    const int S0 = h->S, K0 = h->K, tpc0 = h->tpc;
+    const bool given0 = h->shape_given;
+    auto or_as_before = [&](int rc) -> int {   // after a failure the shape there was
+        if (rc == QEW_OK)
+            return rc;
+        const std::string why = h->err;
+        h->S = S0;
+        h->K = K0;
+        h->tpc = tpc0;
+        h->shape_given = given0;
+        build_layout(h);
+        return fail(h, rc, why);
+    };
     TuneKey key{h->n_sites, h->n_chains, h->kinds_mask,
                 *std::min_element(h->L.begin(), h->L.end()), *std::max_element(h->L.begin(), h->L.end())};
     {
@@ -979,11 +992,9 @@ int autotune(qew_ctx* h)
         if (it != g_tune_cache.end()) {
             std::tie(h->S, h->K, h->tpc) = it->second;
             h->shape_given = true;
-            return build_layout(h);
+            return or_as_before(build_layout(h));
         }
     }
-    const int S0 = h->S, K0 = h->K, tpc0 = h->tpc;
-    const bool given0 = h->shape_given;
     h->shape_given = true;
     const int S_all[] = {7, 15, 23, 31, 39};
     const int K_all[] = {4, 8, 16, 32};
@@ -997,7 +1008,7 @@ int autotune(qew_ctx* h)
     if (ce != cudaSuccess) {
         if (e0)
             cudaEventDestroy(e0);
-        return cuda_fail(h, ce, "creating tuning events");
+        return or_as_before(cuda_fail(h, ce, "creating tuning events"));
     }
     int rc = QEW_OK;
     for (int S : S_all) {
@@ -1058,15 +1069,8 @@ int autotune(qew_ctx* h)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc != QEW_OK) {   // back to the shape there was
-        const std::string why = h->err;
-        h->S = S0;
-        h->K = K0;
-        h->tpc = tpc0;
-        h->shape_given = given0;
-        build_layout(h);
-        return fail(h, rc, why);
-    }
+    if (rc != QEW_OK)
+        return or_as_before(rc);
     h->S = bS;
     h->K = bK;
     h->tpc = bT;
@@ -1074,7 +1078,7 @@ int autotune(qew_ctx* h)
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_tune_cache[key] = std::make_tuple(bS, bK, bT);
     }
-    return build_layout(h);
+    return or_as_before(build_layout(h));
 }
 
 // Sites on whose multiples a chain starts in the FP32-split state: bulk copies need four (16 bytes) for
